@@ -17,6 +17,7 @@
 
 #include "../../include/gke.h"
 #include "gke_common.cuh"
+#include "gke_digits.h"
 #include "gke_kernels.h"
 #include "gke_split.h"
 
@@ -105,6 +106,7 @@ struct gke_plan_s {
     size_t part_count = 0;
     int *fdl0 = nullptr, *pair_i = nullptr, *nonfinite = nullptr;
     SplitWork split;
+    DigitWork digits;                         // FP64 contractions on the tensor cores (empty: FMA kernel)
     long long pair_chunk = 0;
     // diagnostics
     bool timing = false;
@@ -708,6 +710,11 @@ extern "C" gke_status gke_plan(const gke_desc* desc, void* stream, gke_plan_t* o
         gke_status s = split_alloc(p->split, ny, ns, p->Kc);
         if (s != GKE_OK) return bail(s, "split workspace allocation failed");
     }
+    if (d.precision == GKE_PREC_F64 && digits_pays(ny, ns, p->Kc)) {
+        if ((e = digits_setup()) != cudaSuccess)
+            return bail(GKE_ERR_CUDA, std::string("digit setup: ") + cudaGetErrorString(e));
+        digits_alloc(p->digits, ny, p->Kc);
+    }
 #undef ALLOC
     // host tables
     // twiddles e^{-2 pi i m / n}, m < n, from the host's libm in FP64
@@ -853,6 +860,7 @@ extern "C" void gke_destroy(gke_plan_t p)
                     p->fdl0, p->pair_i, p->nonfinite, p->part, p->sep_tab};
     for (void* q : ptrs) if (q) cudaFree(q);
     split_free(p->split);
+    digits_free(p->digits);
     for (auto& m : p->marks) { cudaEventDestroy(m.a); cudaEventDestroy(m.b); }
     for (auto e : p->chunk_ev) cudaEventDestroy(e);
     if (p->copy_st) cudaStreamDestroy(p->copy_st);
@@ -1041,6 +1049,13 @@ static gke_status enqueue_snapshot(gke_plan_t p, const zd* f, int ns)
     // (NkX wavenumbers) into raw
     auto correlate = [&](const void* X, int NkX, int k0, int Kc) -> gke_status {
         StageScope sc(p, GKE_STAGE_CORRELATE);
+        if (digits_ready(p->digits) && digits_pays(ny, ns, Kc)) {
+            int nl = 0;
+            gke_status s = digits_correlate(p->digits, (const zd*)X, ns, ny, NkX, k0, Kc, (zd*)p->raw,
+                                            job_set(p->tset), st, p->err, &nl);
+            p->launches += nl;
+            return s;
+        }
         if (d.precision != GKE_PREC_BF16X3) {
             correlate_launch(f32, X, ns, ny, NkX, k0, Kc, p->raw, job_set(p->tset), st);
             p->launches += 1;
@@ -1350,8 +1365,9 @@ extern "C" gke_status gke_finalize_terms(gke_plan_t p, void* terms, double* prof
     for (cudaEvent_t e : p->chunk_ev) p->spare.push_back(e);
     p->chunk_ev.clear();
     p->finalized = true;
-    if (p->d.precision == GKE_PREC_BF16X3) {
-        gke_status ss = split_check(p->split, p->st, p->err);
+    {
+        gke_status ss = p->d.precision == GKE_PREC_BF16X3 ? split_check(p->split, p->st, p->err)
+                                                          : digits_check(p->digits, p->st, p->err);
         if (ss != GKE_OK) return ss;
     }
     if (bad) return fail(p, GKE_ERR_NONFINITE, "non-finite value in the accumulated input");
@@ -1491,8 +1507,9 @@ extern "C" gke_status gke_compute_graph(gke_plan_t p, const void* fields, int ns
     CUDA_TRY(p, cudaMemcpyAsync(&bad, p->nonfinite, sizeof(int), cudaMemcpyDeviceToHost, p->st));
     CUDA_TRY(p, cudaStreamSynchronize(p->st));
     p->finalized = true;
-    if (p->d.precision == GKE_PREC_BF16X3) {
-        gke_status ss = split_check(p->split, p->st, p->err);
+    {
+        gke_status ss = p->d.precision == GKE_PREC_BF16X3 ? split_check(p->split, p->st, p->err)
+                                                          : digits_check(p->digits, p->st, p->err);
         if (ss != GKE_OK) return ss;
     }
     if (bad) return fail(p, GKE_ERR_NONFINITE, "non-finite value in the accumulated input");

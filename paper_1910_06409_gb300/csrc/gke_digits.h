@@ -1,0 +1,31 @@
+// gke_digits.h -- FP64 contractions over snapshots from exact digit products on
+// the tensor cores (internal; gke_digits.cu describes the method).
+#pragma once
+#include <cuda_runtime.h>
+#include <string>
+#include "../../include/gke.h"
+#include "gke_common.cuh"
+
+namespace gke {
+
+struct DigitWork {
+    void* ws = nullptr;         // digit operands and row exponents of one chunk of wavenumbers
+    size_t bytes = 0;
+    int* err = nullptr;         // device flag: a pipeline wait timed out
+};
+
+// workspace for up to Kc wavenumbers of n wall-normal points (n rows); on
+// failure the work stays empty and digits_ready is false
+void digits_alloc(DigitWork& w, int n, int Kc);
+inline bool digits_ready(const DigitWork& w) { return w.ws != nullptr; }
+cudaError_t digits_setup();
+// whether the digit products are the faster way for a batch (measured; gke_digits.cu)
+bool digits_pays(int n, int ns, long long Kc);
+// the contractions `jobs` of the wavenumbers [k0, k0 + Kc) into raw (as
+// correlate_launch's FP64 form); *launches gets the kernels launched
+gke_status digits_correlate(DigitWork& w, const zd* Xop, int ns, int ny, int Nk, int k0, int Kc, zd* raw,
+                            unsigned jobs, cudaStream_t st, std::string& err, int* launches);
+gke_status digits_check(DigitWork& w, cudaStream_t st, std::string& err);
+void digits_free(DigitWork& w);
+
+}  // namespace gke
