@@ -9,20 +9,20 @@
 // Splitting.  All values of a row (wavenumber k, wall-normal point y) of one
 // group of fields -- velocities; products; pressure -- share the exponent E
 // of the largest of them over the batch's snapshots, |x| < 2^E.  Each value
-// becomes the integer round(x 2^(62 - E)) and that its eight balanced base-256
-// digits s_0 (|s_0| <= 65) .. s_7 (in [-128, 127]), exact in FP16.  62 bits
+// becomes the integer round(x 2^(61 - E)) and that its eight balanced base-256
+// digits s_0 (|s_0| <= 33) .. s_7 (in [-128, 127]), exact in FP16.  61 bits
 // below the row's largest value hold every bit of an FP64 value down to
-// 2^-9 of that maximum; smaller values lose bits below 2^-62 of it, nine
+// 2^-8 of that maximum; smaller values lose bits below 2^-61 of it, eight
 // binary orders under the FP64 rounding of the sums they enter.
 //
 // Products.  With the digit products s_i t_j summed over the terms and
 // snapshots of a contraction by order d = i + j (v_d, d <= 7; the orders
 // above are below 2^-64 of the largest product),
-//   sum a b = 2^(E_a + E_b - 36) [ (v_0 .. v_3) + 2^-32 (v_4 .. v_7) ],
+//   sum a b = 2^(E_a + E_b - 34) [ (v_0 .. v_3) + 2^-32 (v_4 .. v_7) ],
 //   (w_0 .. w_3) = 2^24 w_0 + 2^16 w_1 + 2^8 w_2 + w_3.
 // A sum v_d runs over at most 4 terms x 16 snapshots x 2 real products, so
-// |v_d| <= max(1, d) 4 2^19 <= 2^24: the FP32 accumulation in tensor memory is
-// exact.  The eight sums are joined in a 64-bit integer and rounded to FP64
+// |v_d| <= max(1, d) 4 2^19 < 2^24 (and < 2^22 for d <= 2, where s_0 enters every
+// or all but one product): the FP32 accumulation in tensor memory is exact.  The eight sums are joined in a 64-bit integer and rounded to FP64
 // once, all in integer arithmetic.  A sum over up to 16 snapshots therefore
 // carries one rounding where the FMA chain carries 32 per term; further
 // snapshots come in groups of 16, added in FP64.
@@ -44,10 +44,11 @@
 // Every wait is bounded (gke_split.cu has the same protocol).
 //
 // Measured, correlate stage (operands, contractions; FMA kernel -> here):
-// 256 x 256 x 65, 16 snapshots 232.8 -> 43.2 ms, of which the operand kernel 6.5,
-// the MMAs alone 23 (smem reads of A and B: 18.5 by count) and the epilogue
-// alone 33, which bounds it; 128 x 128 x 65, 32 snapshots 117.4 -> 23.0 ms.
-// Errors against 64-bit references equal the FMA kernel's or are below.
+// 256 x 256 x 65, 16 snapshots 232.8 -> 33.9 ms, of which the operand kernel 6.5
+// and the MMAs alone 23 (smem reads of A and B: 18.5 by count), which bound it
+// with the epilogue (conversions and integer adds) close behind; 128 x 128 x 65,
+// 32 snapshots 117.4 -> 18.2 ms.  Errors against 64-bit references equal the
+// FMA kernel's or are below.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -95,7 +96,7 @@ struct DgArgs {
     int nstep, njob;
     DgStep step[DG_MAXSTEP];
     DgJob job[DG_MAXJOB];
-    int mul[4];                            // 2^3, 2^11, 2^19, 2^27 (mad_wide)
+    int mul[4];                            // 2^5, 2^13, 2^21, 2^29 (mad_wide)
     int Kc, beta;
     zd* raw;
     int* err;
@@ -143,7 +144,7 @@ struct DgPrep {
     __half* Aop; __half* Bop; int* E;
 };
 
-// round(x 2^sh) for |x| 2^sh < 2^62, in integer arithmetic (a conversion would
+// round(x 2^sh) for |x| 2^sh < 2^61, in integer arithmetic (a conversion would
 // run on the FP64 pipe)
 __device__ __forceinline__ unsigned long long dg_fixed(double x, int sh)
 {
@@ -215,8 +216,8 @@ k_dg_prep(const __grid_constant__ DgPrep a)
         for (int e = 0; e < 8; ++e) {
             zd v = mk(0.0, 0.0);
             if (e < ne) v = src[(long long)e * a.s.n];
-            dre[e] = dg_bytes(dg_fixed(v.x, 62 - E + fd.wexp));
-            dim[e] = dg_bytes(dg_fixed(v.y, 62 - E + fd.wexp));
+            dre[e] = dg_bytes(dg_fixed(v.x, 61 - E + fd.wexp));
+            dim[e] = dg_bytes(dg_fixed(v.y, 61 - E + fd.wexp));
         }
         __half* da = fd.ia < 0 || !astore ? nullptr
                    : a.Aop + (((long long)k * a.nfa + fd.ia) * a.s.MT + mb) * (long long)(DG_S * 2 * a.s.RT * DG_KS)
@@ -282,40 +283,52 @@ __device__ __forceinline__ long long mad_wide(int a, int b, long long c)
     asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
     return r;
 }
-// A sum joined as the integer T = round(2^19 (w_0 .. w_3) + 2^-13 (w_4 .. w_7)),
-// (w_0 .. w_3) = 2^24 w_0 + 2^16 w_1 + 2^8 w_2 + w_3: |T| < 2^63 with one unit 2^-55
-// of the largest product.  First the orders 4..7 of column j (|w| <= 2^24),
-// then 0..3 (w_0 <= 2^19.1, w_1 <= 2^21, so both stay in the upper word).
-__device__ __forceinline__ long long dg_low(const uint32_t (&r)[4][4], int j, int m11, int m3)
+// A sum joined as the integer T = 2^21 (w_0 .. w_3) + 2^-11 (w_4 .. w_7) (w_6 and
+// w_7 rounded; one unit is 2^-55 of the largest product),
+// (w_0 .. w_3) = 2^24 w_0 + 2^16 w_1 + 2^8 w_2 + w_3, |T| < 2^62.  The epilogue is bound
+// by the conversions (16 a clock and SM) and the integer adds (64): sums below
+// 2^22 turn integer by an FP32 addition of 1.5 2^23, whose bits are DG_MAGIC + w;
+// DG_BIAS takes the offsets of w_0, w_1, w_2 and of w_6 / 8 + w_7 / 2^11 out again.
+constexpr float DG_MAGF = 12582912.f;                               // 1.5 2^23
+constexpr unsigned long long DG_MAGIC = 0x4B400000ull;              // its bits
+constexpr long long DG_BIAS = (long long)(0ull - DG_MAGIC - (DG_MAGIC << 29) - (DG_MAGIC << 37) - (DG_MAGIC << 45));
+// orders 4..7 of column j (|w| <= 2^24)
+__device__ __forceinline__ long long dg_low(const uint32_t (&r)[4][4], int j, int m13, int m5)
 {
-    auto w = [&](int d) { return __float2int_rz(__uint_as_float(r[d][j])); };
-    const int i67 = w(2) * 32 + (w(3) >> 3);
-    const long long v = mad_wide(w(1), m3, (long long)((i67 + 512) >> 10));
-    return mad_wide(w(0), m11, v);
+    const float g = fmaf(__uint_as_float(r[3][j]), 1.f / 2048.f, fmaf(__uint_as_float(r[2][j]), 1.f / 8.f, DG_MAGF));
+    const long long v = mad_wide(__float2int_rz(__uint_as_float(r[1][j])), m5,
+                                 mad_wide(__float2int_rz(__uint_as_float(r[0][j])), m13, DG_BIAS));
+    return v + (long long)(unsigned long long)__float_as_uint(g);
 }
-__device__ __forceinline__ long long dg_high(const uint32_t (&r)[4][4], int j, long long low, int m19, int m27)
+// with the orders 0..3 (|w_0|, |w_1|, |w_2| < 2^22)
+__device__ __forceinline__ long long dg_high(const uint32_t (&r)[4][4], int j, long long low, int m21, int m29)
 {
-    auto w = [&](int d) { return __float2int_rz(__uint_as_float(r[d][j])); };
-    const long long v = mad_wide(w(2), m27, mad_wide(w(3), m19, low));
-    const int up = (int)(v >> 32) + (w(0) << 11) + (w(1) << 3);
-    return (long long)(((unsigned long long)(unsigned)up << 32) | (unsigned)v);
+    auto bits = [&](int d) { return __float_as_uint(__uint_as_float(r[d][j]) + DG_MAGF); };
+    const long long v = mad_wide((int)bits(2), m29, mad_wide(__float2int_rz(__uint_as_float(r[3][j])), m21, low));
+    const unsigned up = (unsigned)((unsigned long long)v >> 32) + (bits(0) << 13) + (bits(1) << 5);
+    return (long long)(((unsigned long long)up << 32) | (unsigned)v);
 }
-// t 2^(e - 19) where its exponent leaves the normal range
-__device__ __noinline__ double dg_value_edge(long long t, int e) { return scalbn((double)t, e - 19); }
-// t 2^(e - 19), normalised and rounded (half away from zero) in integer
-// arithmetic: a conversion would hold the FP64 pipe of the whole SM for 16
-// clocks a warp, these ~25 instructions one issue slot each
-__device__ __forceinline__ double dg_value(long long t, int e)
+// t 2^(e - 21) in general
+__device__ __noinline__ double dg_value_edge(long long t, int e) { return scalbn((double)t, e - 21); }
+// t 2^(e - 21), normalised and rounded to nearest in integer arithmetic (a
+// conversion would hold the FP64 pipe of the whole SM for 16 clocks a warp).
+// No branch, so that values interleave; edge is raised where the upper
+// word is zero or the exponent may leave the normal range (dg_value_edge then).
+__device__ __forceinline__ double dg_value(long long t, int e, bool& edge)
 {
-    const unsigned long long sg = (unsigned long long)(t >> 63);
-    unsigned long long m = ((unsigned long long)t ^ sg) - sg;
-    const int lz = __clzll((long long)m);
-    if (m == 0) return 0.0;
-    m <<= lz;
-    const int x = 1023 + 44 - lz + e;                                // biased exponent
-    if ((unsigned)(x - 1) >= 2045u) return dg_value_edge(t, e);
-    const unsigned long long b = ((unsigned long long)(unsigned)(x - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
-    return __longlong_as_double((long long)(b | (sg & 0x8000000000000000ull)));
+    unsigned h = (unsigned)((unsigned long long)t >> 32), l = (unsigned)t;
+    const unsigned sg = (unsigned)((int)h >> 31);
+    const unsigned long long m = ((unsigned long long)t ^ (((unsigned long long)sg << 32) | sg)) + (sg & 1u);
+    h = (unsigned)(m >> 32);
+    l = (unsigned)m;
+    const int lz = __clz((int)h);
+    edge |= (h == 0) ? l != 0 : (unsigned)(e + 900) > 1800u;
+    const unsigned mh = __funnelshift_l(l, h, lz), ml = l << (lz & 31);
+    unsigned rl = __funnelshift_r(ml, mh, 11), rh = (mh >> 11) + ((unsigned)(1022 + 42 - lz + e) << 20);
+    const unsigned up = (ml >> 10) & 1u;
+    rl += up;
+    rh += rl < up;
+    return h == 0 ? 0.0 : __hiloint2double((int)(rh | (sg & 0x80000000u)), (int)rl);
 }
 __device__ __forceinline__ void st_256(zd* p, zd a, zd b)
 {
@@ -469,7 +482,7 @@ k_dg_corr(const __grid_constant__ DgArgs a)
         int acc = 0;
         uint32_t aph = 0;
         const int YB = (a.s.n + 7) / 8;
-        const int m3 = a.mul[0], m11 = a.mul[1], m19 = a.mul[2], m27 = a.mul[3];
+        const int m5 = a.mul[0], m13 = a.mul[1], m21 = a.mul[2], m29 = a.mul[3];
         const int r = q * 32 + lane;
         // exponents of an item: this row's, and lane j's column c0 + j, per
         // group; loaded an item ahead
@@ -515,8 +528,8 @@ k_dg_corr(const __grid_constant__ DgArgs a)
                         dg_ready(v);
                         #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            lo[0][4 * g + j] = dg_low(v[0], j, m11, m3);
-                            lo[1][4 * g + j] = dg_low(v[1], j, m11, m3);
+                            lo[0][4 * g + j] = dg_low(v[0], j, m13, m5);
+                            lo[1][4 * g + j] = dg_low(v[1], j, m13, m5);
                         }
                     }
                 }
@@ -535,11 +548,22 @@ k_dg_corr(const __grid_constant__ DgArgs a)
                         dg_ready(v);
                         const int yp = c0 + 4 * g;
                         zd o[4];
+                        bool edge = false;
                         #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             const int e = ej + __shfl_sync(0xffffffffu, ebj, 4 * g + j);
-                            o[j] = mk(dg_value(dg_high(v[0], j, lo[0][4 * g + j], m19, m27), e),
-                                      dg_value(dg_high(v[1], j, lo[1][4 * g + j], m19, m27), e));
+                            long long& t0 = lo[0][4 * g + j];
+                            long long& t1 = lo[1][4 * g + j];
+                            t0 = dg_high(v[0], j, t0, m21, m29);
+                            t1 = dg_high(v[1], j, t1, m21, m29);
+                            o[j] = mk(dg_value(t0, e, edge), dg_value(t1, e, edge));
+                        }
+                        if (__any_sync(0xffffffffu, edge && row)) {
+                            #pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const int e = ej + __shfl_sync(0xffffffffu, ebj, 4 * g + j);
+                                o[j] = mk(dg_value_edge(lo[0][4 * g + j], e), dg_value_edge(lo[1][4 * g + j], e));
+                            }
                         }
                         if (row && yp < 8 * YB) {
                             zd* dst = a.raw + raw_index(job.out, u.k, y, yp, a.Kc, YB);
@@ -704,12 +728,12 @@ void digits_alloc(DigitWork& w, int n, int Kc)
 }
 
 // Against the FMA kernel (correlate stage, us, FMA -> digits): 544 wavenumbers
-// x 4 snapshots: 507 -> 247 at ny = 17, 555 -> 431 at 33, 1991 -> 580 at 65,
-// 7600 -> 1302 at 129; 8320 wavenumbers x 16 snapshots: 7423 -> 1722, 8085 -> 3628,
-// 29421 -> 5504, 112586 -> 10260.  Only where the FMA kernel's CTAs, one
-// 32 x 32 tile of at most one snapshot chunk each, all run at once is it level
-// (40 wavenumbers: 71 us, digits 67 at ny <= 17, 76 at 25): those keep it and
-// need no workspace.
+// x 4 snapshots: 507 -> 240 at ny = 17, 532 -> 407 at 33, 1954 -> 543 at 65,
+// 7535 -> 1130 at 129; 4160 wavenumbers x 16 snapshots: 7423 -> 1659, 8085 -> 2799,
+// 29421 -> 4326, 112586 -> 9462.  Only where the FMA kernel's CTAs, one
+// 32 x 32 tile of at most one snapshot chunk each, all run at once are the two
+// level (40 wavenumbers: 71 us, digits 66 at ny <= 17, 72 at 25): those keep it
+// and need no workspace.
 bool digits_pays(int n, int ns, long long Kc) { return !(Kc <= 64 && n <= 32 && ns <= 8); }
 
 gke_status digits_correlate(DigitWork& w, const zd* Xop, int ns, int ny, int Nk, int k0, int Kc, zd* raw,
@@ -735,11 +759,14 @@ gke_status digits_correlate(DigitWork& w, const zd* Xop, int ns, int ny, int Nk,
     a.nfa = CH_NFA; a.nfb = CH_NFB; a.ngrp = CH_NGRP;
     a.tpk = s.MT * s.NT;
     a.Kc = Kc;
-    for (int i = 0; i < 4; ++i) a.mul[i] = 1 << (3 + 8 * i);
+    for (int i = 0; i < 4; ++i) a.mul[i] = 1 << (5 + 8 * i);
     a.err = w.err;
     std::vector<std::vector<HostTerm>> terms;
     DgRows rows{};
-    for (int j = 0; j < NJOB; ++j) {
+    // long and short contractions alternate: the epilogue of a one-term job
+    // takes longer than its MMAs, that of a four-term job less
+    static const int order[NJOB] = {J_GX, J_E, J_GZ, J_F, J_X, J_QV, J_D};
+    for (int j : order) {
         if (!((jobs >> j) & 1u)) continue;
         const HostJob& h = kJobs[j];
         std::vector<HostTerm> v;
@@ -754,7 +781,7 @@ gke_status digits_correlate(DigitWork& w, const zd* Xop, int ns, int ny, int Nk,
         d.ga = (signed char)(h.fa[0] <= F_W ? 0 : h.fa[0] == F_P ? 1 : 2);
         d.gb = 0;
         d.out = (signed char)j;
-        d.e = -36;
+        d.e = -34;
     }
     if (!a.njob) return GKE_OK;
     dg_schedule(a, terms);
