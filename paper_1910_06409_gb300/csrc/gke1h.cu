@@ -13,12 +13,15 @@
 //              operand blocks X[f][m_x][s][p] and the one-point sums.
 //              k1_onepoint: eps (Parseval in x, stencils in y and z) and the
 //              one-point parts of the terms.
-//   correlate  k1_correlate, one CTA per (tile pair, m_x): the snapshot sums
-//              of the correlation products of Eq. 7 (Parseval, Eq. 8-9), 20
-//              contractions, each added into the per-pair term spectra with
-//              its coefficients; then the one-point parts and the mean-flow
-//              couplings.  Only term spectra reach HBM.  A remainder of at
-//              most 8 points past the last full tile runs as strips
+//   correlate  the snapshot sums of the correlation products of Eq. 7
+//              (Parseval, Eq. 8-9), combined into the per-pair term spectra,
+//              with the one-point parts and the mean-flow couplings; only
+//              term spectra reach HBM.  FP64 plans: 13 contractions on the
+//              tensor cores (digit_correlate).  FP32 plans, and FP64 plans
+//              whose digit workspace could not be allocated: k1_correlate,
+//              one CTA per (tile pair, m_x), 20 contractions, each added into
+//              the term spectra with its coefficients; a remainder of at most
+//              8 points past the last full tile runs as strips
 //              (k1_correlate_strip) instead of as padded tiles.
 //   terms      k1_transform_r (nx = 128, 256, 512; register FFT) or
 //              k1_transform: the inverse x transform of every (term, pair).
@@ -42,6 +45,8 @@
 
 #include "../../include/gke1h.h"
 #include "gke_common.cuh"
+#include "gke_digits.cuh"
+#include "gke_digits.h"
 
 using gke::zd;
 using gke::zf;
@@ -559,6 +564,165 @@ k1_correlate_strip(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int co
     finish_pair<TF>(T, q1, q2, m, nx, kx0, nu, ns, P, prof, op, spec, npair);
 }
 
+// ---------------------------------------------- correlate, digit products
+// FP64 plans: the contractions on the tensor cores (gke_digits.cuh).  Every
+// spectrum is one or two contractions of at most five terms whose A and B
+// fields share exponent groups (g0: u, v, w; g1: the products, pairs u_i u_k
+// doubled; g2: w_a = 2 sum_b d_b U_a u_b, b = y, z; g3: the products again with 4 p):
+//   A     = -2 sum conj(u_i) u_i
+//   Phi_k = [conj(q) u_k + conj(2 u_i u_k) u_i] - [conj(u_k) q + conj(u_i) 2 u_i u_k]
+//   psi_k = [conj(q) u_k - conj(2 u_i u_k) u_i - conj(4 p) u_k] / 2
+//         + [conj(u_k) q - conj(u_i) 2 u_i u_k - conj(u_k) 4 p] / 2
+//   xi    = conj(u_a) w_a + conj(w_a) u_a
+// (add_job's sums; the mean gradients of xi ride on w_a).  Five terms let the
+// sum of order 7 reach 2^24.2: its rounding is below 2^-64 of the largest product.
+// A first part (and every part of the snapshot groups before the last) waits
+// in its spectrum; the last brings the snapshot average,
+// the one-point parts at m = 0 and the mean-flow couplings of finish_pair.
+// Correlate stage (us, k1_correlate -> here), 16 snapshots: 256 x 33 x 33
+// 333880 -> 44130; nx = 256, P = 576 96067 -> 12598, 48 1968 -> 398; nx = 64, 25 points
+// 665 -> 194; nx = 8, 25 points, 1 snapshot 356 -> 188: no size keeps the FMA
+// kernel.  Errors against 64-bit references are a few percent below its own.
+// The MMAs (53 terms x 36 digit pairs a tile) would take 14 ms of the first;
+// the integer and FP64 work on the values bounds it.
+enum DigitKind { DK_PART = 1, DK_SECOND = 2 };
+struct DuctOut {
+    zd* spec;
+    long long npair;
+    int P, nx, m0;
+    bool first, last;                     // first and last group of 16 snapshots
+    double kx0, nu, inv;
+    const double *prof, *op;
+    __device__ __forceinline__ void operator()(const gke::DgJob& job, int k, int q1, int q2, zd (&o)[4]) const
+    {
+        const int nxh = nx / 2 + 1, m = m0 + k, t = job.out;
+        if (q1 >= P || q2 + 3 < q1 || q2 >= P) return;
+        const long long pr = tri(q1, q2, P);                  // of column 0 (a stored one from q2 >= q1 on)
+        zd* dst = spec + ((long long)t * nxh + m) * npair + pr;
+        const double* u = prof + (long long)(t == A_PHIX ? R_U : t == A_PHIY || t == A_PSIY ? R_V : R_W) * P;
+        auto O = [&](int r, int q) { return op[(long long)r * P + q]; };
+        const double kk = (2 * m == nx) ? 0.0 : kx0 * m;
+        #pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int p2 = q2 + j;
+            if (p2 < q1 || p2 >= P) continue;
+            zd v = o[j];
+            if (!first || job.kind == DK_SECOND) v = v + dst[j];
+            if (!last || job.kind == DK_PART) { dst[j] = v; continue; }
+            v = inv * v;
+            if (m == 0) {
+                // one-point parts
+                const int r = t == A_PHIX ? O_SX : t == A_PHIY || t == A_PSIY ? O_SY : O_SZ;
+                if (t == A_A) v.x += O(O_K, q1) + O(O_K, p2);
+                else if (t == A_XI) v.x += O(O_E0, q1) + O(O_E0, p2);
+                else if (t == A_PSIY || t == A_PSIZ)
+                    v.x += 0.5 * (O(r, q1) + O(r, p2)) +
+                           2.0 * (O(t == A_PSIY ? O_PY : O_PZ, q1) + O(t == A_PSIY ? O_PY : O_PZ, p2));
+                else v.x += O(r, p2) - O(r, q1);
+            }
+            if (t != A_A && t != A_XI) {
+                const zd A = (spec + ((long long)A_A * nxh + m) * npair + pr)[j];
+                const double c = (t == A_PSIY || t == A_PSIZ) ? 0.5 * (u[q1] + u[p2]) : u[p2] - u[q1];
+                v.x = fma(c, A.x, v.x);
+                v.y = fma(c, A.y, v.y);
+                if (t == A_PHIX) {
+                    v.x = fma(2.0 * nu * kk, A.y, v.x);
+                    v.y = fma(-2.0 * nu * kk, A.x, v.y);
+                }
+            }
+            dst[j] = v;
+            if (t == A_XI) {
+                const zd x = (spec + ((long long)A_PHIX * nxh + m) * npair + pr)[j];
+                (spec + ((long long)NACC * nxh + m) * npair + pr)[j] = mk(-kk * x.y - v.x, kk * x.x - v.y);
+            }
+        }
+    }
+};
+
+// fields of the digit operands
+enum { D_U = 0, D_V, D_W, D_Q, D_UU, D_UV, D_UW, D_VV, D_VW, D_WW, D_W0, D_W1, D_W2, D_QP, D_UVP, D_UWP, D_VVP, D_VWP,
+       D_WWP, D_P4, ND };
+constexpr int ND_GRP = 4;
+static gke::DgShape digit_shape(int P) { return gke::dg_shape(P, false); }
+static size_t digit_bytes(int P) { return gke::dg_bytes_per_k(digit_shape(P), ND, ND, ND_GRP); }
+
+// the contractions of all wavenumbers into the spectra; kernels launched
+static int digit_correlate(gke::DigitWork& w, const zd* X, int ns, int P, int nx, double kx0, double nu,
+                           const double* prof, const double* op, zd* spec, long long npair, cudaStream_t st)
+{
+    const int nxh = nx / 2 + 1;
+    gke::DgPrep p{};
+    gke::DgArgs a{};
+    gke::dg_init(p, a, digit_shape(P), ND, ND, ND_GRP, true, w.err);
+    auto field = [&](int d, int src, int wexp, int grp) {
+        gke::DgField& f = p.f[p.nf++];
+        f.src = (short)src; f.src2 = -1; f.wexp = (signed char)wexp; f.grp = (signed char)grp;
+        f.ia = f.ib = (short)d;
+    };
+    for (int i = 0; i < 3; ++i) field(D_U + i, G_U + i, 0, 0);
+    field(D_Q, G_Q, 0, 1);
+    for (int i = 0; i < 6; ++i) field(D_UU + i, G_UU + i, 1, 1);
+    for (int i = 0; i < 3; ++i) {
+        field(D_W0 + i, G_V, 1, 2);
+        gke::DgField& f = p.f[p.nf - 1];
+        f.src2 = G_W;
+        f.c = prof + (long long)(R_G + 2 * i) * P;
+        f.c2 = prof + (long long)(R_G + 2 * i + 1) * P;
+    }
+    field(D_QP, G_Q, 0, 3);
+    const int pr[5] = {G_UV, G_UW, G_VV, G_VW, G_WW};
+    for (int i = 0; i < 5; ++i) field(D_UVP + i, pr[i], 1, 3);
+    field(D_P4, G_P, 2, 3);
+    p.X = X; p.nsX = ns; p.Nk = nxh;
+
+    std::vector<std::vector<gke::HostTerm>> terms;
+    auto job = [&](int out, int kind, int ga, int gb, int e, std::vector<gke::HostTerm> v) {
+        gke::DgJob& j = a.job[a.njob++];
+        j.ga = (signed char)ga; j.gb = (signed char)gb; j.out = (signed char)out; j.kind = (signed char)kind;
+        j.e = -34 + e;
+        terms.push_back(std::move(v));
+    };
+    const int pair[3][3] = {{D_UU, D_UV, D_UW}, {D_UV, D_VV, D_VW}, {D_UW, D_VW, D_WW}};
+    const int pairp[3][3] = {{-1, D_UVP, D_UWP}, {D_UVP, D_VVP, D_VWP}, {D_UWP, D_VWP, D_WWP}};
+    job(A_A, 0, 0, 0, 1, {{D_U, D_U, true}, {D_V, D_V, true}, {D_W, D_W, true}});
+    for (int k = 0; k < 3; ++k) {
+        std::vector<gke::HostTerm> f{{D_Q, k, false}}, b{{k, D_Q, true}};
+        for (int i = 0; i < 3; ++i) {
+            f.push_back({pair[i][k], i, false});
+            b.push_back({i, pair[i][k], true});
+        }
+        job(A_PHIX + k, DK_PART, 1, 0, 0, f);
+        job(A_PHIX + k, DK_SECOND, 0, 1, 0, b);
+    }
+    for (int k = 1; k < 3; ++k) {
+        std::vector<gke::HostTerm> f{{D_QP, k, false}, {D_P4, k, true}}, b{{k, D_QP, false}, {k, D_P4, true}};
+        for (int i = 0; i < 3; ++i) {
+            f.push_back({pairp[i][k], i, true});
+            b.push_back({i, pairp[i][k], true});
+        }
+        job(A_PSIY + k - 1, DK_PART, 3, 0, -1, f);
+        job(A_PSIY + k - 1, DK_SECOND, 0, 3, -1, b);
+    }
+    job(A_XI, DK_PART, 0, 2, 0, {{D_U, D_W0, false}, {D_V, D_W1, false}, {D_W, D_W2, false}});
+    job(A_XI, DK_SECOND, 2, 0, 0, {{D_W0, D_U, false}, {D_W1, D_V, false}, {D_W2, D_W, false}});
+    gke::dg_schedule(a, terms);
+    const int kmax = (int)std::min<size_t>((size_t)nxh, w.bytes / digit_bytes(P));
+    int launches = 0;
+    for (int m0 = 0; m0 < nxh; m0 += kmax) {
+        const int nk = std::min(kmax, nxh - m0);
+        gke::dg_place(p, a, w.ws, nk);
+        p.k0 = m0;
+        for (int s0 = 0; s0 < ns; s0 += gke::DG_KS) {
+            p.s0 = s0;
+            p.ns = std::min(gke::DG_KS, ns - s0);
+            gke::dg_pass(p, a, nk, DuctOut{spec, npair, P, nx, m0, s0 == 0, s0 + gke::DG_KS >= ns, kx0, nu, 1.0 / ns,
+                                           prof, op}, st);
+            launches += 2;
+        }
+    }
+    return launches;
+}
+
 // ------------------------------------------------------------- transforms
 // CTA = 2 NB consecutive pairs of one term.  The spectra (nx/2 + 1
 // wavenumbers each, imaginary parts dropped at m = 0 and m = nx/2) are
@@ -860,6 +1024,7 @@ struct gke1h_plan_s {
     float* pf = nullptr;                 // float copy of the mean and gradient rows (FP32 plans)
     void *X = nullptr, *spec = nullptr, *terms = nullptr;
     int smem_prod = 0, smem_tr = 0, NB = 0;
+    gke::DigitWork digits;               // FP64 contractions on the tensor cores (empty: FMA kernel)
     bool reg_tr = false;                 // register-FFT transform (nx = 128, 256, 512)
     bool timing = false;
     struct Mark { int stage; cudaEvent_t a, b; };
@@ -898,6 +1063,7 @@ static void free_plan(gke1h_plan_t p)
     void* bufs[] = {p->wy, p->wz, p->prof, p->m1, p->op, p->terms, p->ly, p->lz, p->pq, p->bad,
                     p->tw, p->twf, p->pf, p->X, p->spec, p->fin};
     for (void* b : bufs) if (b) cudaFree(b);
+    gke::digits_free(p->digits);
     for (auto& mk_ : p->marks) { cudaEventDestroy(mk_.a); cudaEventDestroy(mk_.b); }
     delete p;
 }
@@ -1025,6 +1191,14 @@ extern "C" gke_status gke1h_plan(const gke1h_desc* d, void* stream, gke1h_plan_t
         free_plan(p);
         return fail1(nullptr, GKE_ERR_CUDA, "shared-memory attributes refused");
     }
+    if (!p->f32) {
+        if (gke::dg_attrs<DuctOut>() != cudaSuccess) {
+            cudaGetLastError();
+            free_plan(p);
+            return fail1(nullptr, GKE_ERR_CUDA, "shared-memory attributes refused");
+        }
+        gke::digits_alloc(p->digits, digit_bytes(p->P), p->nxh);
+    }
     *out = p;
     return GKE_OK;
 }
@@ -1074,14 +1248,20 @@ static void launch_pass(gke1h_plan_t p, const zd* f, int ns, TF* T)
     }
     {
         Scope1 sc(p, GKE_STAGE_CORRELATE);
+        const bool digits = sizeof(TF) == 8 && gke::digits_ready(p->digits);
+        if (digits)
+            p->launches += digit_correlate(p->digits, (const zd*)X, ns, P, nx, kx0, p->nu, p->prof, p->op, (zd*)spec,
+                                           p->npair, p->st);
         const int nfull = P / CT, rem = P - nfull * CT;
         const bool strips = nfull > 0 && rem > 0 && rem <= STRIP_MAX;
         const int nt = strips ? nfull : p->nt;
         const long long ntp = (long long)nt * (nt + 1) / 2;
-        k1_correlate<TF><<<dim3((unsigned)ntp, nxh), 256, 0, p->st>>>(X, ns, P, nx, nt, kx0, p->nu, pt, p->op,
-                                                                      spec, p->npair);
-        p->launches += 1;
-        if (strips) {
+        if (!digits) {
+            k1_correlate<TF><<<dim3((unsigned)ntp, nxh), 256, 0, p->st>>>(X, ns, P, nx, nt, kx0, p->nu, pt, p->op,
+                                                                          spec, p->npair);
+            p->launches += 1;
+        }
+        if (strips && !digits) {
             const int cov = nfull * CT;
             const long long n = ((long long)rem * cov + (long long)rem * (rem + 1) / 2) * nxh;
             k1_correlate_strip<TF><<<(unsigned)((n + 127) / 128), 128, 0, p->st>>>(X, ns, P, nx, cov, kx0, p->nu,
@@ -1152,6 +1332,10 @@ extern "C" gke_status gke1h_compute(gke1h_plan_t p, const void* fields, int nsna
     int bad = 0;
     TRY1(p, cudaMemcpyAsync(&bad, p->bad, sizeof(int), cudaMemcpyDeviceToHost, p->st));
     TRY1(p, cudaStreamSynchronize(p->st));
+    {
+        const gke_status ds = gke::digits_check(p->digits, p->st, p->err);
+        if (ds != GKE_OK) return ds;
+    }
     if (bad) return fail1(p, GKE_ERR_NONFINITE, "the input holds a NaN or Inf");
     return GKE_OK;
 }

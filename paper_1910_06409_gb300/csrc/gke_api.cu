@@ -711,9 +711,8 @@ extern "C" gke_status gke_plan(const gke_desc* desc, void* stream, gke_plan_t* o
         if (s != GKE_OK) return bail(s, "split workspace allocation failed");
     }
     if (d.precision == GKE_PREC_F64 && digits_pays(ny, ns, p->Kc)) {
-        if ((e = digits_setup()) != cudaSuccess)
+        if ((e = digits_setup(p->digits, ny, p->Kc)) != cudaSuccess)
             return bail(GKE_ERR_CUDA, std::string("digit setup: ") + cudaGetErrorString(e));
-        digits_alloc(p->digits, ny, p->Kc);
     }
 #undef ALLOC
     // host tables

@@ -14,11 +14,12 @@ struct DigitWork {
     int* err = nullptr;         // device flag: a pipeline wait timed out
 };
 
-// workspace for up to Kc wavenumbers of n wall-normal points (n rows); on
-// failure the work stays empty and digits_ready is false
-void digits_alloc(DigitWork& w, int n, int Kc);
+// workspace for chunks of up to Kc wavenumbers of `per` bytes each; on failure
+// the work stays empty (digits_ready false) and the callers keep their FMA kernels
+void digits_alloc(DigitWork& w, size_t per, int Kc);
 inline bool digits_ready(const DigitWork& w) { return w.ws != nullptr; }
-cudaError_t digits_setup();
+// the channel's kernels and workspace (n wall-normal points)
+cudaError_t digits_setup(DigitWork& w, int n, int Kc);
 // whether the digit products are the faster way for a batch (measured; gke_digits.cu)
 bool digits_pays(int n, int ns, long long Kc);
 // the contractions `jobs` of the wavenumbers [k0, k0 + Kc) into raw (as
