@@ -579,65 +579,95 @@ k1_correlate_strip(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int co
 // A first part (and every part of the snapshot groups before the last) waits
 // in its spectrum; the last brings the snapshot average,
 // the one-point parts at m = 0 and the mean-flow couplings of finish_pair.
-// Correlate stage (us, k1_correlate -> here), 16 snapshots: 256 x 33 x 33
-// 333880 -> 44130; nx = 256, P = 576 96067 -> 12598, 48 1968 -> 398; nx = 64, 25 points
-// 665 -> 194; nx = 8, 25 points, 1 snapshot 356 -> 188: no size keeps the FMA
-// kernel.  Errors against 64-bit references are a few percent below its own.
-// The MMAs (53 terms x 36 digit pairs a tile) would take 14 ms of the first;
-// the integer and FP64 work on the values bounds it.
+// The kernel leaves the sums in the spectra: a first part stored, a second
+// (and the parts of further groups of 16 snapshots) added by L2 reductions,
+// whose one addition per value neither waits for the stored one nor occupies
+// the SM's FP64 pipe.  k1_finish then brings the mean-flow couplings.  With
+// the couplings in the epilogue the stage took 44.1 ms at 256 x 33 x 33.
+//   Correlate stage (us, k1_correlate -> here), 16 snapshots: 256 x 33 x 33
+// 333880 -> 28984 (k1_finish 4750 of it); no size tried keeps the FMA kernel (nx = 8, 25 points, 1 snapshot
+// 356 -> 188).  Errors against 64-bit references are a few percent below its
+// own.  Bound by the MMAs (53 terms x 36 digit pairs a tile: 14 ms).
 enum DigitKind { DK_PART = 1, DK_SECOND = 2 };
 struct DuctOut {
     zd* spec;
     long long npair;
-    int P, nx, m0;
-    bool first, last;                     // first and last group of 16 snapshots
-    double kx0, nu, inv;
-    const double *prof, *op;
+    int P, nxh, m0, first;                // first group of 16 snapshots
     __device__ __forceinline__ void operator()(const gke::DgJob& job, int k, int q1, int q2, zd (&o)[4]) const
     {
-        const int nxh = nx / 2 + 1, m = m0 + k, t = job.out;
         if (q1 >= P || q2 + 3 < q1 || q2 >= P) return;
-        const long long pr = tri(q1, q2, P);                  // of column 0 (a stored one from q2 >= q1 on)
-        zd* dst = spec + ((long long)t * nxh + m) * npair + pr;
-        const double* u = prof + (long long)(t == A_PHIX ? R_U : t == A_PHIY || t == A_PSIY ? R_V : R_W) * P;
-        auto O = [&](int r, int q) { return op[(long long)r * P + q]; };
-        const double kk = (2 * m == nx) ? 0.0 : kx0 * m;
+        // row pointer at column q2 (pairs from q2 >= q1 on are stored)
+        zd* dst = spec + ((long long)job.out * nxh + m0 + k) * npair + tri(q1, q2, P);
+        const bool add = !first || job.kind == DK_SECOND;
         #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int p2 = q2 + j;
-            if (p2 < q1 || p2 >= P) continue;
-            zd v = o[j];
-            if (!first || job.kind == DK_SECOND) v = v + dst[j];
-            if (!last || job.kind == DK_PART) { dst[j] = v; continue; }
-            v = inv * v;
-            if (m == 0) {
-                // one-point parts
-                const int r = t == A_PHIX ? O_SX : t == A_PHIY || t == A_PSIY ? O_SY : O_SZ;
-                if (t == A_A) v.x += O(O_K, q1) + O(O_K, p2);
-                else if (t == A_XI) v.x += O(O_E0, q1) + O(O_E0, p2);
-                else if (t == A_PSIY || t == A_PSIZ)
-                    v.x += 0.5 * (O(r, q1) + O(r, p2)) +
-                           2.0 * (O(t == A_PSIY ? O_PY : O_PZ, q1) + O(t == A_PSIY ? O_PY : O_PZ, p2));
-                else v.x += O(r, p2) - O(r, q1);
-            }
-            if (t != A_A && t != A_XI) {
-                const zd A = (spec + ((long long)A_A * nxh + m) * npair + pr)[j];
-                const double c = (t == A_PSIY || t == A_PSIZ) ? 0.5 * (u[q1] + u[p2]) : u[p2] - u[q1];
-                v.x = fma(c, A.x, v.x);
-                v.y = fma(c, A.y, v.y);
-                if (t == A_PHIX) {
-                    v.x = fma(2.0 * nu * kk, A.y, v.x);
-                    v.y = fma(-2.0 * nu * kk, A.x, v.y);
-                }
-            }
-            dst[j] = v;
-            if (t == A_XI) {
-                const zd x = (spec + ((long long)A_PHIX * nxh + m) * npair + pr)[j];
-                (spec + ((long long)NACC * nxh + m) * npair + pr)[j] = mk(-kk * x.y - v.x, kk * x.x - v.y);
+            if (q2 + j < q1 || q2 + j >= P) continue;
+            if (!add) dst[j] = o[j];
+            else {
+                asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(&dst[j].x), "d"(o[j].x) : "memory");
+                asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(&dst[j].y), "d"(o[j].y) : "memory");
             }
         }
     }
 };
+
+// The spectra of one pair from its summed contractions (finish_pair's
+// formulas): snapshot average (scale 1 where the digits' power of two holds it),
+// one-point parts at m = 0, mean-flow couplings, the residual's spectral part.
+// Thread = one pair, MB wavenumbers: the couplings' mean-flow factors are
+// formed once.  Bound by memory: seven spectra read, eight written.
+constexpr int FIN_MB = 8;
+__global__ void __launch_bounds__(256)
+k1_finish(zd* __restrict__ spec, const int* __restrict__ pq, long long npair, int P, int nx, double kx0, double nu,
+          double scale, const double* __restrict__ prof, const double* __restrict__ op)
+{
+    const long long pr = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (pr >= npair) return;
+    const int nxh = nx / 2 + 1, mb = blockIdx.y * FIN_MB;
+    const int q1 = pq[2 * pr], q2 = pq[2 * pr + 1];
+    auto U = [&](int r, int q) { return prof[(long long)r * P + q]; };
+    auto O = [&](int r, int q) { return op[(long long)r * P + q]; };
+    double c[5];                                     // factors of A in Phi_x .. psi_z
+    #pragma unroll
+    for (int i = 0; i < 3; ++i) c[i] = U(R_U + i, q2) - U(R_U + i, q1);
+    c[3] = 0.5 * (U(R_V, q1) + U(R_V, q2));
+    c[4] = 0.5 * (U(R_W, q1) + U(R_W, q2));
+    for (int m = mb; m < min(mb + FIN_MB, nxh); ++m) {
+        zd* s = spec + (long long)m * npair + pr;
+        const long long ts = (long long)nxh * npair;
+        const double kk = (2 * m == nx) ? 0.0 : kx0 * m;
+        zd v[NACC];
+        #pragma unroll
+        for (int t = 0; t < NACC; ++t) v[t] = gke::ld_stream(s + t * ts);
+        if (scale != 1.0) {
+            #pragma unroll
+            for (int t = 0; t < NACC; ++t) v[t] = scale * v[t];
+        }
+        if (m == 0) {
+            v[A_A].x += O(O_K, q1) + O(O_K, q2);
+            v[A_PHIX].x += O(O_SX, q2) - O(O_SX, q1);
+            v[A_PHIY].x += O(O_SY, q2) - O(O_SY, q1);
+            v[A_PHIZ].x += O(O_SZ, q2) - O(O_SZ, q1);
+            v[A_PSIY].x += 0.5 * (O(O_SY, q1) + O(O_SY, q2)) + 2.0 * (O(O_PY, q1) + O(O_PY, q2));
+            v[A_PSIZ].x += 0.5 * (O(O_SZ, q1) + O(O_SZ, q2)) + 2.0 * (O(O_PZ, q1) + O(O_PZ, q2));
+            v[A_XI].x += O(O_E0, q1) + O(O_E0, q2);
+        }
+        const zd A = v[A_A];
+        #pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            v[A_PHIX + i].x = fma(c[i], A.x, v[A_PHIX + i].x);
+            v[A_PHIX + i].y = fma(c[i], A.y, v[A_PHIX + i].y);
+        }
+        const double nk = 2.0 * nu * kk;
+        v[A_PHIX].x = fma(nk, A.y, v[A_PHIX].x);
+        v[A_PHIX].y = fma(-nk, A.x, v[A_PHIX].y);
+        if (m == 0 || scale != 1.0) gke::st_stream(s, A);
+        #pragma unroll
+        for (int t = A_PHIX; t <= A_PSIZ; ++t) gke::st_stream(s + t * ts, v[t]);
+        if (m == 0 || scale != 1.0) gke::st_stream(s + A_XI * ts, v[A_XI]);
+        gke::st_stream(s + NACC * ts, mk(-kk * v[A_PHIX].y - v[A_XI].x, kk * v[A_PHIX].x - v[A_XI].y));
+    }
+}
 
 // fields of the digit operands
 enum { D_U = 0, D_V, D_W, D_Q, D_UU, D_UV, D_UW, D_VV, D_VW, D_WW, D_W0, D_W1, D_W2, D_QP, D_UVP, D_UWP, D_VVP, D_VWP,
@@ -648,7 +678,8 @@ static size_t digit_bytes(int P) { return gke::dg_bytes_per_k(digit_shape(P), ND
 
 // the contractions of all wavenumbers into the spectra; kernels launched
 static int digit_correlate(gke::DigitWork& w, const zd* X, int ns, int P, int nx, double kx0, double nu,
-                           const double* prof, const double* op, zd* spec, long long npair, cudaStream_t st)
+                           const double* prof, const double* op, const int* pq, zd* spec, long long npair,
+                           cudaStream_t st)
 {
     const int nxh = nx / 2 + 1;
     gke::DgPrep p{};
@@ -675,11 +706,14 @@ static int digit_correlate(gke::DigitWork& w, const zd* X, int ns, int P, int nx
     field(D_P4, G_P, 2, 3);
     p.X = X; p.nsX = ns; p.Nk = nxh;
 
+    // the snapshot average: a power of two goes into the digits' exponents
+    const bool pow2 = (ns & (ns - 1)) == 0;
+    const int se = pow2 ? -gke::ilog2(ns) : 0;
     std::vector<std::vector<gke::HostTerm>> terms;
     auto job = [&](int out, int kind, int ga, int gb, int e, std::vector<gke::HostTerm> v) {
         gke::DgJob& j = a.job[a.njob++];
         j.ga = (signed char)ga; j.gb = (signed char)gb; j.out = (signed char)out; j.kind = (signed char)kind;
-        j.e = -34 + e;
+        j.e = -34 + e + se;
         terms.push_back(std::move(v));
     };
     const int pair[3][3] = {{D_UU, D_UV, D_UW}, {D_UV, D_VV, D_VW}, {D_UW, D_VW, D_WW}};
@@ -715,12 +749,13 @@ static int digit_correlate(gke::DigitWork& w, const zd* X, int ns, int P, int nx
         for (int s0 = 0; s0 < ns; s0 += gke::DG_KS) {
             p.s0 = s0;
             p.ns = std::min(gke::DG_KS, ns - s0);
-            gke::dg_pass(p, a, nk, DuctOut{spec, npair, P, nx, m0, s0 == 0, s0 + gke::DG_KS >= ns, kx0, nu, 1.0 / ns,
-                                           prof, op}, st);
+            gke::dg_pass(p, a, nk, DuctOut{spec, npair, P, nxh, m0, s0 == 0}, st);
             launches += 2;
         }
     }
-    return launches;
+    k1_finish<<<dim3((unsigned)((npair + 255) / 256), (unsigned)((nxh + FIN_MB - 1) / FIN_MB)), 256, 0, st>>>(
+        spec, pq, npair, P, nx, kx0, nu, pow2 ? 1.0 : 1.0 / ns, prof, op);
+    return launches + 1;
 }
 
 // ------------------------------------------------------------- transforms
@@ -1250,8 +1285,8 @@ static void launch_pass(gke1h_plan_t p, const zd* f, int ns, TF* T)
         Scope1 sc(p, GKE_STAGE_CORRELATE);
         const bool digits = sizeof(TF) == 8 && gke::digits_ready(p->digits);
         if (digits)
-            p->launches += digit_correlate(p->digits, (const zd*)X, ns, P, nx, kx0, p->nu, p->prof, p->op, (zd*)spec,
-                                           p->npair, p->st);
+            p->launches += digit_correlate(p->digits, (const zd*)X, ns, P, nx, kx0, p->nu, p->prof, p->op, p->pq,
+                                           (zd*)spec, p->npair, p->st);
         const int nfull = P / CT, rem = P - nfull * CT;
         const bool strips = nfull > 0 && rem > 0 && rem <= STRIP_MAX;
         const int nt = strips ? nfull : p->nt;
