@@ -47,6 +47,7 @@
 #include "gke_common.cuh"
 #include "gke_digits.cuh"
 #include "gke_digits.h"
+#include "gke_fixed.cuh"
 
 using gke::zd;
 using gke::zf;
@@ -822,7 +823,7 @@ k1_transform_r(const cplx<TF>* __restrict__ spec, long long npair, const cplx<TF
     const int t = blockIdx.y;
     const long long pa = ((long long)blockIdx.x * RZ + r) * 2, pb = pa + 1;
     const bool la = pa < npair, lb = pb < npair;
-    gke::load_twiddles(stw, tw, N);
+    gke::load_twiddles2l<TF>(stw, tw, N);
     // spectra [t][m][pair]: the two pairs of a sequence share 32-byte sectors
     const C* sa = spec + (long long)t * nxh * npair + (la ? pa : 0);
     const C* sb = spec + (long long)t * nxh * npair + (lb ? pb : 0);
@@ -838,7 +839,7 @@ k1_transform_r(const cplx<TF>* __restrict__ spec, long long npair, const cplx<TF
         v[j] = mk(a.x - b.y, a.y + b.x);
     }
     __syncthreads();                                  // twiddles staged
-    gke::fft2l<TF, N1, N2, true>(v, lane, xs + r * N1 * (N2 + 1), N2 + 1, 1, stw);
+    gke::fft2l_rows<TF, N1, N2, true>(v, lane, xs + r * N1 * (N2 + 1), N2 + 1, 1, stw);
     #pragma unroll
     for (int j = 0; j < N1; ++j) {
         const int x = lane + N2 * j;
@@ -1165,7 +1166,8 @@ extern "C" gke_status gke1h_plan(const gke1h_desc* d, void* stream, gke1h_plan_t
     std::vector<int> ly(p->ny), lz(p->nz);
     for (int j = 0; j < p->ny; ++j) ly[j] = gke_fd_weights(d->y, p->ny, j, wy.data() + 5 * j);
     for (int j = 0; j < p->nz; ++j) lz[j] = gke_fd_weights(d->z, p->nz, j, wz.data() + 5 * j);
-    std::vector<zd> tw(p->nx);
+    std::vector<zd> tw(2 * p->nx);                    // FP64, then fixed point (gke_fixed.cuh)
+    gke::fx_table(p->nx, tw.data());
     std::vector<zf> twf(p->nx);
     for (int i = 0; i < p->nx; ++i) {
         const double a = -2.0 * M_PI * i / p->nx;

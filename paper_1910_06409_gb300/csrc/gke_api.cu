@@ -18,6 +18,7 @@
 #include "../../include/gke.h"
 #include "gke_common.cuh"
 #include "gke_digits.h"
+#include "gke_fixed.cuh"
 #include "gke_kernels.h"
 #include "gke_split.h"
 
@@ -679,13 +680,13 @@ extern "C" gke_status gke_plan(const gke_desc* desc, void* stream, gke_plan_t* o
     for (cudaEvent_t& ev : p->aux_ev)
         if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess)
             return bail(GKE_ERR_CUDA, std::string("event: ") + cudaGetErrorString(e));
-    ALLOC(p->tw_xd, d.nx);
-    ALLOC(p->tw_zd, d.nz);
+    ALLOC(p->tw_xd, 2 * d.nx);                // FP64, then fixed point (gke_fixed.cuh)
+    ALLOC(p->tw_zd, 2 * d.nz);
     ALLOC(p->tw_xf, d.nx);
     ALLOC(p->tw_zf, d.nz);
     if (p->dec) {
-        ALLOC(p->ttw_xd, p->nxt);
-        ALLOC(p->ttw_zd, p->nzt);
+        ALLOC(p->ttw_xd, 2 * p->nxt);
+        ALLOC(p->ttw_zd, 2 * p->nzt);
         ALLOC(p->ttw_xf, p->nxt);
         ALLOC(p->ttw_zf, p->nzt);
     } else {
@@ -717,7 +718,9 @@ extern "C" gke_status gke_plan(const gke_desc* desc, void* stream, gke_plan_t* o
 #undef ALLOC
     // host tables
     // twiddles e^{-2 pi i m / n}, m < n, from the host's libm in FP64
-    std::vector<zd> twx(d.nx), twz(d.nz);
+    std::vector<zd> twx(2 * d.nx), twz(2 * d.nz);
+    fx_table(d.nx, twx.data());
+    fx_table(d.nz, twz.data());
     std::vector<zf> twxf(d.nx), twzf(d.nz);
     for (int m = 0; m < d.nx; ++m) { twx[m].x = std::cos(2.0 * M_PI * m / d.nx); twx[m].y = -std::sin(2.0 * M_PI * m / d.nx); }
     for (int m = 0; m < d.nz; ++m) { twz[m].x = std::cos(2.0 * M_PI * m / d.nz); twz[m].y = -std::sin(2.0 * M_PI * m / d.nz); }
@@ -765,7 +768,9 @@ extern "C" gke_status gke_plan(const gke_desc* desc, void* stream, gke_plan_t* o
     if (p->dec) {
         // twiddles of the coarse transforms: every s-th entry of the fine ones
         const int sx = d.nx / p->nxt, sz = d.nz / p->nzt;
-        std::vector<zd> cx(p->nxt), cz(p->nzt);
+        std::vector<zd> cx(2 * p->nxt), cz(2 * p->nzt);
+        fx_table(p->nxt, cx.data());
+        fx_table(p->nzt, cz.data());
         std::vector<zf> cxf(p->nxt), czf(p->nzt);
         for (int m = 0; m < p->nxt; ++m) { cx[m] = twx[m * sx]; cxf[m] = twxf[m * sx]; }
         for (int m = 0; m < p->nzt; ++m) { cz[m] = twz[m * sz]; czf[m] = twzf[m * sz]; }

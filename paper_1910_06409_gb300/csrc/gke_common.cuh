@@ -264,8 +264,15 @@ __device__ __forceinline__ void dft_reg(cplx<T>* v)
 // The inner DFT runs in registers, its twiddled result goes through the
 // exchange buffer xs[k1 s1 + n2 s2] and the outer DFT (rows k1 = n2 + N2 j)
 // runs in registers again.  stw: the N-point twiddle table in shared memory.
-// Contains one __syncthreads(); every thread of the block must call it.
-template <typename T, int N1, int N2, bool INV>
+// Contains one __syncthreads(), or with WARP (the lanes of a sequence in one
+// warp, their part of xs their own) one __syncwarp(); every thread of the
+// block, or of the warp, must call it.
+template <bool WARP> __device__ __forceinline__ void sync_lanes()
+{
+    if (WARP) __syncwarp();
+    else __syncthreads();
+}
+template <typename T, int N1, int N2, bool INV, bool WARP = false>
 __device__ __forceinline__ void fft2l(cplx<T>* v, int lane, cplx<T>* xs, int s1, int s2, const cplx<T>* stw)
 {
     static_assert(N1 % N2 == 0, "N1 must be a multiple of N2");
@@ -279,7 +286,7 @@ __device__ __forceinline__ void fft2l(cplx<T>* v, int lane, cplx<T>* xs, int s1,
     }
     #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1) xs[k1 * s1 + lane * s2] = v[k1];
-    __syncthreads();
+    sync_lanes<WARP>();
     #pragma unroll
     for (int jj = 0; jj < R; ++jj) {
         const int k1 = lane + N2 * jj;

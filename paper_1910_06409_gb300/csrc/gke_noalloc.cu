@@ -26,16 +26,20 @@
 
 #include "../../include/gke.h"
 #include "gke_common.cuh"
+#include "gke_fixed.cuh"
 #include "gke_kernels.h"
 
 using namespace gke;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[GKE_NOALLOC_SCRATCH_BYTES];
+// twiddles along x, then along z: FP64 and fixed-point entries (gke_fixed.cuh), 1024 each at most
+static __device__ zd g_noalloc_tw[4 * 1024];
 
 namespace {
 
 constexpr int MAX_DEVICES = 64;
-unsigned char* g_scratch_dev[MAX_DEVICES] = {nullptr};   // device address of the array, per device
+unsigned char* g_scratch_dev[MAX_DEVICES] = {nullptr};   // device addresses of the arrays, per device
+zd* g_tw_dev[MAX_DEVICES] = {nullptr};
 // status only: this entry point keeps no message (its callers read the code),
 // so the texts below are documentation and nothing is formatted
 gke_status fail(gke_status s, const char*) { return s; }
@@ -46,7 +50,10 @@ gke_status setup_device(int dev, cudaStream_t st)
     if (g_scratch_dev[dev]) return GKE_OK;
     void* ptr = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
+    void* tw = nullptr;
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&tw, g_noalloc_tw);
     if (e != cudaSuccess) return fail(GKE_ERR_CUDA, "cudaGetSymbolAddress failed");
+    g_tw_dev[dev] = (zd*)tw;
     int lim = 0;
     cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if ((e = products_set_attrs(lim)) != cudaSuccess || (e = terms_set_attrs(lim)) != cudaSuccess ||
@@ -140,8 +147,8 @@ extern "C" gke_status gke_compute_noalloc(const gke_desc* desc, const void* fiel
     zd* raw = c.take<zd>((size_t)NJOB * ((ny + 7) / 8) * ((ny + 7) / 8) * 64 * Nk);
     zd* comb = c.take<zd>((size_t)npair * NTERM * Nk);
     zd* W = c.take<zd>((size_t)npair * NTERM * Nk);
-    zd* twx = c.take<zd>(nx);
-    zd* twz = c.take<zd>(nz);
+    zd* twx = g_tw_dev[dev];
+    zd* twz = twx + 2 * nx;
     double* mean_sum = c.take<double>(4 * ny);
     double* mean = c.take<double>(4 * ny);
     double* stats = c.take<double>(NSTAT * ny);
@@ -159,14 +166,16 @@ extern "C" gke_status gke_compute_noalloc(const gke_desc* desc, const void* fiel
     // scope; the pair list is built on the device
     cudaError_t e;
 #define TRY(call) do { if ((e = (call)) != cudaSuccess) return fail(GKE_ERR_CUDA, #call); } while (0)
-    zd h_twx[MAX_N], h_twz[MAX_N];
+    zd h_twx[2 * MAX_N], h_twz[2 * MAX_N];
     double h_fdw[5 * MAX_N];
     int h_fdl0[MAX_N];
     for (int m = 0; m < nx; ++m) { h_twx[m].x = std::cos(2.0 * M_PI * m / nx); h_twx[m].y = -std::sin(2.0 * M_PI * m / nx); }
     for (int m = 0; m < nz; ++m) { h_twz[m].x = std::cos(2.0 * M_PI * m / nz); h_twz[m].y = -std::sin(2.0 * M_PI * m / nz); }
+    fx_table(nx, h_twx);
+    fx_table(nz, h_twz);
     for (int j = 0; j < ny; ++j) h_fdl0[j] = gke_fd_weights(d.y, ny, j, h_fdw + 5 * j);
-    TRY(cudaMemcpyAsync(twx, h_twx, nx * sizeof(zd), cudaMemcpyHostToDevice, st));
-    TRY(cudaMemcpyAsync(twz, h_twz, nz * sizeof(zd), cudaMemcpyHostToDevice, st));
+    TRY(cudaMemcpyAsync(twx, h_twx, 2 * nx * sizeof(zd), cudaMemcpyHostToDevice, st));
+    TRY(cudaMemcpyAsync(twz, h_twz, 2 * nz * sizeof(zd), cudaMemcpyHostToDevice, st));
     TRY(cudaMemcpyAsync(fdw, h_fdw, 5 * ny * sizeof(double), cudaMemcpyHostToDevice, st));
     TRY(cudaMemcpyAsync(fdl0, h_fdl0, ny * sizeof(int), cudaMemcpyHostToDevice, st));
     k_pair_table<<<ny, 128, 0, st>>>(ny, pair_i);

@@ -10,6 +10,7 @@
 #include <algorithm>
 
 #include "gke_common.cuh"
+#include "gke_fixed.cuh"
 #include "gke_kernels.h"
 
 namespace gke {
@@ -123,7 +124,8 @@ k_col_inverse_r(const zd* __restrict__ fields_s, int ny, int nxh, int CW, int YB
     const int kx = blockIdx.x * CW + c, y = blockIdx.y * YB + yl, f = blockIdx.z;
     const bool live = kx < nxh && y < ny;
     const long long Nk = (long long)N * nxh;
-    load_twiddles(stw, tw_z, N);
+    load_twiddles2l<TF>(stw, tw_z, N);
+    __shared__ int smx[fx_smx<TF>(256)];
     const zd* src = fields_s + ((long long)f * ny + y) * N * nxh;
     C* xop = Xop + (((long long)f * Nk + kx) * ns + s) * ny + y;
     int bad = 0;
@@ -142,7 +144,7 @@ k_col_inverse_r(const zd* __restrict__ fields_s, int ny, int nxh, int CW, int YB
     }
     if (bad) atomicOr(nonfinite, 1);
     __syncthreads();
-    fft2l<TF, N1, N2, true>(v, lane, xs + (yl * CW + c), N2 * nseq + 1, nseq, stw);
+    fft2l_cols<TF, N1, N2, true>(v, yl * CW + c, nseq, lane, xs + (yl * CW + c), N2 * nseq + 1, nseq, stw, smx);
     if (live) {
         C* dst = G + ((long long)f * ny + y) * N * nxh;
         #pragma unroll
@@ -168,13 +170,14 @@ k_col_forward_r(const cplx<TF>* __restrict__ H, int ny, int nxh, int CW, int YB,
     const int kx = blockIdx.x * CW + c, y = blockIdx.y * YB + yl, j = blockIdx.z;
     const bool live = kx < nxh && y < ny;
     const int Nk = N * nxh;
-    load_twiddles(stw, tw_z, N);
+    load_twiddles2l<TF>(stw, tw_z, N);
+    __shared__ int smx[fx_smx<TF>(256)];
     const C* src = H + ((long long)j * ny + y) * N * nxh;
     C v[N1];
     #pragma unroll
     for (int m = 0; m < N1; ++m) v[m] = live ? src[(long long)(lane + N2 * m) * nxh + kx] : mk((TF)0, (TF)0);
     __syncthreads();
-    fft2l<TF, N1, N2, false>(v, lane, xs + (yl * CW + c), N2 * nseq + 1, nseq, stw);
+    fft2l_cols<TF, N1, N2, false>(v, yl * CW + c, nseq, lane, xs + (yl * CW + c), N2 * nseq + 1, nseq, stw, smx);
     if (live) {
         // the pair products (uu .. vw) carry the factor 2 of the expansion
         const TF inz = (j < 6 ? (TF)2 : (TF)1) / (TF)N;
@@ -271,10 +274,12 @@ __global__ void k_row_products(const cplx<TF>* __restrict__ G, int ny, int nz, i
     }
 }
 
-// Register-FFT row pass for nx = N1 N2 (fft2l): CTA = RZ rows x N2 lanes.
-// Per row: two inverse transforms (u + i v, w + i p), the seven products in
-// registers, four forward transforms, Hermitian split through shared memory.
-// Row sums: FP32 over a thread's N1 points, FP64 across threads.
+// Register-FFT row pass for nx = N1 N2 (fft2l): CTA = RZ rows x N2 lanes, a row
+// within one warp, so only warps synchronise after the twiddles are staged.
+// Per row: two inverse transforms (u + i v, w + i p), the row sums (p is not
+// needed after them), then per packed pair of products a forward transform and
+// its Hermitian split through the row's shared buffer.
+// Row sums: TF over a thread's N1 points, FP64 across threads.
 template <typename TF, int N1, int N2, int RZ>
 __global__ void __launch_bounds__(RZ * N2)
 k_row_products_r(const cplx<TF>* __restrict__ G, int ny, int nz, const cplx<TF>* __restrict__ tw_x,
@@ -282,70 +287,78 @@ k_row_products_r(const cplx<TF>* __restrict__ G, int ny, int nz, const cplx<TF>*
 {
     typedef cplx<TF> C;
     constexpr int N = N1 * N2, nxh = N / 2 + 1;
+    static_assert(32 % N2 == 0, "a row's lanes share a warp");
     extern __shared__ __align__(16) unsigned char sh_raw_rpr[];
     C* stw = (C*)sh_raw_rpr;
-    C* xs = stw + N;                        // [RZ][N1][N2 + 1] exchange
-    C* zb = xs + RZ * N1 * (N2 + 1);        // [RZ][4][N] forward spectra
+    C* xs = stw + N;                        // [RZ][N1][N2 + 1] exchange, then a row's spectrum
+    // u, v, w of the row wait in shared memory [RZ][3][N]: in registers they
+    // would halve the warps in flight
     const int lane = threadIdx.x % N2, r = threadIdx.x / N2;
     const int z = blockIdx.x * RZ + r, y = blockIdx.y;
     const bool live = z < nz;
     const int zz = live ? z : 0;
     C* xr = xs + r * N1 * (N2 + 1);
-    load_twiddles(stw, tw_x, N);
-    C v0[N1], v1[N1];
-    #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const C* ga = G + (((long long)(2 * q) * ny + y) * nz + zz) * nxh;
-        const C* gb = G + (((long long)(2 * q + 1) * ny + y) * nz + zz) * nxh;
-        C* v = q ? v1 : v0;
+    load_twiddles2l<TF>(stw, tw_x, N);
+    __syncthreads();
+    TF* ph = (TF*)(xs + RZ * N1 * (N2 + 1)) + r * 3 * N + lane;
+    TF s6[6] = {0, 0, 0, 0, 0, 0};
+    {
+        C vb[N1];
+        #pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const C* ga = G + (((long long)(2 * q) * ny + y) * nz + zz) * nxh;
+            const C* gb = G + (((long long)(2 * q + 1) * ny + y) * nz + zz) * nxh;
+            C va[N1];
+            C* v = q ? vb : va;
+            #pragma unroll
+            for (int m = 0; m < N1; ++m) {
+                const int k = lane + N2 * m;
+                C A, B;
+                if (k < nxh) { A = ga[k]; B = gb[k]; } else { A = conj(ga[N - k]); B = conj(gb[N - k]); }
+                if (k == 0 || 2 * k == N) { A.y = 0; B.y = 0; }
+                v[m] = mk(A.x - B.y, A.y + B.x);     // A + i B
+            }
+            __syncwarp();
+            fft2l_rows<TF, N1, N2, true>(v, lane, xr, N2 + 1, 1, stw);
+            if (q == 0) {
+                #pragma unroll
+                for (int m = 0; m < N1; ++m) { ph[N2 * m] = va[m].x; ph[N + N2 * m] = va[m].y; }
+            }
+        }
+        // ph: u, v; vb[m] = w + i p at x = lane + N2 m
         #pragma unroll
         for (int m = 0; m < N1; ++m) {
-            const int k = lane + N2 * m;
-            C A, B;
-            if (k < nxh) { A = ga[k]; B = gb[k]; } else { A = conj(ga[N - k]); B = conj(gb[N - k]); }
-            if (k == 0 || 2 * k == N) { A.y = 0; B.y = 0; }
-            v[m] = mk(A.x - B.y, A.y + B.x);     // A + i B
+            const TF u = ph[N2 * m], vv = ph[N + N2 * m], w = vb[m].x, pp = vb[m].y;
+            const TF q = u * u + vv * vv + w * w;
+            s6[0] += q; s6[1] += u * vv; s6[2] += pp * vv; s6[3] += q * u; s6[4] += q * vv; s6[5] += q * w;
+            ph[2 * N + N2 * m] = w;
         }
-        __syncthreads();
-        fft2l<TF, N1, N2, true>(v, lane, xr, N2 + 1, 1, stw);
     }
-    // v0[m] = u + i v, v1[m] = w + i p at x = lane + N2 m
-    TF s6[6] = {0, 0, 0, 0, 0, 0};
-    #pragma unroll
-    for (int m = 0; m < N1; ++m) {
-        const TF u = v0[m].x, vv = v0[m].y, w = v1[m].x, pp = v1[m].y;
-        const TF q = u * u + vv * vv + w * w;
-        s6[0] += q; s6[1] += u * vv; s6[2] += pp * vv; s6[3] += q * u; s6[4] += q * vv; s6[5] += q * w;
-    }
-    #pragma unroll
+    const TF h = (TF)0.5 / (TF)N;
+    #pragma unroll 1
     for (int j = 0; j < 4; ++j) {
         C f[N1];
         #pragma unroll
         for (int m = 0; m < N1; ++m) {
-            const TF u = v0[m].x, vv = v0[m].y, w = v1[m].x;
-            if (j == 0) f[m] = mk(u * u, vv * vv);
-            else if (j == 1) f[m] = mk(w * w, u * vv);
-            else if (j == 2) f[m] = mk(u * w, vv * w);
-            else f[m] = mk(u * u + vv * vv + w * w, (TF)0);
+            const TF u = ph[N2 * m], vv = ph[N + N2 * m], w = ph[2 * N + N2 * m];
+            f[m] = j == 0 ? mk(u * u, vv * vv) : j == 1 ? mk(w * w, u * vv) : j == 2 ? mk(u * w, vv * w)
+                          : mk(u * u + vv * vv + w * w, (TF)0);
         }
-        __syncthreads();
-        fft2l<TF, N1, N2, false>(f, lane, xr, N2 + 1, 1, stw);
+        __syncwarp();
+        fft2l_rows<TF, N1, N2, false>(f, lane, xr, N2 + 1, 1, stw);
+        __syncwarp();
         #pragma unroll
-        for (int m = 0; m < N1; ++m) zb[(r * 4 + j) * N + lane + N2 * m] = f[m];
-    }
-    __syncthreads();
-    const TF h = (TF)0.5 / (TF)N;
-    if (live) {
-        for (int it = lane; it < 4 * nxh; it += N2) {
-            const int j = it / nxh, k = it - j * nxh;
-            const C* seq = zb + (r * 4 + j) * N;
-            const C Z = seq[k], Zc = conj(seq[(N - k) & (N - 1)]);
-            const C A = h * (Z + Zc);
-            const C D = Z - Zc;
-            const C B = mk(h * D.y, -h * D.x);     // -i/2 (Z - Zc)
-            H[(((long long)(2 * j) * ny + y) * nz + z) * nxh + k] = A;
-            if (j < 3) H[(((long long)(2 * j + 1) * ny + y) * nz + z) * nxh + k] = B;
-        }
+        for (int m = 0; m < N1; ++m) xr[lane + N2 * m] = f[m];
+        __syncwarp();
+        if (live)
+            for (int k = lane; k < nxh; k += N2) {
+                const C Z = xr[k], Zc = conj(xr[(N - k) & (N - 1)]);
+                const C A = h * (Z + Zc);
+                const C D = Z - Zc;
+                const C B = mk(h * D.y, -h * D.x);     // -i/2 (Z - Zc)
+                H[(((long long)(2 * j) * ny + y) * nz + z) * nxh + k] = A;
+                if (j < 3) H[(((long long)(2 * j + 1) * ny + y) * nz + z) * nxh + k] = B;
+            }
     }
     // block reduction of the row sums (FP64 across threads)
     __shared__ double red[6][32];
@@ -521,7 +534,7 @@ int products_launch(const ProdArgs& a)
         }
         const int nrb = (nx == 256) ? (nz + 3) / 4 : (nz + a.rz_rp - 1) / a.rz_rp;
         if (nx == 256) {
-            k_row_products_r<TF, 16, 16, 4><<<dim3(nrb, ny), 4 * 16, (256 + 4 * 16 * 17 + 4 * 4 * 256) * sizeof(C),
+            k_row_products_r<TF, 16, 16, 4><<<dim3(nrb, ny), 4 * 16, (256 + 4 * 16 * 17) * sizeof(C) + 4 * 3 * 256 * sizeof(TF),
                                               ss>>>((const C*)G, ny, nz, (const C*)a.tw_x, H, part);
         } else {
             k_row_products<TF><<<dim3(nrb, ny), 256, (1 + 8 * a.rz_rp) * nx * sizeof(C), ss>>>(

@@ -19,6 +19,7 @@
 // one-point part, a function of (Y1, Y2) only, in FP64 once per pair, so the
 // large one-point values never pass through an FP32 difference.
 #include "gke_common.cuh"
+#include "gke_fixed.cuh"
 #include "gke_kernels.h"
 
 namespace gke {
@@ -64,7 +65,7 @@ __global__ void k_terms_colpass(const cplx<TB>* __restrict__ comb, long long pai
 // register-FFT column pass for nz = N1 N2: CTA = CW columns of one term of
 // one pair x N2 lanes (see fft2l)
 template <typename TF, typename TB, int N1, int N2, bool US>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
 k_terms_colpass_r(const cplx<TB>* __restrict__ comb, long long pair0, int nxh, int CW,
                   const cplx<TF>* __restrict__ tw_z, SepMap sm, unsigned tmask, cplx<TF>* __restrict__ W)
 {
@@ -77,7 +78,8 @@ k_terms_colpass_r(const cplx<TB>* __restrict__ comb, long long pair0, int nxh, i
     const int kx = blockIdx.x * CW + c, q = nth_bit(tmask, blockIdx.y);
     const long long pl = blockIdx.z, p = pair0 + pl;
     const int Nk = N * nxh;
-    load_twiddles(stw, tw_z, N);
+    load_twiddles2l<TF>(stw, tw_z, N);
+    __shared__ int smx[fx_smx<TF>(256)];
     const cplx<TB>* src = comb + (p * NTERM + q) * (long long)Nk;
     C v[N1];
     #pragma unroll
@@ -90,7 +92,7 @@ k_terms_colpass_r(const cplx<TB>* __restrict__ comb, long long pair0, int nxh, i
         v[m] = x;
     }
     __syncthreads();
-    fft2l<TF, N1, N2, true>(v, lane, xs + c, N2 * CW + 1, CW, stw);
+    fft2l_cols<TF, N1, N2, true>(v, c, CW, lane, xs + c, N2 * CW + 1, CW, stw, smx);
     if (kx < nxh) {
         C* dst = W + (pl * NTERM + q) * (long long)(US ? sm.nrz : N) * nxh;
         #pragma unroll
@@ -208,12 +210,13 @@ k_terms_rowpass_r(const cplx<TF>* __restrict__ W, const int* __restrict__ pair_i
     const bool live = z < nz;
     const long long pl = blockIdx.y, p = pair0 + pl;
     const int i1 = pair_i[2 * p], i2 = pair_i[2 * p + 1];
-    load_twiddles(stw, tw_x, N);
+    load_twiddles2l<TF>(stw, tw_x, N);
     if (threadIdx.x == 0) {
         double one[NTERM];
         onepoint(prof, ny, i1, i2, one);
         for (int t = 0; t < NTERM; ++t) s_one[t] = (TF)one[t];
     }
+    __syncthreads();                         // s_one, twiddles
     const long long NN = (long long)nz * nrx;
     const TF ic = (TF)inv_count;
     C* xr = xs + r * N1 * (N2 + 1);
@@ -233,8 +236,8 @@ k_terms_rowpass_r(const cplx<TF>* __restrict__ W, const int* __restrict__ pair_i
             if (k == 0 || 2 * k == N) { A.y = 0; B.y = 0; }
             v[m] = mk(A.x - B.y, A.y + B.x);
         }
-        __syncthreads();                     // exchange buffer free (and s_one, twiddles ready)
-        fft2l<TF, N1, N2, true>(v, lane, xr, N2 + 1, 1, stw);
+        __syncwarp();                        // exchange buffer free (a row's lanes share a warp)
+        fft2l_rows<TF, N1, N2, true>(v, lane, xr, N2 + 1, 1, stw);
         if (live) {
             #pragma unroll
             for (int m = 0; m < N1; ++m) {
