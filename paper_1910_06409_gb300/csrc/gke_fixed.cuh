@@ -15,7 +15,8 @@
 //
 // Measured (FP64 transforms -> here): 256 x 256 x 65, 16 snapshots: inverse transforms
 // of the terms 56.9 -> 19.8 ms, products stage 46.7 -> 24.4 ms; duct 256 x 33 x 33:
-// 30.0 -> 12.9 ms.  Errors of the terms against 64-bit references do not grow (duct
+// 30.0 -> 12.9 ms; 128 x 128 x 65, 32 snapshots (from shared-memory stages of FP64):
+// products 28.7 -> 12.3 ms, terms 15.3 -> 5.1 ms.  Errors of the terms against 64-bit references do not grow (duct
 // A 1.6e-16 -> 1.2e-16).  (Exponents from the largest component and 56 bits were as
 // fast, but raised them by up to a half.)
 #pragma once
@@ -171,7 +172,7 @@ __device__ __forceinline__ void fft2l_fixed(zd* v, int E, int lane, zx* xs, int 
 }
 
 // lengths with a register transform
-inline bool fx_len(int n) { return n == 64 || n == 128 || n == 256 || n == 512; }
+inline bool fx_len(int n) { return n == 32 || n == 64 || n == 128 || n == 256 || n == 512; }
 // cos, sin of 2 pi m / 512 times 2^62, rounded, m = 0 .. 64
 static const long long fx_octant[65][2] = {
     {4611686018427387904ll, 0ll}, {4611338766951757487ll, 56592481536850979ll},

@@ -102,6 +102,17 @@ inline bool fft_len_ok(int n)
     return pow2(n) || (n % 3 == 0 && pow2(n / 3));
 }
 
+// lengths whose transforms run in registers (fft2l), with their split N1 N2
+inline bool reg_len(int n) { return n == 32 || n == 64 || n == 128 || n == 256; }
+template <int A, int B> struct RegLen { static constexpr int N1 = A, N2 = B, N = A * B; };
+template <typename F> inline void with_reg_len(int n, F f)
+{
+    if (n == 256) f(RegLen<16, 16>());
+    else if (n == 128) f(RegLen<16, 8>());
+    else if (n == 64) f(RegLen<8, 8>());
+    else f(RegLen<8, 4>());
+}
+
 int combine_kc(bool fp32);
 bool combine_kc_ok(bool fp32, int kc);
 

@@ -8,6 +8,7 @@
 // complex sequence).  The transform arithmetic runs in TF = double (plain
 // path) or float (split path); one-point sums are always FP64.
 #include <algorithm>
+#include <vector>
 
 #include "gke_common.cuh"
 #include "gke_fixed.cuh"
@@ -418,55 +419,80 @@ __global__ void k_col_forward(const cplx<TF>* __restrict__ H, int ny, int nz, in
 //   part[y][chunk] = sum_{s, k in chunk, i} w_k [ (kx^2 + kz^2) |u_i(y,k)|^2 + |d_y u_i(y,k)|^2 ],
 // d_y by the 5-point FD stencil applied to the coefficients (it commutes with
 // the transform); w_k = 1 on the kx = 0 and kx = nx/2 lines, 2 elsewhere (half
-// spectrum).  One thread per y; arithmetic in TF, the running sum compensated
-// (Kahan) so an FP32 pass keeps ~1e-7 relative accuracy; partials reduced in
-// FP64 in a fixed order by k_reduce_partials.
+// spectrum).  CTA = one chunk, threads (y, k mod KT); arithmetic in TF.  The
+// chunk's wavenumbers of a y are then summed in their order, compensated (Kahan)
+// so an FP32 pass keeps ~1e-7 relative accuracy, and the partials reduced in
+// FP64 in a fixed order by k_reduce_partials.  Latency bound on small grids: with
+// one thread per y walking its 16 wavenumbers a launch took 106 us at 32 x 32 x 9, 2
+// snapshots.
+constexpr int EPS_THREADS = 512, EPS_Y = 256;        // threads, rows y of a CTA at most
 template <typename TF>
-__global__ void k_eps(const cplx<TF>* __restrict__ Xop, int ns, int ny, int nz, int nxh, int nx,
-                      double Lx, double Lz, const double* __restrict__ fdw, const int* __restrict__ fdl0,
-                      int kchunk, double* __restrict__ part)
+__global__ void __launch_bounds__(EPS_THREADS)
+k_eps(const cplx<TF>* __restrict__ Xop, int ns, int ny, int nz, int nxh, int nx, double Lx, double Lz,
+      const double* __restrict__ fdw, const int* __restrict__ fdl0, int yt, int kt, double* __restrict__ part)
 {
+    __shared__ TF term[EPS_KCHUNK * EPS_Y];
     const int Nk = nz * nxh;
-    const int kbeg = blockIdx.x * kchunk, kend = min(Nk, kbeg + kchunk);
+    const int kbeg = blockIdx.x * EPS_KCHUNK, nk = min(Nk - kbeg, EPS_KCHUNK);
     const TF cx = (TF)(2.0 * 3.14159265358979323846 / Lx), cz = (TF)(2.0 * 3.14159265358979323846 / Lz);
-    for (int y = threadIdx.x; y < ny; y += blockDim.x) {
-        const int l0 = fdl0[y];
-        TF w5[5];
-        for (int l = 0; l < 5; ++l) w5[l] = (TF)fdw[5 * y + l];
-        TF sum = 0, comp = 0;
-        for (int k = kbeg; k < kend; ++k) {
-            const int kz_i = k / nxh, kx_i = k - kz_i * nxh;
-            const TF kx = cx * (TF)signed_bin(kx_i, nx), kz = cz * (TF)signed_bin(kz_i, nz);
-            const TF wk = (kx_i == 0 || 2 * kx_i == nx) ? (TF)1 : (TF)2;
-            const TF k2 = kx * kx + kz * kz;
-            TF acc = 0;
-            for (int i = 0; i < 3; ++i)
-                for (int s = 0; s < ns; ++s) {
-                    const cplx<TF>* col = Xop + (((long long)i * Nk + k) * ns + s) * ny;
-                    const cplx<TF> a = col[y];
-                    TF dr = 0, di = 0;
-                    #pragma unroll
-                    for (int l = 0; l < 5; ++l) { const cplx<TF> b = col[l0 + l]; dr += w5[l] * b.x; di += w5[l] * b.y; }
-                    acc += k2 * (a.x * a.x + a.y * a.y) + dr * dr + di * di;
-                }
-            // compensated add of this wavenumber's contribution
-            const TF yk = wk * acc - comp;
+    const int KT = kt, yl = threadIdx.x % yt, kk = threadIdx.x / yt;
+    // wavenumber kbeg + kl of row y
+    auto value = [&](int kl, int y, int l0, const TF* w5) {
+        const int k = kbeg + kl, kz_i = k / nxh, kx_i = k - kz_i * nxh;
+        const TF kx = cx * (TF)signed_bin(kx_i, nx), kz = cz * (TF)signed_bin(kz_i, nz);
+        const TF wk = (kx_i == 0 || 2 * kx_i == nx) ? (TF)1 : (TF)2;
+        const TF k2 = kx * kx + kz * kz;
+        TF acc = 0;
+        for (int i = 0; i < 3; ++i)
+            for (int s = 0; s < ns; ++s) {
+                const cplx<TF>* col = Xop + (((long long)i * Nk + k) * ns + s) * ny;
+                const cplx<TF> a = col[y];
+                TF dr = 0, di = 0;
+                #pragma unroll
+                for (int l = 0; l < 5; ++l) { const cplx<TF> b = col[l0 + l]; dr += w5[l] * b.x; di += w5[l] * b.y; }
+                acc += k2 * (a.x * a.x + a.y * a.y) + dr * dr + di * di;
+            }
+        return wk * acc;
+    };
+    for (int y0 = 0; y0 < ny; y0 += yt) {
+        const int y = y0 + yl;
+        const bool live = y < ny && kk < KT;
+        TF w5[5], sum = 0, comp = 0;
+        const int l0 = live ? fdl0[y] : 0;
+        if (live)
+            for (int l = 0; l < 5; ++l) w5[l] = (TF)fdw[5 * y + l];
+        auto add = [&](TF v) {
+            const TF yk = v - comp;
             const TF t = sum + yk;
             comp = (t - sum) - yk;
             sum = t;
+        };
+        if (KT == 1) {
+            if (live)
+                for (int kl = 0; kl < nk; ++kl) add(value(kl, y, l0, w5));
+        } else {
+            if (live)
+                for (int kl = kk; kl < nk; kl += KT) term[kl * yt + yl] = value(kl, y, l0, w5);
+            __syncthreads();
+            if (kk == 0 && live)
+                for (int kl = 0; kl < nk; ++kl) add(term[kl * yt + yl]);
+            __syncthreads();
         }
-        part[(long long)y * gridDim.x + blockIdx.x] = (double)sum;
+        if (kk == 0 && live) part[(long long)y * gridDim.x + blockIdx.x] = (double)sum;
     }
 }
 
-// out[j] += sum_b part[j * nb + b], b in increasing order (deterministic)
+// out[j] += sum_b part[j * nb + b]: a warp per j, 32 strided sums and a tree, in
+// a fixed order (deterministic).  One thread per j took nb dependent additions
+// (and their rounding); 128 threads = 4 values a block.
 __global__ void k_reduce_partials(const double* __restrict__ part, int nvals, int nb, double* __restrict__ out)
 {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j >= nvals) return;
     double acc = 0.0;
-    for (int b = 0; b < nb; ++b) acc += part[(long long)j * nb + b];
-    out[j] += acc;
+    for (int b = lane; b < nb; b += 32) acc += part[(long long)j * nb + b];
+    acc = warp_sum(acc);
+    if (lane == 0) out[j] += acc;
 }
 
 // ------------------------------------------------------------------ host
@@ -480,8 +506,13 @@ int products_launch(const ProdArgs& a)
     C* Xop = (C*)a.Xop;
     int launches = 0;
     const int nch = (ny + ll_rows<TF>() - 1) / ll_rows<TF>(), rows = (ny + nch - 1) / nch;
-    // at nz = 256 the register column pass writes the linear operands itself
-    const bool fused_load = nz == 256;
+    // register transforms, but FP64 ones of 32 points only where enough rows
+    // hide their longer chain of integer instructions (32 x 32 x 9, 2 snapshots: row
+    // pass 21 -> 46 us; 32 x 32 x 33, 4 snapshots: products stage 333 -> 322)
+    auto reg = [&](int n, int other) { return reg_len(n) && (n > 32 || sizeof(TF) == 4 || (long long)other * ny >= 1024); };
+    const bool reg_z = reg(nz, nxh * 2), reg_x = reg(nx, nz);
+    // the register column pass writes the linear operands itself
+    const bool fused_load = reg_z;
     if (!a.up_ev && !fused_load) {
         k_load_linear<TF><<<dim3((Nk + 31) / 32, nch, ns * 4), dim3(32, 8), 0, st>>>(a.fields, ns, ny, Nk, rows, 0,
                                                                                       a.mean, Xop, a.nonfinite);
@@ -522,20 +553,30 @@ int products_launch(const ProdArgs& a)
                                                                                      a.mean, Xop, a.nonfinite);
             ++launches;
         }
-        if (nz == 256) {
-            // FP32: 4 kx x 8 planes per CTA; FP64 4 x 4 (shared memory)
-            constexpr int CWR = 4, YBR = sizeof(TF) == 4 ? 8 : 4;
-            k_col_inverse_r<TF, 16, 16><<<dim3((nxh + CWR - 1) / CWR, (ny + YBR - 1) / YBR, 4), CWR * YBR * 16,
-                                          (256 + 16 * (16 * CWR * YBR + 1)) * sizeof(C), ss>>>(
-                fs, ny, nxh, CWR, YBR, s, ns, a.mean, (const C*)a.tw_z, G, Xop, a.nonfinite);
+        if (reg_z) {
+            // 4 kx x YB planes per CTA, 256 threads in FP64 and 512 in FP32
+            // (operand stores in runs of YB planes; shared memory bounds FP64)
+            with_reg_len(nz, [&](auto L) {
+                typedef decltype(L) R;
+                constexpr int CWR = 4, YBR = (sizeof(TF) == 4 ? 128 : 64) / R::N2;
+                k_col_inverse_r<TF, R::N1, R::N2><<<dim3((nxh + CWR - 1) / CWR, (ny + YBR - 1) / YBR, 4), CWR * YBR * R::N2,
+                                                    (R::N + R::N1 * (R::N2 * CWR * YBR + 1)) * sizeof(C), ss>>>(
+                    fs, ny, nxh, CWR, YBR, s, ns, a.mean, (const C*)a.tw_z, G, Xop, a.nonfinite);
+            });
         } else {
             k_col_inverse<TF><<<dim3((nxh + a.cw_ci - 1) / a.cw_ci, ny, 4), 256, (1 + 2 * a.cw_ci) * nz * sizeof(C), ss>>>(
                 fs, ny, nz, nxh, a.cw_ci, a.mean, (const C*)a.tw_z, G);
         }
-        const int nrb = (nx == 256) ? (nz + 3) / 4 : (nz + a.rz_rp - 1) / a.rz_rp;
-        if (nx == 256) {
-            k_row_products_r<TF, 16, 16, 4><<<dim3(nrb, ny), 4 * 16, (256 + 4 * 16 * 17) * sizeof(C) + 4 * 3 * 256 * sizeof(TF),
-                                              ss>>>((const C*)G, ny, nz, (const C*)a.tw_x, H, part);
+        int nrb = (nz + a.rz_rp - 1) / a.rz_rp;
+        if (reg_x) {
+            with_reg_len(nx, [&](auto L) {
+                typedef decltype(L) R;
+                constexpr int RZ = 64 / R::N2;
+                nrb = (nz + RZ - 1) / RZ;
+                k_row_products_r<TF, R::N1, R::N2, RZ><<<dim3(nrb, ny), 64, (R::N + RZ * R::N1 * (R::N2 + 1)) * sizeof(C) +
+                                                                           RZ * 3 * R::N * sizeof(TF), ss>>>(
+                    (const C*)G, ny, nz, (const C*)a.tw_x, H, part);
+            });
         } else {
             k_row_products<TF><<<dim3(nrb, ny), 256, (1 + 8 * a.rz_rp) * nx * sizeof(C), ss>>>(
                 (const C*)G, ny, nz, nx, a.rz_rp, (const C*)a.tw_x, H, part);
@@ -544,15 +585,16 @@ int products_launch(const ProdArgs& a)
             cudaEventRecord(ev_rp[b], ss);
             cudaStreamWaitEvent(st, ev_rp[b], 0);
         }
-        k_reduce_partials<<<(6 * ny + 127) / 128, 128, 0, st>>>(part, 6 * ny, nrb, a.stats);
+        k_reduce_partials<<<(6 * ny + 3) / 4, 128, 0, st>>>(part, 6 * ny, nrb, a.stats);
         if (two) cudaEventRecord(ev_red[b], st);
-        if (nz == 256) {
-            // FP32: 8 planes per CTA (the operand stores come in 64-byte runs);
-            // FP64 keeps 4 (its exchange buffer would hold one CTA per SM)
-            constexpr int CWR = 4, YBR = sizeof(TF) == 4 ? 8 : 4;
-            k_col_forward_r<TF, 16, 16><<<dim3((nxh + CWR - 1) / CWR, (ny + YBR - 1) / YBR, 7), CWR * YBR * 16,
-                                          (256 + 16 * (16 * CWR * YBR + 1)) * sizeof(C), ss>>>(
-                (const C*)H, ny, nxh, CWR, YBR, s, ns, (const C*)a.tw_z, Xop);
+        if (reg_z) {
+            with_reg_len(nz, [&](auto L) {
+                typedef decltype(L) R;
+                constexpr int CWR = 4, YBR = (sizeof(TF) == 4 ? 128 : 64) / R::N2;
+                k_col_forward_r<TF, R::N1, R::N2><<<dim3((nxh + CWR - 1) / CWR, (ny + YBR - 1) / YBR, 7), CWR * YBR * R::N2,
+                                                    (R::N + R::N1 * (R::N2 * CWR * YBR + 1)) * sizeof(C), ss>>>(
+                    (const C*)H, ny, nxh, CWR, YBR, s, ns, (const C*)a.tw_z, Xop);
+            });
         } else {
             k_col_forward<TF><<<dim3((nxh + a.cw_cf - 1) / a.cw_cf, (ny + a.yb_cf - 1) / a.yb_cf, 7), 256,
                                 (1 + 2 * a.cw_cf * a.yb_cf) * nz * sizeof(C), ss>>>(
@@ -573,12 +615,15 @@ int products_launch(const ProdArgs& a)
             }
         }
     }
-    const int neb = (Nk + a.eps_kchunk - 1) / a.eps_kchunk;
-    // one thread per wall-normal row: no second pass for a ragged last row
-    const int eps_threads = std::min(1024, (ny + 31) / 32 * 32);
-    k_eps<TF><<<neb, eps_threads, 0, st>>>(Xop, ns, ny, nz, nxh, nx, a.Lx, a.Lz, a.fdw, a.fdl0, a.eps_kchunk,
-                                          a.part);
-    k_reduce_partials<<<(ny + 127) / 128, 128, 0, st>>>(a.part, ny, neb, a.stats + S_EPS * ny);
+    const int neb = (Nk + EPS_KCHUNK - 1) / EPS_KCHUNK;
+    // whole rows y per k, as many k side by side as fit; FP32 passes with a
+    // thousand chunks fill the chip with one k at a time, whose rows stream
+    // better (256 x 256 x 129, 16 snapshots: products stage 10.55 -> 9.67 ms; FP64, bound by
+    // its arithmetic, gains from more at any size: 256 x 256 x 65 24.4 -> 23.0 ms)
+    const int yt = std::min(ny, EPS_Y);
+    const int kt = sizeof(TF) == 4 && neb >= 1024 ? 1 : std::min(EPS_KCHUNK, EPS_THREADS / yt);
+    k_eps<TF><<<neb, kt == 1 ? (yt + 31) / 32 * 32 : yt * kt, 0, st>>>(Xop, ns, ny, nz, nxh, nx, a.Lx, a.Lz, a.fdw, a.fdl0, yt, kt, a.part);
+    k_reduce_partials<<<(ny + 3) / 4, 128, 0, st>>>(a.part, ny, neb, a.stats + S_EPS * ny);
     return launches + 2;
 }
 template int products_launch<double>(const ProdArgs&);
@@ -595,14 +640,20 @@ static cudaError_t set_dyn_smem(const void* k, int lim)
 
 cudaError_t products_set_attrs(int lim)
 {
-    const void* ks[] = {(const void*)k_col_inverse<double>, (const void*)k_row_products<double>,
-                        (const void*)k_col_forward<double>, (const void*)k_col_inverse<float>,
-                        (const void*)k_row_products<float>, (const void*)k_col_forward<float>,
-                        (const void*)k_col_inverse_r<double, 16, 16>, (const void*)k_col_inverse_r<float, 16, 16>,
-                        (const void*)k_col_forward_r<double, 16, 16>, (const void*)k_col_forward_r<float, 16, 16>,
-                        (const void*)k_row_products_r<double, 16, 16, 4>, (const void*)k_row_products_r<float, 16, 16, 4>};
+    std::vector<const void*> ks = {(const void*)k_col_inverse<double>, (const void*)k_row_products<double>,
+                                   (const void*)k_col_forward<double>, (const void*)k_col_inverse<float>,
+                                   (const void*)k_row_products<float>, (const void*)k_col_forward<float>};
+    for (int n : {32, 64, 128, 256})
+        with_reg_len(n, [&](auto L) {
+            typedef decltype(L) R;
+            for (const void* k : {(const void*)k_col_inverse_r<double, R::N1, R::N2>, (const void*)k_col_inverse_r<float, R::N1, R::N2>,
+                                  (const void*)k_col_forward_r<double, R::N1, R::N2>, (const void*)k_col_forward_r<float, R::N1, R::N2>,
+                                  (const void*)k_row_products_r<double, R::N1, R::N2, 64 / R::N2>,
+                                  (const void*)k_row_products_r<float, R::N1, R::N2, 64 / R::N2>})
+                ks.push_back(k);
+        });
     cudaError_t e = cudaSuccess;
-    for (const void* k : ks) { cudaError_t r = set_dyn_smem(k, lim); if (r != cudaSuccess) e = r; }
+    for (const void* k : ks) { const cudaError_t r = set_dyn_smem(k, lim); if (r != cudaSuccess) e = r; }
     return e;
 }
 
@@ -617,7 +668,7 @@ cudaError_t products_set_attrs(int lim)
     template __global__ void k_col_forward<TF>(const cplx<TF>*, int, int, int, int, int, int, int,         \
                                                const cplx<TF>*, cplx<TF>*);                                \
     template __global__ void k_eps<TF>(const cplx<TF>*, int, int, int, int, int, double, double,           \
-                                       const double*, const int*, int, double*);
+                                       const double*, const int*, int, int, double*);
 GKE_INST(double)
 GKE_INST(float)
 #undef GKE_INST

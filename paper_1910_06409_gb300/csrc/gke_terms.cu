@@ -18,6 +18,8 @@
 // spectral part of each term (kept apart in FP32 scratch) in FP32 and the
 // one-point part, a function of (Y1, Y2) only, in FP64 once per pair, so the
 // large one-point values never pass through an FP32 difference.
+#include <vector>
+
 #include "gke_common.cuh"
 #include "gke_fixed.cuh"
 #include "gke_kernels.h"
@@ -750,16 +752,20 @@ int terms_launch_t(const TermArgs& a)
         cudaStream_t sc = a.st, sr = two ? a.st2 : a.st;
         if (two && c >= 2) cudaStreamWaitEvent(sc, ev_row[buf], 0);     // W buffer free again
         if (a.planes) {
-            colpass_planes_launch<TF, TB>(a, p0, np, W, sc, us);        } else if (a.nz == 256) {
-            constexpr int CWR = 16;
-            const dim3 g((nxh + CWR - 1) / CWR, ntm, (unsigned)np);
-            const size_t sh = (256 + 16 * (16 * CWR + 1)) * sizeof(C);
-            if (us)
-                k_terms_colpass_r<TF, TB, 16, 16, true><<<g, CWR * 16, sh, sc>>>(
-                    (const cplx<TB>*)a.comb, p0, nxh, CWR, (const C*)a.tw_z, a.sep, a.tmask, W);
-            else
-                k_terms_colpass_r<TF, TB, 16, 16, false><<<g, CWR * 16, sh, sc>>>(
-                    (const cplx<TB>*)a.comb, p0, nxh, CWR, (const C*)a.tw_z, a.sep, a.tmask, W);
+            colpass_planes_launch<TF, TB>(a, p0, np, W, sc, us);
+        } else if (reg_len(a.nz)) {
+            with_reg_len(a.nz, [&](auto L) {
+                typedef decltype(L) R;
+                constexpr int CWR = 16;
+                const dim3 g((nxh + CWR - 1) / CWR, ntm, (unsigned)np);
+                const size_t sh = (R::N + R::N1 * (R::N2 * CWR + 1)) * sizeof(C);
+                if (us)
+                    k_terms_colpass_r<TF, TB, R::N1, R::N2, true><<<g, CWR * R::N2, sh, sc>>>(
+                        (const cplx<TB>*)a.comb, p0, nxh, CWR, (const C*)a.tw_z, a.sep, a.tmask, W);
+                else
+                    k_terms_colpass_r<TF, TB, R::N1, R::N2, false><<<g, CWR * R::N2, sh, sc>>>(
+                        (const cplx<TB>*)a.comb, p0, nxh, CWR, (const C*)a.tw_z, a.sep, a.tmask, W);
+            });
         } else {
             k_terms_colpass<TF, TB><<<dim3((nxh + a.cw - 1) / a.cw, ntm, (unsigned)np), 256,
                                       (1 + 2 * a.cw) * a.nz * sizeof(C), sc>>>(
@@ -771,18 +777,21 @@ int terms_launch_t(const TermArgs& a)
         }
         if (sizeof(TF) == 4 && a.planes && a.nz == 256 && a.nx == 256) {
             rowpass_pt_launch<TF, TO>(a, p0, np, W, sr, us);
-        } else if (a.nx == 256) {
-            constexpr int RZR = 4;
-            const dim3 g((a.sep.nrz + RZR - 1) / RZR, (unsigned)np);
-            const size_t sh = (256 + RZR * 16 * 17) * sizeof(C);
-            if (us)
-                k_terms_rowpass_r<TF, TO, 16, 16, true><<<g, RZR * 16, sh, sr>>>(
-                    W, a.pair_i, p0, a.npair, a.ny, RZR, a.inv_count, a.prof, (const C*)a.tw_x, a.sep,
-                    a.tmask, (TO*)a.terms, a.spec);
-            else
-                k_terms_rowpass_r<TF, TO, 16, 16, false><<<g, RZR * 16, sh, sr>>>(
-                    W, a.pair_i, p0, a.npair, a.ny, RZR, a.inv_count, a.prof, (const C*)a.tw_x, a.sep,
-                    a.tmask, (TO*)a.terms, a.spec);
+        } else if (reg_len(a.nx)) {
+            with_reg_len(a.nx, [&](auto L) {
+                typedef decltype(L) R;
+                constexpr int RZR = 64 / R::N2;
+                const dim3 g((a.sep.nrz + RZR - 1) / RZR, (unsigned)np);
+                const size_t sh = (R::N + RZR * R::N1 * (R::N2 + 1)) * sizeof(C);
+                if (us)
+                    k_terms_rowpass_r<TF, TO, R::N1, R::N2, true><<<g, 64, sh, sr>>>(
+                        W, a.pair_i, p0, a.npair, a.ny, RZR, a.inv_count, a.prof, (const C*)a.tw_x, a.sep,
+                        a.tmask, (TO*)a.terms, a.spec);
+                else
+                    k_terms_rowpass_r<TF, TO, R::N1, R::N2, false><<<g, 64, sh, sr>>>(
+                        W, a.pair_i, p0, a.npair, a.ny, RZR, a.inv_count, a.prof, (const C*)a.tw_x, a.sep,
+                        a.tmask, (TO*)a.terms, a.spec);
+            });
         } else {
             k_terms_rowpass<TF, TO><<<dim3((a.sep.nrz + a.rz - 1) / a.rz, (unsigned)np), 256,
                                       (1 + 8 * a.rz) * a.nx * sizeof(C), sr>>>(
@@ -815,19 +824,9 @@ int terms_launch(const TermArgs& a)
 
 cudaError_t terms_set_attrs(int lim)
 {
-    const void* ks[] = {(const void*)k_terms_colpass<double, double>, (const void*)k_terms_rowpass<double, double>,
+    std::vector<const void*> ks = {(const void*)k_terms_colpass<double, double>, (const void*)k_terms_rowpass<double, double>,
                         (const void*)k_terms_colpass<float, float>, (const void*)k_terms_colpass<float, double>,
                         (const void*)k_terms_rowpass<float, float>,
-                        (const void*)k_terms_colpass_r<double, double, 16, 16, false>,
-                        (const void*)k_terms_colpass_r<float, float, 16, 16, false>,
-                        (const void*)k_terms_colpass_r<float, double, 16, 16, false>,
-                        (const void*)k_terms_rowpass_r<double, double, 16, 16, false>,
-                        (const void*)k_terms_rowpass_r<float, float, 16, 16, false>,
-                        (const void*)k_terms_colpass_r<double, double, 16, 16, true>,
-                        (const void*)k_terms_colpass_r<float, float, 16, 16, true>,
-                        (const void*)k_terms_colpass_r<float, double, 16, 16, true>,
-                        (const void*)k_terms_rowpass_r<double, double, 16, 16, true>,
-                        (const void*)k_terms_rowpass_r<float, float, 16, 16, true>,
                         (const void*)k_terms_colpass_planes_r<float, float, 16, 16, false>,
                         (const void*)k_terms_colpass_planes_r<float, double, 16, 16, false>,
                         (const void*)k_terms_colpass_planes_r<float, float, 16, 16, true>,
@@ -840,6 +839,17 @@ cudaError_t terms_set_attrs(int lim)
                         (const void*)k_terms_colpass_pt<float, double, 16, 16, true>,
                         (const void*)k_terms_rowpass_p4<float, float, 16, 16, false>,
                         (const void*)k_terms_rowpass_p4<float, float, 16, 16, true>};
+    for (int n : {32, 64, 128, 256})
+        with_reg_len(n, [&](auto L) {
+            typedef decltype(L) R;
+            constexpr int A = R::N1, B = R::N2;
+            for (const void* k : {(const void*)k_terms_colpass_r<double, double, A, B, false>, (const void*)k_terms_colpass_r<double, double, A, B, true>,
+                                  (const void*)k_terms_colpass_r<float, float, A, B, false>, (const void*)k_terms_colpass_r<float, float, A, B, true>,
+                                  (const void*)k_terms_colpass_r<float, double, A, B, false>, (const void*)k_terms_colpass_r<float, double, A, B, true>,
+                                  (const void*)k_terms_rowpass_r<double, double, A, B, false>, (const void*)k_terms_rowpass_r<double, double, A, B, true>,
+                                  (const void*)k_terms_rowpass_r<float, float, A, B, false>, (const void*)k_terms_rowpass_r<float, float, A, B, true>})
+                ks.push_back(k);
+        });
     cudaError_t e = cudaSuccess;
     for (const void* k : ks) {
         cudaFuncAttributes fa;
