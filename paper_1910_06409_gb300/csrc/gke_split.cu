@@ -74,10 +74,6 @@ __constant__ TcJob c_tcplanes[NPLANE];
 // partner-free form below needs no per-row factor
 __constant__ TcJob c_tcoff[NPLANE];
 
-// cross-slice pairs (i, j), 0 < i + j <= 2; the pair (0, 0) goes last
-__constant__ int c_pi[5] = {1, 0, 2, 1, 0};
-__constant__ int c_pj[5] = {1, 2, 0, 0, 1};
-
 // Packed K (one snapshot group of ns <= 5): the six slice products of a term
 // in three MMA K steps instead of six zero-padded ones, one step per order of
 // magnitude so that an MMA never sums products of different sizes: step 0
@@ -269,12 +265,58 @@ struct TcArgs {
     int* err;
 };
 
+// The MMAs of one stage of one term.  Slice pairs (i, j), 0 < i + j <= 2, in
+// pass 0 and (0, 0) in pass 1; packed, the K steps 0 and 1, then 2.  An MMA of
+// 64 to 128 clocks is issued at that rate only if its descriptors are
+// immediate offsets in straight-line code of a converged warp: with a loop
+// over the pairs from one lane an issue took 94 to 174 clocks.  Correlation
+// stage of 256 x 256 x 129, 16 snapshots: 11.7 -> 10.5 ms (9.0 ms without
+// any MMA, 9.4 ms without the epilogue); 128 x 128 x 65, 32 snapshots:
+// 5.1 -> 4.6 ms.
+enum { PS_CROSS, PS_PACKED, PS_LAST };
+template <int PS> struct PairSet {
+    static constexpr int n = PS == PS_CROSS ? 5 : PS == PS_PACKED ? 2 : 1;
+    static __device__ __forceinline__ constexpr int i(int p) { return PS == PS_CROSS ? (p == 0 || p == 3 ? 1 : p == 2 ? 2 : 0) : p; }
+    static __device__ __forceinline__ constexpr int j(int p) { return PS == PS_CROSS ? (p == 0 || p == 4 ? 1 : p == 1 ? 2 : 0) : p; }
+};
+// A blocks (re, im per slice) at descriptor x, B blocks [br | bi] at z
+template <int PS>
+__device__ __forceinline__ void tc_pairs(uint32_t d, uint64_t x, uint64_t z, uint32_t neg, uint32_t accum)
+{
+    const uint32_t xl = (uint32_t)x, xh = (uint32_t)(x >> 32), zl = (uint32_t)z, zh = (uint32_t)(z >> 32);
+    #pragma unroll
+    for (int p = 0; p < PairSet<PS>::n; ++p) {
+        const uint32_t re = xl + PairSet<PS>::i(p) * (2 * A_BLK * 2 >> 4), im = re + (A_BLK * 2 >> 4);
+        const uint32_t ri = zl + PairSet<PS>::j(p) * (B_BLK * 2 >> 4), bi = ri + ((TM / 8) * 128 >> 4);
+        mma_f16_u(d, re, xh, ri, zh, IDESC | neg, p ? 1 : accum);              // Re += ar br, Im += ar bi
+        mma_f16_u(d, im, xh, bi, zh, IDESC_N128 | neg, 1);                     // Re += ai bi
+        mma_f16_u(d + TM, im, xh, ri, zh, (IDESC_N128 | neg) ^ NEG_A, 1);      // Im -= ai br
+    }
+}
+// swapped terms of an off-diagonal tile: A role conj(B_t(y)) from the B-layout
+// block [br | bi] at x, B role A_t(y') from the A-layout blocks at z
+template <int PS>
+__device__ __forceinline__ void tc_swapped(uint32_t d, uint64_t x, uint64_t z, uint32_t neg)
+{
+    const uint32_t xl = (uint32_t)x, xh = (uint32_t)(x >> 32), zl = (uint32_t)z, zh = (uint32_t)(z >> 32);
+    const uint32_t id = IDESC_N128 | neg;
+    #pragma unroll
+    for (int p = 0; p < PairSet<PS>::n; ++p) {
+        const uint32_t br = xl + PairSet<PS>::i(p) * (B_BLK * 2 >> 4), bi = br + ((TM / 8) * 128 >> 4);
+        const uint32_t ar = zl + PairSet<PS>::j(p) * (2 * A_BLK * 2 >> 4), ai = ar + (A_BLK * 2 >> 4);
+        mma_f16_u(d, br, xh, ar, zh, id, 1);                // Re += br ar
+        mma_f16_u(d, bi, xh, ai, zh, id, 1);                // Re += bi ai
+        mma_f16_u(d + TM, br, xh, ai, zh, id, 1);           // Im += br ai
+        mma_f16_u(d + TM, bi, xh, ar, zh, id ^ NEG_A, 1);   // Im -= bi ar
+    }
+}
+
 // ------------------------------------------------ tensor-core kernel
 // One CTA per SM walks the work items blockIdx.x, blockIdx.x + gridDim.x, ...
 // Roles:
 //   warp 0 (one lane): bulk copies of the operand blocks into a ring of NST
 //     shared-memory stages (full[s] completes when a stage's bytes land);
-//   warp 1 (one lane): the MMAs of an item into one of two 256-column TMEM
+//   warp 1 (one lane issues): the MMAs of an item into one of two 256-column TMEM
 //     accumulators, each stage released by a commit to empty[s], the
 //     finished accumulator announced by a commit to acc_full[b];
 //   warps 2-5: the epilogue of an item (TMEM -> registers -> shared memory ->
@@ -508,86 +550,71 @@ k_corr_tc_pipe(const TcArgs a)
             if (b_issued) mbar_wait(&bars->bfull, (uint32_t)((b_issued - 1) & 1));
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            int st = 0, acc = 0;
-            uint32_t ph = 0, aph = 0, bph = 0;
-            bool ok = true;
-            for (long long it = blockIdx.x; it < a.nitems && !*abort && ok; it += gridDim.x) {
-                const Units<MODE> u = item_units<MODE>(a, njt, it);
-                if (MODE == 2) {
-                    if (!mbar_wait_ab(&bars->bfull, bph, abort)) { fail(); break; }
-                    bph ^= 1;
-                }
-                for (int un = 0; un < u.n && ok; ++un) {
-                    const int job = u.job(un);
-                    const bool off = MODE == 1 && u.mt != u.nt;
-                    const TcJob& jd = off ? c_tcoff[job] : job_desc<MODE>(job);
-                    const int nterm = off ? off_terms(jd, job) : jd.nterm;
-                    if (!mbar_wait_ab(&bars->acc_empty[acc], aph ^ 1, abort)) { fail(); ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t d = tmem + (uint32_t)(acc * 256);
-                    uint32_t accum = 0;
-                    for (int pass = 0; pass < 2 && ok; ++pass)
-                        for (int tt = 0; tt < nterm && ok; ++tt) {
-                            const bool sw = tt >= jd.nterm;
-                            const int t = sw ? tt - jd.nterm : tt;
-                            // a term of sign -1: the negate-A bit (13) of the instruction descriptor
-                            const bool ng = (((jd.neg >> t) & 1u) != 0) != (sw && off_flip(job));
-                            const uint32_t neg = ng ? NEG_A : 0u;
-                            const uint32_t id = IDESC | neg, id128 = IDESC_N128 | neg;
-                            for (int g = 0; g < G; ++g) {
-                                if (!mbar_wait_ab(&bars->full[st], ph, abort)) { fail(); ok = false; break; }
-                                tc_fence_after();
-                                const uint8_t* sa = smem + stage_a<MODE>(st);
-                                const uint8_t* sb = MODE == 2 ? smem + jd.fb[t] * SM_B : sa + SM_A;
-                                // slice pairs (i, j) of this stage, or the packed K steps 0, 1 (pass 0)
-                                // and 2 (pass 1: copied to the stage's front; resident B keeps it at 2)
-                                const int npr = pass ? 1 : a.nks ? 2 : 5;
-                                if (sw) {
-                                    // A role: conj(B_t(y)) from the B-layout block [br | bi] (slices of
-                                    // B_BLK); B role: A_t(y') from the A-layout blocks (re, im per slice)
-                                    for (int pr = 0; pr < npr; ++pr) {
-                                        const int i = pass ? 0 : a.nks ? pr : c_pi[pr], j = pass ? 0 : a.nks ? pr : c_pj[pr];
-                                        const uint64_t x_r = sdesc(sa + i * B_BLK * 2, B_LBO, CM_SBO);
-                                        const uint64_t x_i = sdesc(sa + i * B_BLK * 2 + (TM / 8) * 128, B_LBO, CM_SBO);
-                                        const uint64_t y_r = sdesc(sb + (j * 2 + 0) * A_BLK * 2, A_LBO, CM_SBO);
-                                        const uint64_t y_i = sdesc(sb + (j * 2 + 1) * A_BLK * 2, A_LBO, CM_SBO);
-                                        mma_f16(d, x_r, y_r, id128, 1);                 // Re += br ar
-                                        mma_f16(d, x_i, y_i, id128, 1);                 // Re += bi ai
-                                        mma_f16(d + TM, x_r, y_i, id128, 1);            // Im += br ai
-                                        mma_f16(d + TM, x_i, y_r, id128 ^ NEG_A, 1);    // Im -= bi ar
-                                    }
-                                    mma_commit(&bars->empty[st]);
-                                    if (++st == NST) { st = 0; ph ^= 1; }
-                                    continue;
-                                }
-                                for (int pr = 0; pr < npr; ++pr) {
-                                    const int i = pass ? 0 : a.nks ? pr : c_pi[pr];
-                                    const int j = pass ? (MODE == 2 && a.nks ? 2 : 0) : a.nks ? pr : c_pj[pr];
-                                    const uint64_t a_re = sdesc(sa + (i * 2 + 0) * A_BLK * 2, A_LBO, CM_SBO);
-                                    const uint64_t a_im = sdesc(sa + (i * 2 + 1) * A_BLK * 2, A_LBO, CM_SBO);
-                                    const uint64_t b_ri = sdesc(sb + j * B_BLK * 2, B_LBO, CM_SBO);
-                                    const uint64_t b_i = sdesc(sb + j * B_BLK * 2 + (TM / 8) * 128, B_LBO, CM_SBO);
-                                    mma_f16(d, a_re, b_ri, id, accum);              // Re += ar br, Im += ar bi
-                                    accum = 1;
-                                    mma_f16(d, a_im, b_i, id128, 1);                // Re += ai bi
-                                    mma_f16(d + TM, a_im, b_ri, id128 ^ NEG_A, 1);  // Im -= ai br
-                                }
-                                mma_commit(&bars->empty[st]);
-                                if (++st == NST) { st = 0; ph ^= 1; }
-                            }
-                        }
-                    if (!ok) break;
-                    mma_commit(&bars->acc_full[acc]);
-                    if (++acc == 2) { acc = 0; aph ^= 1; }
-                }
-                // the resident B blocks are free once this item's MMAs complete
-                if (MODE == 2 && ok) mma_commit(&bars->bempty);
+        // every lane walks the items (uniform control flow); one issues
+        int st = 0, acc = 0;
+        uint32_t ph = 0, aph = 0, bph = 0;
+        auto wait = [&](uint64_t* b, uint32_t parity) {
+            return __all_sync(0xffffffffu, mbar_wait_ab(b, parity, abort));
+        };
+        bool ok = true;
+        for (long long it = blockIdx.x; it < a.nitems && ok; it += gridDim.x) {
+            const Units<MODE> u = item_units<MODE>(a, njt, it);
+            if (MODE == 2) {
+                if (!wait(&bars->bfull, bph)) { ok = false; break; }
+                bph ^= 1;
             }
-            // every MMA of this thread has completed before TMEM is released
-            mma_commit(&bars->drain);
-            mbar_wait(&bars->drain, 0);
+            for (int un = 0; un < u.n && ok; ++un) {
+                const int job = u.job(un);
+                const bool off = MODE == 1 && u.mt != u.nt;
+                const TcJob& jd = off ? c_tcoff[job] : job_desc<MODE>(job);
+                const int nterm = off ? off_terms(jd, job) : jd.nterm;
+                if (!wait(&bars->acc_empty[acc], aph ^ 1)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)(acc * 256);
+                uint32_t accum = 0;
+                for (int pass = 0; pass < 2 && ok; ++pass)
+                    for (int tt = 0; tt < nterm && ok; ++tt) {
+                        const bool sw = tt >= jd.nterm;
+                        const int t = sw ? tt - jd.nterm : tt;
+                        // a term of sign -1: the negate-A bit (13) of the instruction descriptor
+                        const bool ng = (((jd.neg >> t) & 1u) != 0) != (sw && off_flip(job));
+                        const uint32_t neg = ng ? NEG_A : 0u;
+                        for (int g = 0; g < G; ++g) {
+                            if (!wait(&bars->full[st], ph)) { ok = false; break; }
+                            tc_fence_after();
+                            const uint8_t* sa = smem + stage_a<MODE>(st);
+                            const uint8_t* sb = MODE == 2 ? smem + jd.fb[t] * SM_B : sa + SM_A;
+                            // the slice pairs of this stage, or the packed K steps 0, 1 (pass 0)
+                            // and 2 (pass 1: copied to the stage's front; resident B keeps it at 2)
+                            if (sw) {
+                                const uint64_t x = sdesc(sa, B_LBO, CM_SBO), z = sdesc(sb, A_LBO, CM_SBO);
+                                if (pass) tc_swapped<PS_LAST>(d, x, z, neg);
+                                else if (a.nks) tc_swapped<PS_PACKED>(d, x, z, neg);
+                                else tc_swapped<PS_CROSS>(d, x, z, neg);
+                            } else {
+                                const uint64_t x = sdesc(sa, A_LBO, CM_SBO);
+                                const uint64_t z = sdesc(sb + (MODE == 2 && pass && a.nks ? 2 * B_BLK * 2 : 0), B_LBO, CM_SBO);
+                                if (pass) tc_pairs<PS_LAST>(d, x, z, neg, accum);
+                                else if (a.nks) tc_pairs<PS_PACKED>(d, x, z, neg, accum);
+                                else tc_pairs<PS_CROSS>(d, x, z, neg, accum);
+                                accum = 1;
+                            }
+                            mma_commit_el(&bars->empty[st]);
+                            if (++st == NST) { st = 0; ph ^= 1; }
+                        }
+                    }
+                if (!ok) break;
+                mma_commit_el(&bars->acc_full[acc]);
+                if (++acc == 2) { acc = 0; aph ^= 1; }
+            }
+            // the resident B blocks are free once this item's MMAs complete
+            if (MODE == 2 && ok) mma_commit_el(&bars->bempty);
         }
+        if (!ok && lane == 0) fail();
+        // every MMA has completed before TMEM is released
+        mma_commit_el(&bars->drain);
+        mbar_wait(&bars->drain, 0);
+        __syncwarp();
     } else if (MODE == 0) {
         const int q = warp & 3;                       // TMEM lane quarter of this warp
         zf* xp = (zf*)(smem + SMP_EPI) + (warp - 2) * 32 * 33;
