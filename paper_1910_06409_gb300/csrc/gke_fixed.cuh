@@ -14,9 +14,9 @@
 // 16 times the 2-norm.  An FP64 transform's error is about 2^-52.3 of the 2-norm.
 //
 // Measured (FP64 transforms -> here): 256 x 256 x 65, 16 snapshots: inverse transforms
-// of the terms 56.9 -> 19.8 ms, products stage 46.7 -> 24.4 ms; duct 256 x 33 x 33:
+// of the terms 56.9 -> 19.8 ms, products stage 46.7 -> 21.0 ms; duct 256 x 33 x 33:
 // 30.0 -> 12.9 ms; 128 x 128 x 65, 32 snapshots (from shared-memory stages of FP64):
-// products 28.7 -> 12.3 ms, terms 15.3 -> 5.1 ms.  Errors of the terms against 64-bit references do not grow (duct
+// products 28.7 -> 11.0 ms, terms 15.3 -> 5.1 ms.  Errors of the terms against 64-bit references do not grow (duct
 // A 1.6e-16 -> 1.2e-16).  (Exponents from the largest component and 56 bits were as
 // fast, but raised them by up to a half.)
 #pragma once
@@ -121,20 +121,26 @@ __device__ __forceinline__ double fx_to(long long v, int e)
     rh += rl < up;
     return h == 0 ? 0.0 : __hiloint2double((int)(rh | (sg & 0x80000000u)), (int)rl);
 }
-__device__ __noinline__ static double fx_to_edge(long long v, int e) { return scalbn((double)v, e); }
-__device__ __noinline__ static double fx_scale_edge(double x, int e) { return scalbn(x, e); }
 
+constexpr int FX_NAN = 8192;                              // exponent of a sequence with an infinity or a NaN
+__device__ __forceinline__ bool fx_safe(int E) { return E > -900 && E < 900; }
+// v 2^e of a sequence of any exponent E
+__device__ __noinline__ static double fx_to_edge(long long v, int e, int E)
+{
+    return E == FX_NAN ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)v, e);
+}
+__device__ __noinline__ static double fx_scale_edge(double x, int e) { return scalbn(x, e); }
 // Two-level transform of a sequence in fixed point: fft2l's arguments; E: the
-// sequence's exponent.  Exponents near the ends of the FP64 range take the
-// conversions of the math library.
-template <int N1, int N2, bool INV, bool WARP>
-__device__ __forceinline__ void fft2l_fixed(zd* v, int E, int lane, zx* xs, int s1, int s2, const zx* stw)
+// sequence's exponent.  put(m, w, false) takes output m of this thread, the
+// value w 2^(E - FX_IB + FX_S), |w| < 2^59.5; exponents near the ends of the FP64
+// range take the conversions of the math library and put(m, w, true) as well.
+template <int N1, int N2, bool INV, bool WARP, typename F>
+__device__ __forceinline__ void fft2l_raw(const zd* v, int E, int lane, zx* xs, int s1, int s2, const zx* stw, F put)
 {
     static_assert(N1 % N2 == 0, "N1 must be a multiple of N2");
     constexpr int R = N1 / N2;
-    const bool safe = E > -900 && E < 900;
     zx w[N1];
-    if (safe) {
+    if (fx_safe(E)) {
         const int s = E + 1085 - FX_IB;
         #pragma unroll
         for (int j = 0; j < N1; ++j) w[j] = mk(fx_from(v[j].x, s), fx_from(v[j].y, s));
@@ -154,7 +160,6 @@ __device__ __forceinline__ void fft2l_fixed(zd* v, int E, int lane, zx* xs, int 
     #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1) xs[k1 * s1 + lane * s2] = w[k1];
     sync_lanes<WARP>();
-    const int e = E - FX_IB + FX_S;
     #pragma unroll
     for (int jj = 0; jj < R; ++jj) {
         const int k1 = lane + N2 * jj;
@@ -163,12 +168,21 @@ __device__ __forceinline__ void fft2l_fixed(zd* v, int E, int lane, zx* xs, int 
         for (int n2 = 0; n2 < N2; ++n2) b[n2] = xs[k1 * s1 + n2 * s2];
         dft_reg<long long, N2, INV>(b);
         #pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) v[jj + R * k2] = mk(fx_to(b[k2].x, e), fx_to(b[k2].y, e));
-        if (!safe) {
+        for (int k2 = 0; k2 < N2; ++k2) put(jj + R * k2, b[k2], false);
+        if (!fx_safe(E)) {
             #pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) v[jj + R * k2] = mk(fx_to_edge(b[k2].x, e), fx_to_edge(b[k2].y, e));
+            for (int k2 = 0; k2 < N2; ++k2) put(jj + R * k2, b[k2], true);
         }
     }
+}
+// the same back to FP64, times 2^sh
+template <int N1, int N2, bool INV, bool WARP>
+__device__ __forceinline__ void fft2l_fixed(zd* v, int E, int sh, int lane, zx* xs, int s1, int s2, const zx* stw)
+{
+    const int e = E - FX_IB + FX_S + sh;
+    fft2l_raw<N1, N2, INV, WARP>(v, E, lane, xs, s1, s2, stw, [&](int m, zx w, bool edge) {
+        v[m] = edge ? mk(fx_to_edge(w.x, e, E), fx_to_edge(w.y, e, E)) : mk(fx_to(w.x, e), fx_to(w.y, e));
+    });
 }
 
 // lengths with a register transform
@@ -272,6 +286,7 @@ template <int N1, int N2> __device__ __forceinline__ int fx_rows_exponent(const 
     if (__any_sync(0xffffffffu, fx_far<N1>(s, v))) {
         bias = (fx_reduce<N2>(fx_max<N1>(v), [](int a, int b) { return max(a, b); }) >> 20) - 127;
         s = fx_reduce<N2>(fx_norm<N1>(v, bias), add);
+        if (bias == 0x7ff - 127) return FX_NAN;
     }
     return fx_exponent(s, bias);
 }
@@ -285,14 +300,21 @@ template <typename T, int N1, int N2, bool INV>
 __device__ __forceinline__ void fft2l_rows(cplx<T>* v, int lane, cplx<T>* xs, int s1, int s2, const cplx<T>* stw)
 {
     if constexpr (sizeof(T) == 4) fft2l<T, N1, N2, INV, true>(v, lane, xs, s1, s2, stw);
-    else fft2l_fixed<N1, N2, INV, true>(v, fx_rows_exponent<N1, N2>(v), lane, (zx*)xs, s1, s2, (const zx*)stw);
+    else fft2l_fixed<N1, N2, INV, true>(v, fx_rows_exponent<N1, N2>(v), 0, lane, (zx*)xs, s1, s2, (const zx*)stw);
 }
+// (results times 2^sh)
 template <typename T, int N1, int N2, bool INV>
 __device__ __forceinline__ void fft2l_cols(cplx<T>* v, int seq, int nseq, int lane, cplx<T>* xs, int s1, int s2,
-                                           const cplx<T>* stw, int* smx)
+                                           const cplx<T>* stw, int* smx, int sh = 0)
 {
-    if constexpr (sizeof(T) == 4) fft2l<T, N1, N2, INV>(v, lane, xs, s1, s2, stw);
-    else {
+    if constexpr (sizeof(T) == 4) {
+        fft2l<T, N1, N2, INV>(v, lane, xs, s1, s2, stw);
+        if (sh != 0) {
+            const T c = __int_as_float((127 + sh) << 23);
+            #pragma unroll
+            for (int m = 0; m < N1; ++m) v[m] = c * v[m];
+        }
+    } else {
         const float n = fx_norm<N1>(v, 896);
         auto sum = [&]() {
             float s = 0.f;
@@ -316,7 +338,50 @@ __device__ __forceinline__ void fft2l_cols(cplx<T>* v, int seq, int nseq, int la
             __syncthreads();
             s = sum();
         }
-        fft2l_fixed<N1, N2, INV, false>(v, fx_exponent(s, bias), lane, (zx*)xs, s1, s2, (const zx*)stw);
+        const int E = bias == 0x7ff - 127 ? FX_NAN : fx_exponent(s, bias);
+        fft2l_fixed<N1, N2, INV, false>(v, E, sh, lane, (zx*)xs, s1, s2, (const zx*)stw);
+    }
+}
+// Forward transform of a + i b (a, b real) and its Hermitian split
+// a^(m) = (Z(m) + conj Z(-m)) / (2 N), b^(m) = (Z(m) - conj Z(-m)) / (2 i N),
+// N = N1 N2, handed to put(m, a^, b^), m = 0 .. N / 2, by the N2 lanes of the
+// sequence; xr: their shared buffer.  FP64: the sums are integers' and 1 / (2 N)
+// is in the exponent (in FP64 they took half of the row kernels' FP64 operations:
+// products stage of 256 x 256 x 65, 16 snapshots, 23.0 -> 21.0 ms).
+template <typename T, int N1, int N2, typename F>
+__device__ __forceinline__ void fft2l_split(cplx<T>* f, int lane, cplx<T>* xr, const cplx<T>* stw, F put)
+{
+    constexpr int N = N1 * N2;
+    if constexpr (sizeof(T) == 4) {
+        fft2l<T, N1, N2, false, true>(f, lane, xr, N2 + 1, 1, stw);
+        __syncwarp();
+        #pragma unroll
+        for (int m = 0; m < N1; ++m) xr[lane + N2 * m] = f[m];
+        __syncwarp();
+        const T h = (T)0.5 / (T)N;
+        for (int k = lane; k <= N / 2; k += N2) {
+            const cplx<T> Z = xr[k], Zc = conj(xr[(N - k) & (N - 1)]);
+            const cplx<T> D = Z - Zc;
+            put(k, h * (Z + Zc), mk(h * D.y, -h * D.x));
+        }
+    } else {
+        const int E = fx_rows_exponent<N1, N2>(f);
+        zx* x = (zx*)xr;
+        zx w[N1];
+        fft2l_raw<N1, N2, false, true>(f, E, lane, x, N2 + 1, 1, (const zx*)stw, [&](int m, zx a, bool) { w[m] = a; });
+        __syncwarp();
+        #pragma unroll
+        for (int m = 0; m < N1; ++m) x[lane + N2 * m] = w[m];
+        __syncwarp();
+        constexpr int lg = N == 32 ? 5 : N == 64 ? 6 : N == 128 ? 7 : N == 256 ? 8 : 9;
+        static_assert(N == 1 << lg, "lengths with a register transform");
+        const int e = E - FX_IB + FX_S - lg - 1;
+        for (int k = lane; k <= N / 2; k += N2) {
+            const zx Z = x[k], Y = x[(N - k) & (N - 1)];
+            const long long ax = Z.x + Y.x, ay = Z.y - Y.y, bx = Z.y + Y.y, by = Y.x - Z.x;
+            if (fx_safe(E)) put(k, mk(fx_to(ax, e), fx_to(ay, e)), mk(fx_to(bx, e), fx_to(by, e)));
+            else put(k, mk(fx_to_edge(ax, e, E), fx_to_edge(ay, e, E)), mk(fx_to_edge(bx, e, E), fx_to_edge(by, e, E)));
+        }
     }
 }
 // ints of the smx array (none for FP32)

@@ -178,14 +178,16 @@ k_col_forward_r(const cplx<TF>* __restrict__ H, int ny, int nxh, int CW, int YB,
     #pragma unroll
     for (int m = 0; m < N1; ++m) v[m] = live ? src[(long long)(lane + N2 * m) * nxh + kx] : mk((TF)0, (TF)0);
     __syncthreads();
-    fft2l_cols<TF, N1, N2, false>(v, yl * CW + c, nseq, lane, xs + (yl * CW + c), N2 * nseq + 1, nseq, stw, smx);
+    // scale 1 / N; the pair products (uu .. vw) carry the factor 2 of the expansion
+    constexpr int lg = N == 32 ? 5 : N == 64 ? 6 : N == 128 ? 7 : 8;
+    static_assert(N == 1 << lg, "register lengths");
+    fft2l_cols<TF, N1, N2, false>(v, yl * CW + c, nseq, lane, xs + (yl * CW + c), N2 * nseq + 1, nseq, stw, smx,
+                                  (j < 6) - lg);
     if (live) {
-        // the pair products (uu .. vw) carry the factor 2 of the expansion
-        const TF inz = (j < 6 ? (TF)2 : (TF)1) / (TF)N;
         #pragma unroll
         for (int m = 0; m < N1; ++m) {
             const long long k = (long long)(lane + N2 * m) * nxh + kx;
-            Xop[((((long long)(F_UU + j)) * Nk + k) * ns + s) * ny + y] = inz * v[m];
+            Xop[((((long long)(F_UU + j)) * Nk + k) * ns + s) * ny + y] = v[m];
         }
     }
 }
@@ -335,7 +337,6 @@ k_row_products_r(const cplx<TF>* __restrict__ G, int ny, int nz, const cplx<TF>*
             ph[2 * N + N2 * m] = w;
         }
     }
-    const TF h = (TF)0.5 / (TF)N;
     #pragma unroll 1
     for (int j = 0; j < 4; ++j) {
         C f[N1];
@@ -346,20 +347,14 @@ k_row_products_r(const cplx<TF>* __restrict__ G, int ny, int nz, const cplx<TF>*
                           : mk(u * u + vv * vv + w * w, (TF)0);
         }
         __syncwarp();
-        fft2l_rows<TF, N1, N2, false>(f, lane, xr, N2 + 1, 1, stw);
-        __syncwarp();
-        #pragma unroll
-        for (int m = 0; m < N1; ++m) xr[lane + N2 * m] = f[m];
-        __syncwarp();
-        if (live)
-            for (int k = lane; k < nxh; k += N2) {
-                const C Z = xr[k], Zc = conj(xr[(N - k) & (N - 1)]);
-                const C A = h * (Z + Zc);
-                const C D = Z - Zc;
-                const C B = mk(h * D.y, -h * D.x);     // -i/2 (Z - Zc)
-                H[(((long long)(2 * j) * ny + y) * nz + z) * nxh + k] = A;
-                if (j < 3) H[(((long long)(2 * j + 1) * ny + y) * nz + z) * nxh + k] = B;
+        C* ha = H + (((long long)(2 * j) * ny + y) * nz + zz) * nxh;
+        C* hb = ha + (long long)ny * nz * nxh;
+        fft2l_split<TF, N1, N2>(f, lane, xr, stw, [&](int k, C A, C B) {
+            if (live) {
+                ha[k] = A;
+                if (j < 3) hb[k] = B;
             }
+        });
     }
     // block reduction of the row sums (FP64 across threads)
     __shared__ double red[6][32];
