@@ -927,22 +927,31 @@ __global__ void k_stencil_res(double* __restrict__ terms, long long npair, const
     const long long N = (long long)sm.nrz * sm.nrx;
     const long long p = blockIdx.x;
     const long long e = (long long)blockIdx.y * blockDim.x + threadIdx.x;
+    const int i1 = pair_i[2 * p], i2 = pair_i[2 * p + 1];
+    // (y2 - y1) / 2 + h1 + h2 as one sum, the halves in the weights: bound by the
+    // FP64 pipe (21 operations instead of 25; both stencils of 256 x 256 x 65
+    // 10.0 -> 9.7 ms)
+    __shared__ double sw[4][5];                      // -w1 / 2, w2 / 2, w1, w2
+    if (threadIdx.x < 5) {
+        const double w1 = fdw[5 * i1 + threadIdx.x], w2 = fdw[5 * i2 + threadIdx.x];
+        sw[0][threadIdx.x] = -0.5 * w1; sw[1][threadIdx.x] = 0.5 * w2;
+        sw[2][threadIdx.x] = w1; sw[3][threadIdx.x] = w2;
+    }
+    __syncthreads();
     if (e >= N) return;
     const int mz = (int)(e / sm.nrx), mx = (int)(e - (long long)mz * sm.nrx);
-    const int i1 = pair_i[2 * p], i2 = pair_i[2 * p + 1];
     const double* Py = terms + (long long)T_PHIY * npair * N;
     const double* Ph = terms + (long long)T_PHI * npair * N;
-    double y1 = 0.0, y2 = 0.0, h1 = 0.0, h2 = 0.0;
     const int a1 = fdl0[i1], a2 = fdl0[i2];
+    double d = 0.0;
     #pragma unroll
     for (int l = 0; l < 5; ++l) {
-        double w1 = fdw[5 * i1 + l], w2 = fdw[5 * i2 + l];
-        y1 += w1 * tri_value<WEDGE, US>(Py, a1 + l, i2, ny, sm, mz, mx, -1, 1);
-        y2 += w2 * tri_value<WEDGE, US>(Py, i1, a2 + l, ny, sm, mz, mx, -1, 1);
-        h1 += w1 * tri_value<WEDGE, US>(Ph, a1 + l, i2, ny, sm, mz, mx, 1, -1);
-        h2 += w2 * tri_value<WEDGE, US>(Ph, i1, a2 + l, ny, sm, mz, mx, 1, -1);
+        d += sw[0][l] * tri_value<WEDGE, US>(Py, a1 + l, i2, ny, sm, mz, mx, -1, 1);
+        d += sw[1][l] * tri_value<WEDGE, US>(Py, i1, a2 + l, ny, sm, mz, mx, -1, 1);
+        d += sw[2][l] * tri_value<WEDGE, US>(Ph, a1 + l, i2, ny, sm, mz, mx, 1, -1);
+        d += sw[3][l] * tri_value<WEDGE, US>(Ph, i1, a2 + l, ny, sm, mz, mx, 1, -1);
     }
-    terms[((long long)T_RES * npair + p) * N + e] += 0.5 * (y2 - y1) + (h1 + h2);
+    terms[((long long)T_RES * npair + p) * N + e] += d;
 }
 
 // ------------------------------------- split path: FP32 stencils
