@@ -40,7 +40,7 @@
 #include <cmath>
 #include <initializer_list>
 #include <string>
-#include <tuple>
+#include <utility>
 #include <vector>
 
 #include "../../include/gke1h.h"
@@ -77,63 +77,44 @@ __host__ __device__ inline int prod_field(int i, int k)
     return a == 0 ? (b == 0 ? G_UU : b == 1 ? G_UV : G_UW) : a == 1 ? (b == 1 ? G_VV : G_VW) : G_WW;
 }
 
-// A contraction: sum over its terms t of w_t conj(X[fa_t](p1)) X[fb_t](p2),
-// summed over snapshots; added to the accumulators with the constant
-// coefficients c[A .. psi_z]; ra >= 0 marks <u_ra(p1) u_rb(p2)'>, whose
-// coefficient in xi depends on the pair (k1_correlate).
-struct Job { int nt; int fa[8]; int fb[8]; double w[8]; double c[6]; int ra, rb; };
-constexpr int NJ = 20;
+// A contraction: sum over its terms t of conj(X[fa_t](p1)) X[fb_t](p2), summed
+// over snapshots; added to the accumulators with the constant coefficients
+// c[A .. psi_z]; ra >= 0 marks <u_ra(p1) u_rb(p2)'>, whose coefficient in xi
+// depends on the pair (add_job).
+struct Job { int nt; int fa[3]; int fb[3]; double c[6]; int ra, rb; };
+constexpr int NJ = 23;
 __constant__ Job c_job[NJ];
 
 static void make_jobs(std::vector<Job>& js)
 {
     js.clear();
-    auto job = [](std::initializer_list<std::tuple<int, int, double>> terms, std::initializer_list<double> c,
-                  int ra = -1, int rb = -1) {
+    auto job = [&](std::initializer_list<std::pair<int, int>> terms, std::initializer_list<std::pair<int, double>> c,
+                   int ra = -1, int rb = -1) {
         Job j{};
-        j.nt = 0;
-        for (auto& t : terms) {
-            j.fa[j.nt] = std::get<0>(t); j.fb[j.nt] = std::get<1>(t); j.w[j.nt] = std::get<2>(t); ++j.nt;
-        }
-        int i = 0;
-        for (double v : c) j.c[i++] = v;
+        for (auto& t : terms) { j.fa[j.nt] = t.first; j.fb[j.nt] = t.second; ++j.nt; }
+        for (auto& v : c) j.c[v.first] = v.second;
         j.ra = ra; j.rb = rb;
-        return j;
+        js.push_back(j);
     };
     // <u_a(p1) u_b(p2)'>: -2 into A when a = b; xi through the mean gradients
     for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) js.push_back(job({{a, b, 1.0}}, {a == b ? -2.0 : 0.0, 0, 0, 0, 0, 0}, a, b));
+        for (int b = 0; b < 3; ++b) job({{a, b}}, {{A_A, a == b ? -2.0 : 0.0}}, a, b);
     // Phi_x: <du^2 du> = G1 - G2, G1 = <q u'> + 2 <(u_i u) u_i'>, G2 = <u q'> + 2 <u_i (u_i u)'>
-    js.push_back(job({{G_Q, G_U, 1.0}, {G_UU, G_U, 2.0}, {G_UV, G_V, 2.0}, {G_UW, G_W, 2.0},
-                      {G_U, G_Q, -1.0}, {G_U, G_UU, -2.0}, {G_V, G_UV, -2.0}, {G_W, G_UW, -2.0}},
-                     {0, 1.0, 0, 0, 0, 0}));
+    job({{G_Q, G_U}}, {{A_PHIX, 1.0}});
+    job({{G_UU, G_U}, {G_UV, G_V}, {G_UW, G_W}}, {{A_PHIX, 2.0}});
+    job({{G_U, G_Q}}, {{A_PHIX, -1.0}});
+    job({{G_U, G_UU}, {G_V, G_UV}, {G_W, G_UW}}, {{A_PHIX, -2.0}});
     for (int k = 1; k <= 2; ++k) {
-        const int phi = k == 1 ? 2 : 3, psi = k == 1 ? 4 : 5;
-        auto cc = [&](double cphi, double cpsi) {
-            std::vector<double> c(6, 0.0);
-            c[phi] = cphi; c[psi] = cpsi;
-            return c;
-        };
-        auto jobv = [&](std::vector<std::tuple<int, int, double>> terms, std::vector<double> c) {
-            Job j{};
-            j.nt = (int)terms.size();
-            for (int t = 0; t < j.nt; ++t) {
-                j.fa[t] = std::get<0>(terms[t]); j.fb[t] = std::get<1>(terms[t]); j.w[t] = std::get<2>(terms[t]);
-            }
-            for (int i = 0; i < 6; ++i) j.c[i] = c[i];
-            j.ra = j.rb = -1;
-            return j;
-        };
+        const int phi = k == 1 ? A_PHIY : A_PHIZ, psi = k == 1 ? A_PSIY : A_PSIZ;
+        const int u = prod_field(0, k), v = prod_field(1, k), w = prod_field(2, k);
         // Q1 = <q u_k'>, Q2 = <u_k q'>, X1 = sum_i <(u_i u_k) u_i'>, X2 = sum_i <u_i (u_i u_k)'>:
         // <du^2 du_k> = Q1 + 2 X1 - Q2 - 2 X2, <u_k* du^2> = (Q1 + Q2)/2 - X1 - X2
-        js.push_back(jobv({{G_Q, k, 1.0}}, cc(1.0, 0.5)));
-        js.push_back(jobv({{k, G_Q, 1.0}}, cc(-1.0, 0.5)));
-        js.push_back(jobv({{prod_field(0, k), 0, 1.0}, {prod_field(1, k), 1, 1.0}, {prod_field(2, k), 2, 1.0}},
-                          cc(2.0, -1.0)));
-        js.push_back(jobv({{0, prod_field(0, k), 1.0}, {1, prod_field(1, k), 1.0}, {2, prod_field(2, k), 1.0}},
-                          cc(-2.0, -1.0)));
+        job({{G_Q, k}}, {{phi, 1.0}, {psi, 0.5}});
+        job({{k, G_Q}}, {{phi, -1.0}, {psi, 0.5}});
+        job({{u, 0}, {v, 1}, {w, 2}}, {{phi, 2.0}, {psi, -1.0}});
+        job({{0, u}, {1, v}, {2, w}}, {{phi, -2.0}, {psi, -1.0}});
         // <dp du_k> = <p u_k>(p1) + <p u_k>(p2) - <p u_k'> - <u_k p'>
-        js.push_back(jobv({{G_P, k, 1.0}, {k, G_P, 1.0}}, cc(0.0, -2.0)));
+        job({{G_P, k}, {k, G_P}}, {{psi, -2.0}});
     }
 }
 
@@ -420,19 +401,51 @@ __device__ __forceinline__ void finish_pair(const cplx<TF>* T, int q1, int q2, i
     spec[((long long)NACC * nxh + m) * npair + pr] = res;
 }
 
+// add_job for an RB x RB block of pairs (one coefficient test per job)
+template <typename TF, int RB>
+__device__ __forceinline__ void fold_job(cplx<TF> (&T)[NACC][RB][RB], const Job& jb, const cplx<TF> (&acc)[RB][RB],
+                                         const int (&p1)[RB], const int (&p2)[RB], int P, const TF* __restrict__ prof)
+{
+    #pragma unroll
+    for (int t = 0; t < 6; ++t) {
+        const TF c = (TF)jb.c[t];
+        if (c == (TF)0) continue;
+        #pragma unroll
+        for (int a = 0; a < RB; ++a)
+            #pragma unroll
+            for (int b = 0; b < RB; ++b) {
+                T[t][a][b].x = fma(c, acc[a][b].x, T[t][a][b].x);
+                T[t][a][b].y = fma(c, acc[a][b].y, T[t][a][b].y);
+            }
+    }
+    if (jb.ra >= 0) {
+        const int ra = jb.ra, rb = jb.rb;
+        #pragma unroll
+        for (int a = 0; a < RB; ++a)
+            #pragma unroll
+            for (int b = 0; b < RB; ++b) {
+                TF c = (TF)0;
+                if (rb >= 1 && p2[b] < P) c += (TF)2 * prof[(long long)(R_G + 2 * ra + rb - 1) * P + p2[b]];
+                if (ra >= 1 && p1[a] < P) c += (TF)2 * prof[(long long)(R_G + 2 * rb + ra - 1) * P + p1[a]];
+                T[A_XI][a][b].x = fma(c, acc[a][b].x, T[A_XI][a][b].x);
+                T[A_XI][a][b].y = fma(c, acc[a][b].y, T[A_XI][a][b].y);
+            }
+    }
+}
+
 // CTA = (tile pair T1 <= T2 of the nt full tiles, wavenumber m); 16 x 16
 // threads, each an RB x RB block of pairs (p1 = T1 CT + ty + 16 a,
 // p2 = T2 CT + tx + 16 b).  With strips, the points past the last full tile
 // are left to k1_correlate_strip; otherwise the last tile is padded.
-template <typename TF>
-__global__ void __launch_bounds__(256, sizeof(TF) == 4 ? 2 : 1)
-k1_correlate(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int nt, double kx0, double nu,
-             const TF* __restrict__ prof, const double* __restrict__ op, cplx<TF>* __restrict__ spec,
+__global__ void __launch_bounds__(256, 1)
+k1_correlate(const zd* __restrict__ X, int ns, int P, int nx, int nt, double kx0, double nu,
+             const double* __restrict__ prof, const double* __restrict__ op, zd* __restrict__ spec,
              long long npair)
 {
-    typedef cplx<TF> C;
+    typedef double TF;
+    typedef zd C;
     constexpr int RB = 2;
-    constexpr int SC = sizeof(TF) == 4 ? 2 * SCH : SCH;     // snapshots per staged chunk
+    constexpr int SC = SCH;                                 // snapshots per staged chunk
     __shared__ C As[SC][CT];
     __shared__ C Bs[SC][CT];
     const int nxh = nx / 2 + 1;
@@ -458,9 +471,6 @@ k1_correlate(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int nt, doub
             #pragma unroll
             for (int b = 0; b < RB; ++b) acc[a][b] = mk((TF)0, (TF)0);
         for (int t = 0; t < jb.nt; ++t) {
-            // the term's weight (real) scales its A operand as it is staged:
-            // conj(w a) b = w conj(a) b, so the sum goes straight into acc
-            const TF wt = (TF)jb.w[t];
             const C* A = X + ((long long)jb.fa[t] * nxh + m) * ns * P;
             const C* B = X + ((long long)jb.fb[t] * nxh + m) * ns * P;
             for (int s0 = 0; s0 < ns; s0 += SC) {
@@ -468,7 +478,7 @@ k1_correlate(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int nt, doub
                 for (int e = threadIdx.x; e < SC * CT; e += blockDim.x) {
                     const int ss = e / CT, yy = e - ss * CT, s = s0 + ss;
                     C va = mk((TF)0, (TF)0), vb = va;
-                    if (s < ns && T1 * CT + yy < P) { va = A[(long long)s * P + T1 * CT + yy]; va.x *= wt; va.y *= wt; }
+                    if (s < ns && T1 * CT + yy < P) va = A[(long long)s * P + T1 * CT + yy];
                     if (s < ns && T2 * CT + yy < P) vb = B[(long long)s * P + T2 * CT + yy];
                     As[ss][yy] = va;
                     Bs[ss][yy] = vb;
@@ -486,32 +496,7 @@ k1_correlate(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int nt, doub
                 }
             }
         }
-        // the contraction into the term spectra (as add_job, one coefficient test per job)
-        #pragma unroll
-        for (int t = 0; t < 6; ++t) {
-            const TF c = (TF)jb.c[t];
-            if (c == (TF)0) continue;
-            #pragma unroll
-            for (int a = 0; a < RB; ++a)
-                #pragma unroll
-                for (int b = 0; b < RB; ++b) {
-                    T[t][a][b].x = fma(c, acc[a][b].x, T[t][a][b].x);
-                    T[t][a][b].y = fma(c, acc[a][b].y, T[t][a][b].y);
-                }
-        }
-        if (jb.ra >= 0) {
-            const int ra = jb.ra, rb = jb.rb;
-            #pragma unroll
-            for (int a = 0; a < RB; ++a)
-                #pragma unroll
-                for (int b = 0; b < RB; ++b) {
-                    TF c = (TF)0;
-                    if (rb >= 1 && p2[b] < P) c += (TF)2 * prof[(long long)(R_G + 2 * ra + rb - 1) * P + p2[b]];
-                    if (ra >= 1 && p1[a] < P) c += (TF)2 * prof[(long long)(R_G + 2 * rb + ra - 1) * P + p1[a]];
-                    T[A_XI][a][b].x = fma(c, acc[a][b].x, T[A_XI][a][b].x);
-                    T[A_XI][a][b].y = fma(c, acc[a][b].y, T[A_XI][a][b].y);
-                }
-        }
+        fold_job<TF, RB>(T, jb, acc, p1, p2, P, prof);
     }
     #pragma unroll
     for (int a = 0; a < RB; ++a)
@@ -522,6 +507,91 @@ k1_correlate(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int nt, doub
             #pragma unroll
             for (int t = 0; t < NACC; ++t) v[t] = T[t][a][b];
             finish_pair<TF>(v, p1[a], p2[b], m, nx, kx0, nu, ns, P, prof, op, spec, npair);
+        }
+}
+
+// FP32 plans: k1_correlate's tiles with the operands of both tiles, every field
+// and up to SG32 snapshots, staged at once (cp.async): 37 terms read 22
+// staged field tiles, and no barrier stands between them.  (Staging the two
+// operands of each term took 74 tile loads behind 37 pairs of barriers: correlate
+// stage of 256 x 33 x 33, 16 snapshots 17.9 -> 12.7 ms; with 4 x 2 pairs on 128 threads
+// 13.4, too few warps.)  More snapshots are added group by group.
+constexpr int SG32 = 16;
+static size_t corr32_smem(int ns)
+{
+    return (size_t)2 * NFLD * ((std::min(ns, SG32) + 3) / 4 * 4) * CT * sizeof(zf);
+}
+__global__ void __launch_bounds__(256, 2)
+k1_correlate32(const zf* __restrict__ X, int ns, int P, int nx, int nt, double kx0, double nu,
+               const float* __restrict__ prof, const double* __restrict__ op, zf* __restrict__ spec, long long npair)
+{
+    constexpr int RB = 2;
+    extern __shared__ __align__(16) unsigned char sh_c32[];
+    zf* fld = (zf*)sh_c32;                              // [tile][field][snapshot][CT]
+    const int nxh = nx / 2 + 1;
+    const int m = blockIdx.y;
+    int T1 = 0, rem = blockIdx.x;
+    while (rem >= nt - T1) { rem -= nt - T1; ++T1; }
+    const int T2 = T1 + rem;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    int p1[RB], p2[RB];
+    for (int a = 0; a < RB; ++a) { p1[a] = T1 * CT + ty + 16 * a; p2[a] = T2 * CT + tx + 16 * a; }
+    zf T[NACC][RB][RB];
+    #pragma unroll
+    for (int t = 0; t < NACC; ++t)
+        #pragma unroll
+        for (int a = 0; a < RB; ++a)
+            #pragma unroll
+            for (int b = 0; b < RB; ++b) T[t][a][b] = mk(0.f, 0.f);
+    const int SS = (min(ns, SG32) + 3) / 4 * 4;         // staged snapshots, zeros past ns
+    const int yy = threadIdx.x % CT;
+    for (int s0 = 0; s0 < ns; s0 += SG32) {
+        if (s0) __syncthreads();
+        // a warp copies one row of CT points; rows (tile, field, snapshot)
+        for (int r = threadIdx.x / CT; r < 2 * NFLD * SS; r += 256 / CT) {
+            const int ss = r % SS, f = (r / SS) % NFLD, y = (r >= NFLD * SS ? T2 : T1) * CT + yy;
+            const bool in = s0 + ss < ns && y < P;
+            const zf* src = in ? X + (((long long)f * nxh + m) * ns + s0 + ss) * P + y : X;
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(fld + r * CT + yy);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(in ? 8 : 0) : "memory");
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        for (int j = 0; j < NJ; ++j) {
+            const Job& jb = c_job[j];
+            zf acc[RB][RB];
+            #pragma unroll
+            for (int a = 0; a < RB; ++a)
+                #pragma unroll
+                for (int b = 0; b < RB; ++b) acc[a][b] = mk(0.f, 0.f);
+            for (int t = 0; t < jb.nt; ++t) {
+                const zf* A = fld + jb.fa[t] * SS * CT + ty;
+                const zf* B = fld + (NFLD + jb.fb[t]) * SS * CT + tx;
+                for (int ss = 0; ss < SS; ss += 4, A += 4 * CT, B += 4 * CT) {
+                    #pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        zf av[RB], bv[RB];
+                        #pragma unroll
+                        for (int i = 0; i < RB; ++i) { av[i] = A[q * CT + 16 * i]; bv[i] = B[q * CT + 16 * i]; }
+                        #pragma unroll
+                        for (int a = 0; a < RB; ++a)
+                            #pragma unroll
+                            for (int b = 0; b < RB; ++b) cmac(acc[a][b], av[a], bv[b]);
+                    }
+                }
+            }
+            fold_job<float, RB>(T, jb, acc, p1, p2, P, prof);
+        }
+    }
+    #pragma unroll
+    for (int a = 0; a < RB; ++a)
+        #pragma unroll
+        for (int b = 0; b < RB; ++b) {
+            if (p1[a] >= P || p2[b] >= P || p2[b] < p1[a]) continue;
+            zf v[NACC];
+            #pragma unroll
+            for (int t = 0; t < NACC; ++t) v[t] = T[t][a][b];
+            finish_pair<float>(v, p1[a], p2[b], m, nx, kx0, nu, ns, P, prof, op, spec, npair);
         }
 }
 
@@ -555,10 +625,7 @@ k1_correlate_strip(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int co
         for (int t = 0; t < jb.nt; ++t) {
             const C* A = X + ((long long)jb.fa[t] * nxh + m) * ns * P;
             const C* B = X + ((long long)jb.fb[t] * nxh + m) * ns * P;
-            C part = mk((TF)0, (TF)0);
-            for (int s = 0; s < ns; ++s) cmac(part, A[(long long)s * P + q1], B[(long long)s * P + q2]);
-            acc.x = fma((TF)jb.w[t], part.x, acc.x);
-            acc.y = fma((TF)jb.w[t], part.y, acc.y);
+            for (int s = 0; s < ns; ++s) cmac(acc, A[(long long)s * P + q1], B[(long long)s * P + q2]);
         }
         add_job(T, jb, acc, q1, q2, P, prof);
     }
@@ -1151,6 +1218,8 @@ static cudaError_t set_attrs(gke1h_plan_t p)
 {
     typedef cplx<TF> C;
     cudaError_t e = cudaFuncSetAttribute(k1_products<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem_prod);
+    if (e == cudaSuccess && sizeof(TF) == 4)
+        e = cudaFuncSetAttribute(k1_correlate32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)corr32_smem(SG32));
     if (e != cudaSuccess) return e;
     if (p->nx == 128 || p->nx == 256 || p->nx == 512) {
         const void* fn = p->nx == 128 ? (const void*)k1_transform_r<TF, 16, 8>
@@ -1329,7 +1398,11 @@ static void launch_pass(gke1h_plan_t p, const zd* f, int ns, TF* T)
         const int nt = strips ? nfull : p->nt;
         const long long ntp = (long long)nt * (nt + 1) / 2;
         if (!digits) {
-            k1_correlate<TF><<<dim3((unsigned)ntp, nxh), 256, 0, p->st>>>(X, ns, P, nx, nt, kx0, p->nu, pt, p->op,
+            if constexpr (sizeof(TF) == 4)
+                k1_correlate32<<<dim3((unsigned)ntp, nxh), 256, corr32_smem(ns), p->st>>>(X, ns, P, nx, nt, kx0, p->nu,
+                                                                                          pt, p->op, spec, p->npair);
+            else
+                k1_correlate<<<dim3((unsigned)ntp, nxh), 256, 0, p->st>>>(X, ns, P, nx, nt, kx0, p->nu, pt, p->op,
                                                                           spec, p->npair);
             p->launches += 1;
         }
