@@ -291,6 +291,7 @@ static cudaError_t set_smem_attrs()
     cudaError_t e = products_set_attrs(lim);
     if (e == cudaSuccess) e = terms_set_attrs(lim);
     if (e == cudaSuccess) e = combine_set_attrs();
+    if (e == cudaSuccess) e = correlate_set_attrs();
     return e;
 }
 

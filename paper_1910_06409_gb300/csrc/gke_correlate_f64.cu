@@ -20,6 +20,8 @@
 // Chebyshev grids ny = 32 m + 1 leave one wall row), that remainder is done
 // as row and column strips, one (y, y') per thread, instead of as mostly empty
 // padded tiles (which cost half as much again as the useful work at ny = 129).
+#include <type_traits>
+
 #include "gke_common.cuh"
 #include "gke_kernels.h"
 
@@ -150,6 +152,88 @@ k_correlate(const cplx<T>* __restrict__ Xop, int ns, int ny, int Nk, int k0, int
     }
 }
 
+// FP32, one tile of 16 RB >= ny points and at most TILE_NS snapshots: every
+// field of a wavenumber staged once (cp.async) for all its contractions, so a CTA
+// waits for memory once and not per term, and the tile fits ny.  Small passes are
+// bound by those waits: correlate stage of 96 x 48 x 41, 6 snapshots 217 us,
+// 628 with k_correlate<float, 4>'s tiles of 64 staged term by term.
+constexpr int TILE_NS = 16;
+static int tile_rb(int ny) { return (ny + 15) / 16; }
+static size_t tile_smem(int rb, int ns) { return (size_t)NFIELD * ((ns + 1) / 2 * 2) * 16 * rb * sizeof(zf); }
+template <int RB>
+__global__ void __launch_bounds__(256)
+k_correlate_tile(const zf* __restrict__ Xop, int ns, int ny, int Nk, int k0, int Kc, JobList jl, zf* __restrict__ raw)
+{
+    constexpr int CT = 16 * RB;
+    extern __shared__ __align__(16) unsigned char sh_ct[];
+    zf* fld = (zf*)sh_ct;                            // [field][snapshot][CT], zeros past ns and ny
+    const int kl = blockIdx.x, SS = (ns + 1) / 2 * 2;
+    const zf* X = Xop + (long long)(k0 + kl) * ns * ny;
+    for (int f = 0; f < NFIELD; ++f)
+        for (int e = threadIdx.x; e < SS * CT; e += 256) {
+            const int ss = e / CT, y = e - ss * CT;
+            const bool in = ss < ns && y < ny;
+            const zf* src = in ? X + (long long)f * Nk * ns * ny + ss * ny + y : Xop;
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(fld + f * SS * CT + e);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(in ? 8 : 0) : "memory");
+        }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, yb = (ny + 7) / 8;
+    for (int jj = 0; jj < jl.n; ++jj) {
+        const int job = jl.j[jj];
+        const JobDesc& jd = c_jobs[job];
+        zf acc[RB][RB];
+        #pragma unroll
+        for (int a = 0; a < RB; ++a)
+            #pragma unroll
+            for (int b = 0; b < RB; ++b) acc[a][b] = mk(0.f, 0.f);
+        for (int t = 0; t < jd.nterm; ++t) {
+            const zf* A = fld + jd.fa[t] * SS * CT + ty;
+            const zf* B = fld + jd.fb[t] * SS * CT + tx;
+            for (int ss = 0; ss < SS; ss += 2, A += 2 * CT, B += 2 * CT) {
+                #pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    zf a[RB], b[RB];
+                    #pragma unroll
+                    for (int i = 0; i < RB; ++i) { a[i] = A[q * CT + 16 * i]; b[i] = B[q * CT + 16 * i]; }
+                    #pragma unroll
+                    for (int i = 0; i < RB; ++i)
+                        #pragma unroll
+                        for (int j = 0; j < RB; ++j) cmac_conj(acc[i][j], a[i], b[j]);
+                }
+            }
+        }
+        #pragma unroll
+        for (int a = 0; a < RB; ++a)
+            #pragma unroll
+            for (int b = 0; b < RB; ++b) {
+                const int y = ty + 16 * a, yp = tx + 16 * b;
+                if (y >= ny || yp >= ny || (job == NJSQ && yp < y)) continue;
+                raw[raw_index(job, kl, y, yp, Kc, yb)] = acc[a][b];
+            }
+    }
+}
+
+template <typename F> static void with_tile(int rb, F f)
+{
+    if (rb == 1) f(std::integral_constant<int, 1>());
+    else if (rb == 2) f(std::integral_constant<int, 2>());
+    else if (rb == 3) f(std::integral_constant<int, 3>());
+    else f(std::integral_constant<int, 4>());
+}
+cudaError_t correlate_set_attrs()
+{
+    cudaError_t e = cudaSuccess;
+    for (int rb = 1; rb <= 4; ++rb)
+        with_tile(rb, [&](auto R) {
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k_correlate_tile<decltype(R)::value>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)tile_smem(decltype(R)::value, TILE_NS));
+        });
+    return e;
+}
+
 // wavenumbers [k0, k0 + Kc) of Nk; raw holds the chunk (raw_index with Kc)
 void correlate_launch(bool fp32, const void* Xop, int ns, int ny, int Nk, int k0, int Kc, void* raw, unsigned jobs,
                       cudaStream_t st)
@@ -158,7 +242,12 @@ void correlate_launch(bool fp32, const void* Xop, int ns, int ny, int Nk, int k0
     for (int j = 0; j < NJOB; ++j)
         if ((jobs >> j) & 1u) jl.j[jl.n++] = j;
     if (jl.n == 0) return;
-    if (fp32)
+    if (fp32 && ny <= 64 && ns <= TILE_NS)
+        with_tile(tile_rb(ny), [&](auto R) {
+            k_correlate_tile<decltype(R)::value><<<Kc, 256, tile_smem(decltype(R)::value, ns), st>>>(
+                (const zf*)Xop, ns, ny, Nk, k0, Kc, jl, (zf*)raw);
+        });
+    else if (fp32)
         k_correlate<float, 4><<<dim3(Kc, jl.n), 256, 0, st>>>((const zf*)Xop, ns, ny, Nk, k0, Kc, jl, (zf*)raw);
     else
         k_correlate<double, 2><<<dim3(Kc, jl.n), 256, 0, st>>>((const zd*)Xop, ns, ny, Nk, k0, Kc, jl, (zd*)raw);

@@ -118,6 +118,7 @@ bool combine_kc_ok(bool fp32, int kc);
 
 __global__ void k_mean_accum(const zd* fields, int ns, int ny, long long plane, double* mean_sum);
 __global__ void k_reduce_partials(const double* part, int nvals, int nb, double* out);
+cudaError_t correlate_set_attrs();
 void correlate_launch(bool fp32, const void* Xop, int ns, int ny, int Nk, int k0, int Kc, void* raw, unsigned jobs,
                       cudaStream_t st);
 
