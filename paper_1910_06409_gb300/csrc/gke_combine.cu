@@ -135,31 +135,24 @@ k_combine(const cplx<TI>* __restrict__ raw, int ny, int nz, int nx, double Lx, d
         s_nkx[kk] = (TC)2 * (TC)nu * s_kx[kk];
         s_nkz[kk] = (TC)2 * (TC)nu * s_kz[kk];
     }
-    // two consecutive values per thread (one 16-byte load on the split path)
-    for (int e = threadIdx.x; e < nslot * KC * PB * PB / 2; e += blockDim.x) {
-        const int e2 = 2 * e;
-        const int slot = e2 / (KC * PB * PB);
-        const int rem = e2 - slot * KC * PB * PB;
+    // asynchronous copies, so that all of a block's loads are in flight
+    // (FP64, 256 x 256 x 65: 10.5 -> 9.0 ms with loads through registers before);
+    // contractions outside the term set and rows and columns outside the
+    // grid become zeros without a read
+    for (int e = threadIdx.x; e < nslot * KC * PB * PB; e += blockDim.x) {
+        const int slot = e / (KC * PB * PB);
+        const int rem = e - slot * KC * PB * PB;
         const int q = rem / (PB * PB), rr = (rem / PB) % PB, cc = rem % PB;
         const int j = slot >> 1, partner = slot & 1;
         const int kq = k0 + q;
         const int yb = partner ? b : a, ypb = partner ? a : b;
-        C v0 = mk((TI)0, (TI)0), v1 = v0;
-        // contractions outside the term set stay zero, rows and columns outside the grid unread
-        if (kq < Nk && ((jmask >> j) & 1u) && rr < (partner ? nc : nr) && cc < (partner ? nr : nc)) {
-            const C* src = raw + ((((long long)j * nblk + yb) * nblk + ypb) * Nk + kq) * 64 + rr * PB + cc;
-            if (sizeof(C) == 8) {
-                const float4 f4 = __ldcs((const float4*)src);
-                v0 = *(const C*)&f4.x;
-                v1 = *(const C*)&f4.z;
-            } else {
-                v0 = src[0];
-                v1 = src[1];
-            }
-        }
-        at(slot, q, rr, cc) = v0;
-        at(slot, q, rr, cc + 1) = v1;
+        const bool in = kq < Nk && ((jmask >> j) & 1u) && rr < (partner ? nc : nr) && cc < (partner ? nr : nc);
+        const C* src = in ? raw + ((((long long)j * nblk + yb) * nblk + ypb) * Nk + kq) * 64 + rr * PB + cc : raw;
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(&at(slot, q, rr, cc));
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(sizeof(C)),
+                     "r"(in ? (int)sizeof(C) : 0) : "memory");
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     for (int it = threadIdx.x; it < KC * nr * nc; it += blockDim.x) {
         const int kk = it % KC, pm = it / KC, r = nc == PB ? pm / PB : pm / nc, m = pm - r * nc;
