@@ -81,9 +81,15 @@ __host__ __device__ inline int prod_field(int i, int k)
 // over snapshots; added to the accumulators with the constant coefficients
 // c[A .. psi_z]; ra >= 0 marks <u_ra(p1) u_rb(p2)'>, whose coefficient in xi
 // depends on the pair (add_job).
-struct Job { int nt; int fa[3]; int fb[3]; double c[6]; int ra, rb; };
+struct Job { int nt; int fa[3]; int fb[3]; double c[6]; float cf[6]; int ra, rb; };
 constexpr int NJ = 23;
 __constant__ Job c_job[NJ];
+// coefficient t in the sums' type (a conversion from double runs on the FP64 pipe)
+template <typename T> __device__ __forceinline__ T coef(const Job& jb, int t)
+{
+    if constexpr (sizeof(T) == 4) return jb.cf[t];
+    else return jb.c[t];
+}
 
 static void make_jobs(std::vector<Job>& js)
 {
@@ -92,7 +98,7 @@ static void make_jobs(std::vector<Job>& js)
                    int ra = -1, int rb = -1) {
         Job j{};
         for (auto& t : terms) { j.fa[j.nt] = t.first; j.fb[j.nt] = t.second; ++j.nt; }
-        for (auto& v : c) j.c[v.first] = v.second;
+        for (auto& v : c) { j.c[v.first] = v.second; j.cf[v.first] = (float)v.second; }
         j.ra = ra; j.rb = rb;
         js.push_back(j);
     };
@@ -335,7 +341,7 @@ __device__ __forceinline__ void add_job(cplx<TA>* T, const Job& jb, const cplx<T
 {
     #pragma unroll
     for (int t = 0; t < 6; ++t) {
-        const TA c = (TA)jb.c[t];
+        const TA c = coef<TA>(jb, t);
         if (c == (TA)0) continue;
         T[t].x = fma(c, acc.x, T[t].x);
         T[t].y = fma(c, acc.y, T[t].y);
@@ -408,7 +414,7 @@ __device__ __forceinline__ void fold_job(cplx<TF> (&T)[NACC][RB][RB], const Job&
 {
     #pragma unroll
     for (int t = 0; t < 6; ++t) {
-        const TF c = (TF)jb.c[t];
+        const TF c = coef<TF>(jb, t);
         if (c == (TF)0) continue;
         #pragma unroll
         for (int a = 0; a < RB; ++a)
@@ -514,7 +520,8 @@ k1_correlate(const zd* __restrict__ X, int ns, int P, int nx, int nt, double kx0
 // and up to SG32 snapshots, staged at once (cp.async): 37 terms read 22
 // staged field tiles, and no barrier stands between them.  (Staging the two
 // operands of each term took 74 tile loads behind 37 pairs of barriers: correlate
-// stage of 256 x 33 x 33, 16 snapshots 17.9 -> 12.7 ms; with 4 x 2 pairs on 128 threads
+// stage of 256 x 33 x 33, 16 snapshots 17.9 -> 12.7 ms, and 11.8 once the coefficients were
+// no longer converted from double; with 4 x 2 pairs on 128 threads
 // 13.4, too few warps.)  More snapshots are added group by group.
 constexpr int SG32 = 16;
 static size_t corr32_smem(int ns)
@@ -876,8 +883,9 @@ k1_transform(const cplx<TF>* __restrict__ spec, int nx, long long npair, int NB,
 // Register-FFT variant for nx = N1 N2 (gke::fft2l, twiddles resolved at
 // compile time): CTA = RZ sequences x N2 lanes, each sequence two pairs
 // packed as above; lane l holds the wavenumbers l + N2 j of its sequence.
+// Two CTAs per SM (256 x 33 x 33, FP64: 12.5 -> 9.6 ms, one CTA at 190 registers before).
 template <typename TF, int N1, int N2>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, N1 == 32 ? 1 : 2)
 k1_transform_r(const cplx<TF>* __restrict__ spec, long long npair, const cplx<TF>* __restrict__ tw,
                TF* __restrict__ terms)
 {
@@ -1000,7 +1008,7 @@ k1_stencil_a(TO* __restrict__ terms, const int* __restrict__ pq, Sten S, int nx,
 // changes sign under r-inversion (by the sign bit).  FP64: the stencils are bound
 // by their pipe, and in one sum with nothing but its 40 products k1_stencil_res
 // takes 41 operations a value instead of 49 or more (both stencils of 256 x 33 x 33
-// 26.2 -> 22.3 ms).  FP32 keeps derivs4's short sums: in one chain it is slower
+// 26.2 -> 22.3 ms; -> 19.9 with the registers of three CTAs instead of one per SM).  FP32 keeps derivs4's short sums: in one chain it is slower
 // (11.9 -> 14.2 ms).
 __device__ __forceinline__ void sum10(const double* __restrict__ plane, const long long* off, const signed char* flip,
                                       const double* w, int m, int nx, bool odd, double& d)
@@ -1015,7 +1023,7 @@ __device__ __forceinline__ void sum10(const double* __restrict__ plane, const lo
 }
 
 template <typename TO>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, sizeof(TO) == 8 ? 3 : 0)
 k1_stencil_res(TO* __restrict__ terms, const int* __restrict__ pq, Sten S, int nx, long long npair)
 {
     __shared__ long long off[SG][20];
