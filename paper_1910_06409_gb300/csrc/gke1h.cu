@@ -7,7 +7,8 @@
 // Stages of one evaluation (FP64 plans; FP32 plans as noted at the end):
 //   mean       k1_mean: U_f(p), the m_x = 0 coefficient averaged over the
 //              snapshots (Step 1); k1_grad: d_y U_i, d_z U_i by the stencils.
-//   products   k1_products, one CTA per point p: per snapshot the inverse x
+//   products   k1_products (k1_products_r at nx = 128, 256), one CTA per point
+//              p: per snapshot the inverse x
 //              transform of the fluctuations u, v, w, p, the in-plane
 //              products q = u_i u_i and u_i u_j, their forward transform; the
 //              operand blocks X[f][m_x][s][p] and the one-point sums.
@@ -17,9 +18,9 @@
 //              (Parseval, Eq. 8-9), combined into the per-pair term spectra,
 //              with the one-point parts and the mean-flow couplings; only
 //              term spectra reach HBM.  FP64 plans: 13 contractions on the
-//              tensor cores (digit_correlate).  FP32 plans, and FP64 plans
-//              whose digit workspace could not be allocated: k1_correlate,
-//              one CTA per (tile pair, m_x), 20 contractions, each added into
+//              tensor cores (digit_correlate).  FP32 plans (k1_correlate32), and
+//              FP64 plans whose digit workspace could not be allocated
+//              (k1_correlate): one CTA per (tile pair, m_x), 23 contractions, each added into
 //              the term spectra with its coefficients; a remainder of at most
 //              8 points past the last full tile runs as strips
 //              (k1_correlate_strip) instead of as padded tiles.
@@ -244,6 +245,112 @@ k1_products(const zd* __restrict__ f, int ns, int P, int nx, const zd* __restric
         m1[(long long)threadIdx.x * P + p] = v / ((double)ns * nx);
     }
     if (nonfinite) atomicExch(bad, 1);
+}
+
+// The same for nx = N1 N2 = 128, 256 by register transforms in fixed point, the
+// fields packed in pairs: two inverse and four forward transforms a snapshot
+// instead of 4 + 7 in FP64 through shared memory.  CTA = one point; N2 lanes of a warp take one
+// snapshot, u, v, w of it in shared memory between the transforms
+// (256 x 33 x 33, 16 snapshots: products stage 3.46 -> 1.35 ms, FP32 plans 3.87 -> 1.70).  512 points would
+// need more registers than a thread has.
+template <typename TF, int N1, int N2>
+__global__ void __launch_bounds__(128)
+k1_products_r(const zd* __restrict__ f, int ns, int P, const zd* __restrict__ tw, const double* __restrict__ prof,
+              cplx<TF>* __restrict__ X, double* __restrict__ m1, int* __restrict__ bad)
+{
+    constexpr int N = N1 * N2, nxh = N / 2 + 1, GR = 128 / N2;
+    extern __shared__ zd sm_pr[];
+    zd* stw = sm_pr;
+    const int lane = threadIdx.x % N2, g = threadIdx.x / N2;
+    zd* xr = stw + N + g * N1 * (N2 + 1);
+    double* ph = (double*)(stw + N + GR * N1 * (N2 + 1)) + g * 3 * N + lane;
+    gke::load_twiddles2l<double>(stw, tw, N);
+    const int p = blockIdx.x;
+    double acc[NM1];
+    #pragma unroll
+    for (int k = 0; k < NM1; ++k) acc[k] = 0.0;
+    bool nonfinite = false;
+    __syncthreads();
+    for (int s0 = 0; s0 < ns; s0 += GR) {
+        const bool live = s0 + g < ns;
+        const int s = live ? s0 + g : 0;
+        zd vb[N1];
+        #pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const zd* fa = f + ((long long)(s * 4 + 2 * q) * P + p) * nxh;
+            const zd* fb = fa + (long long)P * nxh;
+            const double ma = prof[(long long)(R_U + 2 * q) * P + p], mb = prof[(long long)(R_U + 2 * q + 1) * P + p];
+            #pragma unroll
+            for (int m = 0; m < N1; ++m) {
+                const int k = lane + N2 * m, kk = k < nxh ? k : N - k;
+                zd a = fa[kk], b = fb[kk];
+                if (k < nxh) nonfinite |= !isfinite(a.x) || !isfinite(a.y) || !isfinite(b.x) || !isfinite(b.y);
+                if (kk == 0) { a.x -= ma; b.x -= mb; }
+                if (kk == 0 || 2 * kk == N) a.y = b.y = 0.0;
+                if (k < nxh) {
+                    if (live) {
+                        X[(((long long)(2 * q) * nxh + k) * ns + s) * P + p] = cvt<TF>(a);
+                        X[(((long long)(2 * q + 1) * nxh + k) * ns + s) * P + p] = cvt<TF>(b);
+                    }
+                } else { a.y = -a.y; b.y = -b.y; }
+                vb[m] = mk(a.x - b.y, a.y + b.x);        // a + i b
+            }
+            __syncwarp();
+            gke::fft2l_rows<double, N1, N2, true>(vb, lane, xr, N2 + 1, 1, stw);
+            if (q == 0) {
+                #pragma unroll
+                for (int m = 0; m < N1; ++m) { ph[N2 * m] = vb[m].x; ph[N + N2 * m] = vb[m].y; }
+            }
+        }
+        #pragma unroll
+        for (int m = 0; m < N1; ++m) {
+            const double u = ph[N2 * m], v = ph[N + N2 * m], w = vb[m].x, pp = vb[m].y;
+            ph[2 * N + N2 * m] = w;
+            if (!live) continue;
+            const double uu = u * u, vv = v * v, ww = w * w, q = uu + vv + ww;
+            acc[M_UU] += uu; acc[M_VV] += vv; acc[M_WW] += ww;
+            acc[M_UV] += u * v; acc[M_UW] += u * w; acc[M_VW] += v * w;
+            acc[M_QU] += q * u; acc[M_QV] += q * v; acc[M_QW] += q * w;
+            acc[M_PV] += pp * v; acc[M_PW] += pp * w;
+        }
+        #pragma unroll 1
+        for (int j = 0; j < 4; ++j) {
+            zd h[N1];
+            #pragma unroll
+            for (int m = 0; m < N1; ++m) {
+                const double u = ph[N2 * m], v = ph[N + N2 * m], w = ph[2 * N + N2 * m];
+                h[m] = j == 0 ? mk(u * u, v * v) : j == 1 ? mk(w * w, u * v) : j == 2 ? mk(u * w, v * w)
+                              : mk(u * u + v * v + w * w, 0.0);
+            }
+            const int fa = j == 0 ? G_UU : j == 1 ? G_WW : j == 2 ? G_UW : G_Q, fb = j == 0 ? G_VV : j == 1 ? G_UV : G_VW;
+            __syncwarp();
+            gke::fft2l_split<double, N1, N2>(h, lane, xr, stw, [&](int k, zd a, zd b) {
+                if (!live) return;
+                X[(((long long)fa * nxh + k) * ns + s) * P + p] = cvt<TF>(a);
+                if (j < 3) X[(((long long)fb * nxh + k) * ns + s) * P + p] = cvt<TF>(b);
+            });
+        }
+        __syncwarp();
+    }
+    // block sums of the one-point statistics
+    __shared__ double red[NM1][4];
+    const int wl = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    #pragma unroll
+    for (int k = 0; k < NM1; ++k) {
+        double v = acc[k];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (wl == 0) red[k][wid] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < NM1)
+        m1[(long long)threadIdx.x * P + p] = (red[threadIdx.x][0] + red[threadIdx.x][1] + red[threadIdx.x][2] +
+                                              red[threadIdx.x][3]) / ((double)ns * N);
+    if (nonfinite) atomicExch(bad, 1);
+}
+static size_t products_r_smem(int n1, int n2)
+{
+    const int gr = 128 / n2;
+    return (size_t)(n1 * n2 + gr * n1 * (n2 + 1)) * sizeof(zd) + (size_t)gr * 3 * n1 * n2 * sizeof(double);
 }
 
 // eps by Parseval in x (signed wavenumber, 0 at the Nyquist index; weight 2
@@ -1226,6 +1333,12 @@ static cudaError_t set_attrs(gke1h_plan_t p)
 {
     typedef cplx<TF> C;
     cudaError_t e = cudaFuncSetAttribute(k1_products<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem_prod);
+    if (e == cudaSuccess && p->nx == 256)
+        e = cudaFuncSetAttribute(k1_products_r<TF, 16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)products_r_smem(16, 16));
+    if (e == cudaSuccess && p->nx == 128)
+        e = cudaFuncSetAttribute(k1_products_r<TF, 16, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)products_r_smem(16, 8));
     if (e == cudaSuccess && sizeof(TF) == 4)
         e = cudaFuncSetAttribute(k1_correlate32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)corr32_smem(SG32));
     if (e != cudaSuccess) return e;
@@ -1386,7 +1499,12 @@ static void launch_pass(gke1h_plan_t p, const zd* f, int ns, TF* T)
     }
     {
         Scope1 sc(p, GKE_STAGE_PRODUCTS);
-        k1_products<TF><<<P, 256, p->smem_prod, p->st>>>(f, ns, P, nx, p->tw, p->prof, X, p->m1, p->bad);
+        if (nx == 256)
+            k1_products_r<TF, 16, 16><<<P, 128, products_r_smem(16, 16), p->st>>>(f, ns, P, p->tw, p->prof, X, p->m1, p->bad);
+        else if (nx == 128)
+            k1_products_r<TF, 16, 8><<<P, 128, products_r_smem(16, 8), p->st>>>(f, ns, P, p->tw, p->prof, X, p->m1, p->bad);
+        else
+            k1_products<TF><<<P, 256, p->smem_prod, p->st>>>(f, ns, P, nx, p->tw, p->prof, X, p->m1, p->bad);
         k1_onepoint<TF><<<P, 128, 0, p->st>>>(X, ns, p->ny, p->nz, nx, kx0, p->nu, p->wy, p->ly, p->wz, p->lz,
                                              p->m1, p->prof, p->op);
         p->launches += 2;

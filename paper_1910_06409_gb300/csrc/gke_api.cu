@@ -995,7 +995,7 @@ static void products_stage(gke_plan_t p, const zd* f, int ns)
     a.tw_x = f32 ? (const void*)p->tw_xf : (const void*)p->tw_xd;
     a.tw_z = f32 ? (const void*)p->tw_zf : (const void*)p->tw_zd;
     a.part = p->part; a.stats = p->stats; a.nonfinite = p->nonfinite;
-    a.cw_ci = t.cw_ci; a.rz_rp = t.rz_rp; a.cw_cf = t.cw_cf; a.yb_cf = t.yb_cf; a.eps_kchunk = EPS_KCHUNK;
+    a.cw_ci = t.cw_ci; a.rz_rp = t.rz_rp; a.cw_cf = t.cw_cf; a.yb_cf = t.yb_cf;
     a.Lx = d.Lx; a.Lz = d.Lz; a.fdw = p->fdw; a.fdl0 = p->fdl0; a.st = p->st;
     a.st2 = p->aux_st; a.G2 = p->G2; a.H2 = p->H2; a.part2 = p->part2; a.ev = p->aux_ev;
     a.up_ev = p->up_active;

@@ -127,7 +127,7 @@ struct ProdArgs {
     const zd* fields; int ns, ny, nz, nx, nxh, Nk;
     const double* mean; void* Xop; void* G; void* H; const void* tw_x; const void* tw_z;
     double* part; double* stats; int* nonfinite;
-    int cw_ci, rz_rp, cw_cf, yb_cf, eps_kchunk;
+    int cw_ci, rz_rp, cw_cf, yb_cf;
     double Lx, Lz; const double* fdw; const int* fdl0;
     cudaStream_t st;
     // optional second stream and buffers: odd snapshots run there

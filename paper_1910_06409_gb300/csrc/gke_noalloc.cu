@@ -196,7 +196,7 @@ extern "C" gke_status gke_compute_noalloc(const gke_desc* desc, const void* fiel
     a.fields = f; a.ns = ns; a.ny = ny; a.nz = nz; a.nx = nx; a.nxh = nxh; a.Nk = Nk;
     a.mean = mean; a.Xop = Xop; a.G = G; a.H = H; a.tw_x = twx; a.tw_z = twz;
     a.part = part; a.stats = stats; a.nonfinite = nonfinite;
-    a.cw_ci = tl.cw_ci; a.rz_rp = tl.rz_rp; a.cw_cf = tl.cw_cf; a.yb_cf = tl.yb_cf; a.eps_kchunk = EPS_KCHUNK;
+    a.cw_ci = tl.cw_ci; a.rz_rp = tl.rz_rp; a.cw_cf = tl.cw_cf; a.yb_cf = tl.yb_cf;
     a.Lx = d.Lx; a.Lz = d.Lz; a.fdw = fdw; a.fdl0 = fdl0; a.st = st;
     products_launch<double>(a);
     correlate_launch(false, Xop, ns, ny, Nk, 0, Nk, raw, job_set(tset), st);
