@@ -151,6 +151,8 @@ __device__ __forceinline__ zd dg_load(const DgPrep& a, const DgField& fd, int k,
     return mk(p * v.x + q * w.x, p * v.y + q * w.y);
 }
 
+constexpr int DG_NAN = 8192;                                // exponent of a row with an infinity or a NaN
+
 // round(x 2^sh) for |x| 2^sh < 2^61, in integer arithmetic (a conversion would
 // run on the FP64 pipe)
 __device__ __forceinline__ unsigned long long dg_fixed(double x, int sh)
@@ -186,7 +188,7 @@ __device__ __forceinline__ uint32_t dg_pair(uint32_t a, uint32_t b, int c)
 static __global__ void __launch_bounds__(256)
 k_dg_prep(const __grid_constant__ DgPrep a)
 {
-    __shared__ int s_hi[128];
+    __shared__ unsigned s_hi[128];
     const int nb = a.s.nrow / 128;
     int b = blockIdx.x;
     const int mb = b % nb; b /= nb;
@@ -196,19 +198,20 @@ k_dg_prep(const __grid_constant__ DgPrep a)
     if (threadIdx.x < 128) s_hi[threadIdx.x] = 0;
     __syncthreads();
     const int e0 = kc * 8, ne = y < a.s.n ? max(0, min(8, a.ns - e0)) : 0;
-    int hi = 0;
+    unsigned hi = 0;
     for (int f = 0; f < a.nf; ++f) {
         const DgField fd = a.f[f];
         if (fd.grp != g) continue;
         for (int e = 0; e < ne; ++e) {
             const zd v = dg_load(a, fd, k, e0 + e, y);
-            const int h = max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
-            if (h >= 0x00100000) hi = max(hi, h + fd.wexp * 0x00100000);
+            // (unsigned: an infinity or a NaN times 2^wexp stays above 0x7ff00000)
+            const unsigned h = (unsigned)max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+            if (h >= 0x00100000u) hi = max(hi, h + fd.wexp * 0x00100000u);
         }
     }
     atomicMax(&s_hi[r], hi);
     __syncthreads();
-    const int E = max(s_hi[r] >> 20, 1) - 1022;              // |x| < 2^E
+    const int E = s_hi[r] >= 0x7ff00000u ? DG_NAN : max((int)(s_hi[r] >> 20), 1) - 1022;              // |x| < 2^E
     if (kc == 0) a.E[((long long)k * a.ngrp + g) * a.s.nrow + y] = E;
     const bool arow = mb < a.s.MT && r < a.s.RT && y < a.s.cov, astore = mb < a.s.MT && r < a.s.RT;
     const int c = y / a.s.CW, rc = y - c * a.s.CW;
@@ -313,8 +316,11 @@ __device__ __forceinline__ long long dg_high(const uint32_t (&r)[4][4], int j, l
     const unsigned up = (unsigned)((unsigned long long)v >> 32) + (bits(0) << 13) + (bits(1) << 5);
     return (long long)(((unsigned long long)up << 32) | (unsigned)v);
 }
-// t 2^(e - 21) in general
-static __device__ __noinline__ double dg_value_edge(long long t, int e) { return scalbn((double)t, e - 21); }
+// t 2^(e - 21) in general; NaN where an operand row holds an infinity or a NaN
+static __device__ __noinline__ double dg_value_edge(long long t, int e)
+{
+    return e > DG_NAN / 2 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)t, e - 21);
+}
 // t 2^(e - 21), normalised and rounded to nearest in integer arithmetic (a
 // conversion would hold the FP64 pipe of the whole SM for 16 clocks a warp).
 // No branch, so that values interleave; edge is raised where the upper
@@ -527,6 +533,7 @@ k_dg_corr(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
                     if (job.gb == g) ebj = eb[g];
                 }
                 ej += job.e;
+                const bool bad = __any_sync(0xffffffffu, max(ej, ebj) > DG_NAN / 2);
                 long long lo[2][HC];
                 uint32_t v[2][4][4];
                 // orders 4..7
@@ -560,7 +567,7 @@ k_dg_corr(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
                         dg_ready(v);
                         const int yp = c0 + 4 * g;
                         zd o[4];
-                        bool edge = false;
+                        bool edge = bad;
                         #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             const int e = ej + __shfl_sync(0xffffffffu, ebj, 4 * g + j);
