@@ -77,7 +77,7 @@ def correlator_cmac(wl, ns):
 # (profiles/dram_small_cases_split_and_f64.md); a stage missing here reports
 # null (not captured since its kernels changed).
 NCU_TRAFFIC_GB = {
-    "f64": {"correlate": 96.7, "combine": 93.0, "terms": 104.0, "stencil": 38.0, "products": 27.8},
+    "f64": {"stencil": 38.0},
     "bf16x3": {"correlate": 36.6, "terms": 55.9, "stencil": 20.5, "products": 16.4},
 }
 
@@ -95,8 +95,9 @@ def stage_rooflines(wl, ns, precision, stage_ms, pk, pk_kind):
 
     Bytes count each stage's essential inputs read once and outputs written
     once (workspaces between kernels of a stage are not counted); the
-    contraction stage counts flops (tensor BF16 on the split path, FP64 DFMA
-    on the plain path)."""
+    contraction stage counts flops (tensor BF16 on the split path; FP64 on the
+    plain path, against the FP64 FMA pipe: the exact digit products on the tensor
+    cores pass it)."""
     f32 = precision != "f64"
     cz = 8 if f32 else 16                          # bytes of one complex operand / spectrum value
     tz = 4 if f32 else 8                           # bytes of one term value
@@ -155,8 +156,8 @@ def stage_rooflines(wl, ns, precision, stage_ms, pk, pk_kind):
             out["correlate"] = {"bound": "alu", "achieved": flops / (ms / 1e3) / 1e12, "peak": peak,
                                 "unit": "TFLOP/s", "flops": flops, "launch_ms": ms,
                                 "traffic": ncu_traffic(wl, precision, "correlate"),
-                                "peak_source": "derived: 152 SM x 2 DFMA/clk x 2 flop x max SM clock "
-                                               "(nominal 1.25 TFLOP/s FP64)"}
+                                "peak_source": "derived: FP64 FMA pipe, 152 SM x 2 DFMA/clk x 2 flop x max SM clock "
+                                               "(nominal 1.25 TFLOP/s); exact digit products on the tensor cores pass it"}
         out["correlate"]["frac"] = out["correlate"]["achieved"] / out["correlate"]["peak"]
     return out
 
@@ -555,10 +556,10 @@ def run_step1(args, world, rank, local):
 METRIC_1H = "GKE one-homogeneous-direction (p1,p2)-pair correlations/s, FP64"
 
 
-# DRAM bytes of one k1_correlate launch on the small case duct_256x17x17_s16
-# (41,905 pairs), scaled in proportion to the pairs of the workload run
-# (profiles/k1_correlate_profile_duct_256x17x17_s16.md)
-NCU_CORR_1H = (0.749e9, 41905)
+# DRAM bytes of one pass's k_dg_prep, k_dg_corr and k1_finish launches on the small
+# case duct_256x17x17_s16 (41,905 pairs), scaled in proportion to the pairs of the
+# workload run (profiles/counters_fp64_digits_128x128x65_s16_and_duct_256x17x17_s16.md)
+NCU_CORR_1H = (3.994e9, 41905)
 
 
 def correlator_cmac_1h(wl, ns):
@@ -653,7 +654,8 @@ def run_one_homog(args, world, rank, local):
             "flops": flops, "launch_ms": cms, "stage": "correlate",
             "traffic": int(NCU_CORR_1H[0] * wl.npair / NCU_CORR_1H[1]) if ns == 16 else None,
             "traffic_note": "small-case ncu capture scaled by pairs",
-            "peak_source": "derived: 152 SM x 2 DFMA/clk x 2 flop x max SM clock (nominal 1.25 TFLOP/s FP64)"}
+            "peak_source": "derived: FP64 FMA pipe, 152 SM x 2 DFMA/clk x 2 flop x max SM clock (nominal 1.25 TFLOP/s); "
+                           "exact digit products on the tensor cores pass it"}
     cpu = None
     if not args.no_cpu:
         phys = S.duct_physical(wl)

@@ -97,7 +97,7 @@ typedef enum {
     GKE_ERR_UNSUPPORTED = -7   /* grid size or option the library does not support   */
 } gke_status;
 
-enum { GKE_PREC_F64 = 0,       /* plain FP64 path (DFMA)                              */
+enum { GKE_PREC_F64 = 0,       /* plain FP64 path                                     */
        GKE_PREC_BF16X3 = 1,    /* split-BF16 correlator on the tensor cores, FP32 rest */
        GKE_PREC_F32 = 2 };     /* FP32 correlator on the CUDA cores (FFMA), FP32 rest  */
 

@@ -2,10 +2,10 @@
 // (gke_digits.cuh has the method).
 //
 // Measured, correlate stage (operands, contractions; FMA kernel -> here):
-// 256 x 256 x 65, 16 snapshots 232.8 -> 33.9 ms, of which the operand kernel 6.5
+// 256 x 256 x 65, 16 snapshots 232.8 -> 34.7 ms, of which the operand kernel 6.5
 // and the MMAs alone 23 (smem reads of A and B: 18.5 by count), which bound it
 // with the epilogue (conversions and integer adds) close behind; 128 x 128 x 65,
-// 32 snapshots 117.4 -> 18.2 ms.  Errors against 64-bit references equal the
+// 32 snapshots 117.4 -> 18.6 ms.  Errors against 64-bit references equal the
 // FMA kernel's or are below.
 #include "gke_digits.h"
 #include "gke_digits.cuh"

@@ -14,9 +14,9 @@
 // 16 times the 2-norm.  An FP64 transform's error is about 2^-52.3 of the 2-norm.
 //
 // Measured (FP64 transforms -> here): 256 x 256 x 65, 16 snapshots: inverse transforms
-// of the terms 56.9 -> 19.8 ms, products stage 46.7 -> 21.0 ms; duct 256 x 33 x 33:
-// 30.0 -> 12.9 ms; 128 x 128 x 65, 32 snapshots (from shared-memory stages of FP64):
-// products 28.7 -> 11.0 ms, terms 15.3 -> 5.1 ms.  Errors of the terms against 64-bit references do not grow (duct
+// of the terms 56.9 -> 19.3 ms, products stage 46.7 -> 20.6 ms; duct 256 x 33 x 33:
+// 30.0 -> 9.6 ms; 128 x 128 x 65, 32 snapshots (from shared-memory stages of FP64):
+// products 28.7 -> 10.9 ms, terms 15.3 -> 4.8 ms.  Errors of the terms against 64-bit references do not grow (duct
 // A 1.6e-16 -> 1.2e-16).  (Exponents from the largest component and 56 bits were as
 // fast, but raised them by up to a half.)
 #pragma once
