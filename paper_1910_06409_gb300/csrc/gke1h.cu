@@ -1459,7 +1459,7 @@ extern "C" gke_status gke1h_plan(const gke1h_desc* d, void* stream, gke1h_plan_t
             free_plan(p);
             return fail1(nullptr, GKE_ERR_CUDA, "shared-memory attributes refused");
         }
-        gke::digits_alloc(p->digits, digit_bytes(p->P), p->nxh);
+        gke::digits_alloc(p->digits, digit_bytes(p->P), p->nxh, p->st);
     }
     *out = p;
     return GKE_OK;

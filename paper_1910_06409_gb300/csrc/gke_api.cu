@@ -709,11 +709,11 @@ extern "C" gke_status gke_plan(const gke_desc* desc, void* stream, gke_plan_t* o
         ALLOC(p->part2, p->part_count);
     }
     if (d.precision == GKE_PREC_BF16X3) {
-        gke_status s = split_alloc(p->split, ny, ns, p->Kc);
+        gke_status s = split_alloc(p->split, ny, ns, p->Kc, p->st);
         if (s != GKE_OK) return bail(s, "split workspace allocation failed");
     }
     if (d.precision == GKE_PREC_F64 && digits_pays(ny, ns, p->Kc)) {
-        if ((e = digits_setup(p->digits, ny, p->Kc)) != cudaSuccess)
+        if ((e = digits_setup(p->digits, ny, p->Kc, p->st)) != cudaSuccess)
             return bail(GKE_ERR_CUDA, std::string("digit setup: ") + cudaGetErrorString(e));
     }
 #undef ALLOC

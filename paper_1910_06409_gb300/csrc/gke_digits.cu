@@ -81,19 +81,19 @@ constexpr int CH_NFA = 11, CH_NFB = 3, CH_NGRP = 3;
 // digit operands are made and used in chunks of wavenumbers of this many bytes
 static const size_t DG_CHUNK_BYTES = (size_t)512 << 20;
 
-void digits_alloc(DigitWork& w, size_t per, int Kc)
+void digits_alloc(DigitWork& w, size_t per, int Kc, cudaStream_t st)
 {
     w.bytes = per * std::max<size_t>(1, std::min<size_t>((size_t)Kc, DG_CHUNK_BYTES / per));
     if (cudaMalloc(&w.ws, w.bytes) != cudaSuccess) w.ws = nullptr;
-    if (w.ws && (cudaMalloc((void**)&w.err, sizeof(int)) != cudaSuccess || cudaMemset(w.err, 0, sizeof(int)) != cudaSuccess))
+    if (w.ws && (cudaMalloc((void**)&w.err, sizeof(int)) != cudaSuccess || cudaMemsetAsync(w.err, 0, sizeof(int), st) != cudaSuccess))
         digits_free(w);
     cudaGetLastError();
 }
 
-cudaError_t digits_setup(DigitWork& w, int n, int Kc)
+cudaError_t digits_setup(DigitWork& w, int n, int Kc, cudaStream_t st)
 {
     const cudaError_t e = dg_attrs<RawOut>();
-    if (e == cudaSuccess) digits_alloc(w, dg_bytes_per_k(dg_shape(n, true), CH_NFA, CH_NFB, CH_NGRP), Kc);
+    if (e == cudaSuccess) digits_alloc(w, dg_bytes_per_k(dg_shape(n, true), CH_NFA, CH_NFB, CH_NGRP), Kc, st);
     return e;
 }
 

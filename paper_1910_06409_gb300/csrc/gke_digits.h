@@ -15,11 +15,12 @@ struct DigitWork {
 };
 
 // workspace for chunks of up to Kc wavenumbers of `per` bytes each; on failure
-// the work stays empty (digits_ready false) and the callers keep their FMA kernels
-void digits_alloc(DigitWork& w, size_t per, int Kc);
+// the work stays empty (digits_ready false) and the callers keep their FMA kernels;
+// st: the stream of the passes (the error flag is cleared in its order)
+void digits_alloc(DigitWork& w, size_t per, int Kc, cudaStream_t st);
 inline bool digits_ready(const DigitWork& w) { return w.ws != nullptr; }
 // the channel's kernels and workspace (n wall-normal points)
-cudaError_t digits_setup(DigitWork& w, int n, int Kc);
+cudaError_t digits_setup(DigitWork& w, int n, int Kc, cudaStream_t st);
 // whether the digit products are the faster way for a batch (measured; gke_digits.cu)
 bool digits_pays(int n, int ns, long long Kc);
 // the contractions `jobs` of the wavenumbers [k0, k0 + Kc) into raw (as

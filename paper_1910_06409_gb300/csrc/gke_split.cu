@@ -946,7 +946,7 @@ static void tile_geometry(int ny, int& MT, int& cov)
 }
 
 // operand slices for Kc wavenumbers (one chunk)
-gke_status split_alloc(SplitWork& w, int ny, int ns, int Kc)
+gke_status split_alloc(SplitWork& w, int ny, int ns, int Kc, cudaStream_t st)
 {
     const int Nk = Kc;
 
@@ -957,7 +957,7 @@ gke_status split_alloc(SplitWork& w, int ny, int ns, int Kc)
     w.b_bytes = (size_t)Nk * NFB * G * MT * B_STAGE * sizeof(bf16);
     if (cudaMalloc(&w.ops, w.a_bytes + w.b_bytes) != cudaSuccess) { w.ops = nullptr; return GKE_ERR_OOM; }
     if (cudaMalloc((void**)&w.err, sizeof(int)) != cudaSuccess) { w.err = nullptr; return GKE_ERR_OOM; }
-    if (cudaMemset(w.err, 0, sizeof(int)) != cudaSuccess) return GKE_ERR_CUDA;
+    if (cudaMemsetAsync(w.err, 0, sizeof(int), st) != cudaSuccess) return GKE_ERR_CUDA;
     w.ops_bytes = w.a_bytes + w.b_bytes;
     return GKE_OK;
 }

@@ -14,7 +14,8 @@ struct SplitWork {
     int* err = nullptr;         // device flag: a pipeline wait timed out
 };
 
-gke_status split_alloc(SplitWork& w, int ny, int ns, int Kc);
+// st: the stream of the passes (the error flag is cleared in its order)
+gke_status split_alloc(SplitWork& w, int ny, int ns, int Kc, cudaStream_t st);
 cudaError_t split_setup(cudaStream_t st);
 gke_status split_correlate(SplitWork& w, const zf* Xop, int ns, int ny, int Nk, int k0, int Kc, zf* raw,
                            unsigned jobs, cudaStream_t st, std::string& err, int* launches);
