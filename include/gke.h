@@ -149,7 +149,11 @@ unsigned gke_term_set(unsigned term_mask);
 /* Create a plan: validates the descriptor, computes the FD weights and
  * twiddles on the host, allocates every workspace on the current device.
  * stream: a cudaStream_t (NULL = legacy default stream).  Nothing is
- * allocated later except the staging buffer of a first host-output finalize. */
+ * allocated later except the staging buffer of a first host-output finalize.
+ * GKE_PREC_F64 plans take up to 512 MiB for the operands of their
+ * contractions; with less free they take less, and without room for one
+ * wavenumber's their contractions run without tensor cores, several times
+ * slower.                                                                     */
 gke_status gke_plan(const gke_desc* desc, void* stream, gke_plan_t* out);
 
 /* Step 1 (Sec. 3.2) for databases in velocity-vorticity form: the fields

@@ -89,7 +89,10 @@ typedef struct {
  * the stencil weights and twiddles on the host and allocates every
  * workspace on the current device (about c (8 npair + 11 max_snap P)
  * (nx/2 + 1) bytes, c = 16 on GKE_PREC_F64 plans and 8 on GKE_PREC_F32;
- * GKE_ERR_OOM if the device has not that much free).
+ * GKE_ERR_OOM if the device has not that much free).  A GKE_PREC_F64 plan
+ * also takes up to 512 MiB for the operands of its contractions; with less
+ * free it takes less, and without room for one wavenumber's (about 30 kB per
+ * point) its contractions run without tensor cores, several times slower.
  * stream: a cudaStream_t (NULL = legacy default stream).  Nothing is
  * allocated later except a staging buffer of the terms (8 or 4 bytes x
  * GKE1H_NTERM npair nx) on the first call with host-memory terms.           */

@@ -1657,4 +1657,15 @@ extern "C" long long gke1h_launch_count(gke1h_plan_t p) { return p ? p->launches
 
 extern "C" const char* gke1h_last_error(gke1h_plan_t p) { return p ? p->err.c_str() : g1_err.c_str(); }
 
+// Internal, for the tests: as gke_test_digit_workspace.
+extern "C" gke_status gke1h_test_digit_workspace(gke1h_plan_t p, long long bytes)
+{
+    if (!p || p->f32) return GKE_ERR_STATE;
+    TRY1(p, cudaStreamSynchronize(p->st));
+    gke::digits_free(p->digits);
+    if (bytes <= 0) return GKE_OK;
+    gke::digits_alloc(p->digits, digit_bytes(p->P), p->nxh, p->st, (size_t)bytes);
+    return gke::digits_ready(p->digits) ? GKE_OK : GKE_ERR_OOM;
+}
+
 extern "C" void gke1h_destroy(gke1h_plan_t p) { free_plan(p); }

@@ -822,6 +822,18 @@ extern "C" gke_status gke_plan(const gke_desc* desc, void* stream, gke_plan_t* o
     return GKE_OK;
 }
 
+// Internal, for the tests: another digit workspace, of at most `bytes` (but one
+// wavenumber), or with bytes <= 0 none, which leaves the contractions to the FMA kernel.
+extern "C" gke_status gke_test_digit_workspace(gke_plan_t p, long long bytes)
+{
+    if (!p || p->d.precision != GKE_PREC_F64 || p->graph) return GKE_ERR_STATE;
+    CUDA_TRY(p, cudaStreamSynchronize(p->st));
+    digits_free(p->digits);
+    if (bytes <= 0) return GKE_OK;
+    digits_alloc(p->digits, digits_per_k(p->d.ny), p->Kc, p->st, (size_t)bytes);
+    return digits_ready(p->digits) ? GKE_OK : GKE_ERR_OOM;
+}
+
 extern "C" unsigned gke_term_set(unsigned term_mask) { return term_set(term_mask & GKE_ALL_TERMS); }
 
 extern "C" gke_status gke_reset(gke_plan_t p)

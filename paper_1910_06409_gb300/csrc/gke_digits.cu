@@ -78,13 +78,15 @@ static const HostJob kJobs[NJOB] = {
 // channel: 11 A fields, 3 B fields, 3 exponent groups
 constexpr int CH_NFA = 11, CH_NFB = 3, CH_NGRP = 3;
 
-// digit operands are made and used in chunks of wavenumbers of this many bytes
-static const size_t DG_CHUNK_BYTES = (size_t)512 << 20;
+size_t digits_per_k(int n) { return dg_bytes_per_k(dg_shape(n, true), CH_NFA, CH_NFB, CH_NGRP); }
 
-void digits_alloc(DigitWork& w, size_t per, int Kc, cudaStream_t st)
+void digits_alloc(DigitWork& w, size_t per, int Kc, cudaStream_t st, size_t limit)
 {
-    w.bytes = per * std::max<size_t>(1, std::min<size_t>((size_t)Kc, DG_CHUNK_BYTES / per));
-    if (cudaMalloc(&w.ws, w.bytes) != cudaSuccess) w.ws = nullptr;
+    w.ws = nullptr;
+    for (size_t nk = std::max<size_t>(1, std::min<size_t>((size_t)Kc, limit / per)); nk && !w.ws; nk /= 2) {
+        w.bytes = per * nk;
+        if (cudaMalloc(&w.ws, w.bytes) != cudaSuccess) w.ws = nullptr;
+    }
     if (w.ws && (cudaMalloc((void**)&w.err, sizeof(int)) != cudaSuccess || cudaMemsetAsync(w.err, 0, sizeof(int), st) != cudaSuccess))
         digits_free(w);
     cudaGetLastError();
@@ -93,7 +95,7 @@ void digits_alloc(DigitWork& w, size_t per, int Kc, cudaStream_t st)
 cudaError_t digits_setup(DigitWork& w, int n, int Kc, cudaStream_t st)
 {
     const cudaError_t e = dg_attrs<RawOut>();
-    if (e == cudaSuccess) digits_alloc(w, dg_bytes_per_k(dg_shape(n, true), CH_NFA, CH_NFB, CH_NGRP), Kc, st);
+    if (e == cudaSuccess) digits_alloc(w, digits_per_k(n), Kc, st);
     return e;
 }
 
@@ -114,7 +116,7 @@ gke_status digits_correlate(DigitWork& w, const zd* Xop, int ns, int ny, int Nk,
     DgArgs a{};
     const DgShape s = dg_shape(ny, true);
     dg_init(p, a, s, CH_NFA, CH_NFB, CH_NGRP, false, w.err);
-    const int kmax = (int)std::min<size_t>((size_t)Kc, w.bytes / dg_bytes_per_k(s, CH_NFA, CH_NFB, CH_NGRP));
+    const int kmax = (int)std::min<size_t>((size_t)Kc, w.bytes / digits_per_k(ny));
     for (int f = 0; f < NFIELD; ++f) {
         DgField& d = p.f[p.nf++];
         d.src = (short)f;

@@ -14,13 +14,18 @@ struct DigitWork {
     int* err = nullptr;         // device flag: a pipeline wait timed out
 };
 
-// workspace for chunks of up to Kc wavenumbers of `per` bytes each; on failure
-// the work stays empty (digits_ready false) and the callers keep their FMA kernels;
+// operands are made and used in chunks of wavenumbers of this many bytes at most
+constexpr size_t DG_CHUNK_BYTES = (size_t)512 << 20;
+// workspace for chunks of up to Kc wavenumbers of `per` bytes each, `limit`
+// bytes (but one wavenumber) at most; where the device has less free, half of it
+// and so on.  Only where one wavenumber's operands find no room the work stays
+// empty (digits_ready false) and the callers keep their FMA kernels;
 // st: the stream of the passes (the error flag is cleared in its order)
-void digits_alloc(DigitWork& w, size_t per, int Kc, cudaStream_t st);
+void digits_alloc(DigitWork& w, size_t per, int Kc, cudaStream_t st, size_t limit = DG_CHUNK_BYTES);
 inline bool digits_ready(const DigitWork& w) { return w.ws != nullptr; }
 // the channel's kernels and workspace (n wall-normal points)
 cudaError_t digits_setup(DigitWork& w, int n, int Kc, cudaStream_t st);
+size_t digits_per_k(int n);                 // bytes of one wavenumber
 // whether the digit products are the faster way for a batch (measured; gke_digits.cu)
 bool digits_pays(int n, int ns, long long Kc);
 // the contractions `jobs` of the wavenumbers [k0, k0 + Kc) into raw (as
