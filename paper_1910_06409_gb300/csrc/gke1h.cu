@@ -17,7 +17,7 @@
 //   correlate  the snapshot sums of the correlation products of Eq. 7
 //              (Parseval, Eq. 8-9), combined into the per-pair term spectra,
 //              with the one-point parts and the mean-flow couplings; only
-//              term spectra reach HBM.  FP64 plans: 13 contractions on the
+//              term spectra reach HBM.  FP64 plans: 17 contractions on the
 //              tensor cores (digit_correlate).  FP32 plans (k1_correlate32), and
 //              FP64 plans whose digit workspace could not be allocated
 //              (k1_correlate): one CTA per (tile pair, m_x), 23 contractions, each added into
@@ -748,16 +748,18 @@ k1_correlate_strip(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int co
 
 // ---------------------------------------------- correlate, digit products
 // FP64 plans: the contractions on the tensor cores (gke_digits.cuh).  Every
-// spectrum is one or two contractions of at most five terms whose A and B
-// fields share exponent groups (g0: u, v, w; g1: the products, pairs u_i u_k
-// doubled; g2: w_a = 2 sum_b d_b U_a u_b, b = y, z; g3: the products again with 4 p):
+// spectrum is a sum of contractions of one to four terms:
 //   A     = -2 sum conj(u_i) u_i
-//   Phi_k = [conj(q) u_k + conj(2 u_i u_k) u_i] - [conj(u_k) q + conj(u_i) 2 u_i u_k]
-//   psi_k = [conj(q) u_k - conj(2 u_i u_k) u_i - conj(4 p) u_k] / 2
-//         + [conj(u_k) q - conj(u_i) 2 u_i u_k - conj(u_k) 4 p] / 2
-//   xi    = conj(u_a) w_a + conj(w_a) u_a
-// (add_job's sums; the mean gradients of xi ride on w_a).  Five terms let the
-// sum of order 7 reach 2^24.2: its rounding is below 2^-64 of the largest product.
+//   Phi_x = [conj(q) u + conj(2 u_i u) u_i] - [conj(u) q + conj(u_i) 2 u_i u]
+//   Phi_k = Q1 + X1 - Q2 - X2, psi_k = (R1 + R2 - X1 - X2) / 2 (k = y, z),
+//           Q1 = conj(q) u_k, Q2 = conj(u_k) q, R1 = conj(q - 4 p) u_k, R2 = conj(u_k) (q - 4 p),
+//           X1 = conj(2 u_i u_k) u_i, X2 = conj(u_i) 2 u_i u_k
+//   xi    = conj(u_a) w_a + conj(w_a) u_a, w_a = 2 sum_b d_b U_a u_b, b = y, z
+// (add_job's sums; the mean gradients of xi ride on w_a).  Fields that are added share
+// an exponent group (u, v, w; q with 2 u_i u; 2 u_i v; 2 u_i w; w_a); v, w, q and q - 4 p also
+// stand alone.  v and w vanish faster than u at their walls, so Q and X of Phi_y and Phi_z
+// stay apart: between two points near a wall no term of their sum would reach
+// exponents shared with q u.
 // A first part (and every part of the snapshot groups before the last) waits
 // in its spectrum; the last brings the snapshot average,
 // the one-point parts at m = 0 and the mean-flow couplings of finish_pair.
@@ -767,10 +769,19 @@ k1_correlate_strip(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int co
 // the SM's FP64 pipe.  k1_finish then brings the mean-flow couplings.  With
 // the couplings in the epilogue the stage took 44.1 ms at 256 x 33 x 33.
 //   Correlate stage (us, k1_correlate -> here), 16 snapshots: 256 x 33 x 33
-// 333880 -> 28984 (k1_finish 4750 of it); no size tried keeps the FMA kernel (nx = 8, 25 points, 1 snapshot
-// 356 -> 188).  Errors against 64-bit references are a few percent below its
-// own.  Bound by the MMAs (53 terms x 36 digit pairs a tile: 14 ms).
-enum DigitKind { DK_PART = 1, DK_SECOND = 2 };
+// 333880 -> 34204 (k1_finish 4760 of it, the marked values of m = 0 1850); no size tried keeps the
+// FMA kernel (nx = 8, 25 points, 1 snapshot 356 -> 188).  Bound by the epilogue and the L2
+// reductions; the MMAs (37 terms x 36 digit pairs a tile) take 10 ms by count.
+// (Q, X and 4 p in joint sums of five terms took 28984, but lost what lies far below q u.)
+// x / 2, or -x / 2, by the exponent (a multiplication would run on the FP64 pipe)
+static __device__ __noinline__ double half_edge(double x) { return 0.5 * x; }
+__device__ __forceinline__ double half(double x, int neg)
+{
+    const int hi = __double2hiint(x), e = hi & 0x7ff00000;
+    double h = __hiloint2double(hi - 0x00100000, __double2loint(x));
+    if (e <= 0x00100000 || e == 0x7ff00000) h = half_edge(x);
+    return __hiloint2double(__double2hiint(h) ^ neg, __double2loint(h));
+}
 struct DuctOut {
     zd* spec;
     long long npair;
@@ -779,17 +790,26 @@ struct DuctOut {
     {
         if (q1 >= P || q2 + 3 < q1 || q2 >= P) return;
         // row pointer at column q2 (pairs from q2 >= q1 on are stored)
-        zd* dst = spec + ((long long)job.out * nxh + m0 + k) * npair + tri(q1, q2, P);
-        const bool add = !first || job.kind == DK_SECOND;
+        const long long ts = (long long)nxh * npair;
+        zd* dst = spec + (long long)job.out * ts + (long long)(m0 + k) * npair + tri(q1, q2, P);
+        const bool add = !first || (job.kind & gke::DJ_ADD);
         #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (q2 + j < q1 || q2 + j >= P) continue;
             if (!add) dst[j] = o[j];
-            else {
-                asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(&dst[j].x), "d"(o[j].x) : "memory");
-                asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(&dst[j].y), "d"(o[j].y) : "memory");
-            }
+            else red_add(&dst[j], o[j]);
         }
+        if (job.out2 < 0) return;
+        dst += (long long)(job.out2 - job.out) * ts;
+        const int neg = job.half < 0 ? (int)0x80000000 : 0;
+        #pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (q2 + j >= q1 && q2 + j < P) red_add(&dst[j], mk(half(o[j].x, neg), half(o[j].y, neg)));
+    }
+    static __device__ __forceinline__ void red_add(zd* p, zd v)
+    {
+        asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(&p->x), "d"(v.x) : "memory");
+        asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(&p->y), "d"(v.y) : "memory");
     }
 };
 
@@ -851,12 +871,12 @@ k1_finish(zd* __restrict__ spec, const int* __restrict__ pq, long long npair, in
     }
 }
 
-// fields of the digit operands
-enum { D_U = 0, D_V, D_W, D_Q, D_UU, D_UV, D_UW, D_VV, D_VW, D_WW, D_W0, D_W1, D_W2, D_QP, D_UVP, D_UWP, D_VVP, D_VWP,
-       D_WWP, D_P4, ND };
-constexpr int ND_GRP = 4;
+// digit operands (A and B alike) and their exponent groups
+enum { D_V = 0, D_V1 = 3, D_W1, D_Q1, D_R1, D_PX, D_PY = D_PX + 4, D_PZ = D_PY + 3, D_WA = D_PZ + 3, ND = D_WA + 3 };
+enum { DG_V = 0, DG_V1, DG_W1, DG_Q1, DG_R1, DG_PX, DG_PY, DG_PZ, DG_WA, ND_GRP };
+constexpr int ND_JOB = 17;
 static gke::DgShape digit_shape(int P) { return gke::dg_shape(P, false); }
-static size_t digit_bytes(int P) { return gke::dg_bytes_per_k(digit_shape(P), ND, ND, ND_GRP); }
+static size_t digit_bytes(int P) { return gke::dg_bytes_per_k(digit_shape(P), ND, ND, ND_GRP, ND_JOB, true); }
 
 // the contractions of all wavenumbers into the spectra; kernels launched
 static int digit_correlate(gke::DigitWork& w, const zd* X, int ns, int P, int nx, double kx0, double nu,
@@ -866,73 +886,77 @@ static int digit_correlate(gke::DigitWork& w, const zd* X, int ns, int P, int nx
     const int nxh = nx / 2 + 1;
     gke::DgPrep p{};
     gke::DgArgs a{};
-    gke::dg_init(p, a, digit_shape(P), ND, ND, ND_GRP, true, w.err);
-    auto field = [&](int d, int src, int wexp, int grp) {
-        gke::DgField& f = p.f[p.nf++];
-        f.src = (short)src; f.src2 = -1; f.wexp = (signed char)wexp; f.grp = (signed char)grp;
-        f.ia = f.ib = (short)d;
-    };
-    for (int i = 0; i < 3; ++i) field(D_U + i, G_U + i, 0, 0);
-    field(D_Q, G_Q, 0, 1);
-    for (int i = 0; i < 6; ++i) field(D_UU + i, G_UU + i, 1, 1);
+    gke::dg_init(p, a, digit_shape(P), ND, ND, ND_GRP, true, X, nxh, ns, w.err);
+    auto field = [&](int d, int grp, int src, int wexp) -> gke::DgField& { return gke::dg_field(p, a, grp, src, d, d, wexp); };
+    for (int i = 0; i < 3; ++i) field(D_V + i, DG_V, G_U + i, 0);
+    field(D_V1, DG_V1, G_V, 0);
+    field(D_W1, DG_W1, G_W, 0);
+    field(D_Q1, DG_Q1, G_Q, 0);
+    {
+        gke::DgField& f = field(D_R1, DG_R1, G_Q, 0);
+        f.src2 = G_P;
+        f.w2 = -4.f;
+    }
     for (int i = 0; i < 3; ++i) {
-        field(D_W0 + i, G_V, 1, 2);
-        gke::DgField& f = p.f[p.nf - 1];
+        field(D_PX + i, DG_PX, prod_field(i, 0), 1);
+        field(D_PY + i, DG_PY, prod_field(i, 1), 1);
+        field(D_PZ + i, DG_PZ, prod_field(i, 2), 1);
+        gke::DgField& f = field(D_WA + i, DG_WA, G_V, 1);
         f.src2 = G_W;
         f.c = prof + (long long)(R_G + 2 * i) * P;
         f.c2 = prof + (long long)(R_G + 2 * i + 1) * P;
     }
-    field(D_QP, G_Q, 0, 3);
-    const int pr[5] = {G_UV, G_UW, G_VV, G_VW, G_WW};
-    for (int i = 0; i < 5; ++i) field(D_UVP + i, pr[i], 1, 3);
-    field(D_P4, G_P, 2, 3);
-    p.X = X; p.nsX = ns; p.Nk = nxh;
+    field(D_PX + 3, DG_PX, G_Q, 0);
 
     // the snapshot average: a power of two goes into the digits' exponents
     const bool pow2 = (ns & (ns - 1)) == 0;
     const int se = pow2 ? -gke::ilog2(ns) : 0;
     std::vector<std::vector<gke::HostTerm>> terms;
-    auto job = [&](int out, int kind, int ga, int gb, int e, std::vector<gke::HostTerm> v) {
+    auto job = [&](int out, int add, int ga, int gb, int e, std::vector<gke::HostTerm> v, int out2 = -1, int half = 0) {
         gke::DgJob& j = a.job[a.njob++];
-        j.ga = (signed char)ga; j.gb = (signed char)gb; j.out = (signed char)out; j.kind = (signed char)kind;
-        j.e = -34 + e + se;
+        j.ga = (signed char)ga; j.gb = (signed char)gb; j.out = (signed char)out;
+        j.kind = (signed char)(add ? gke::DJ_ADD : 0);
+        j.out2 = (signed char)out2; j.half = (signed char)half;
+        j.ex = (short)(e + se);
         terms.push_back(std::move(v));
     };
-    const int pair[3][3] = {{D_UU, D_UV, D_UW}, {D_UV, D_VV, D_VW}, {D_UW, D_VW, D_WW}};
-    const int pairp[3][3] = {{-1, D_UVP, D_UWP}, {D_UVP, D_VVP, D_VWP}, {D_UWP, D_VWP, D_WWP}};
-    job(A_A, 0, 0, 0, 1, {{D_U, D_U, true}, {D_V, D_V, true}, {D_W, D_W, true}});
-    for (int k = 0; k < 3; ++k) {
-        std::vector<gke::HostTerm> f{{D_Q, k, false}}, b{{k, D_Q, true}};
-        for (int i = 0; i < 3; ++i) {
-            f.push_back({pair[i][k], i, false});
-            b.push_back({i, pair[i][k], true});
-        }
-        job(A_PHIX + k, DK_PART, 1, 0, 0, f);
-        job(A_PHIX + k, DK_SECOND, 0, 1, 0, b);
+    // three terms of a group a with u, v, w (and q u): A role, B role of the group
+    auto front = [](int d, int n) {
+        std::vector<gke::HostTerm> v;
+        for (int i = 0; i < n; ++i) v.push_back({d + i, D_V + i % 3, false});
+        return v;
+    };
+    auto back = [](int d, int n, bool neg) {
+        std::vector<gke::HostTerm> v;
+        for (int i = 0; i < n; ++i) v.push_back({D_V + i % 3, d + i, neg});
+        return v;
+    };
+    // long and short alternate; a spectrum's first part is stored before the others are added
+    job(A_A, 0, DG_V, DG_V, 1, back(D_V, 3, true));
+    for (int k = 0; k < 2; ++k) {
+        const int u = k ? D_W1 : D_V1, gu = k ? DG_W1 : DG_V1, pk = k ? D_PZ : D_PY, gp = k ? DG_PZ : DG_PY;
+        const int phi = A_PHIY + k, psi = A_PSIY + k;
+        job(phi, 0, DG_Q1, gu, 0, {{D_Q1, u, false}});
+        if (k == 0) job(A_PHIX, 0, DG_PX, DG_V, 0, front(D_PX, 4));
+        else job(A_XI, 0, DG_V, DG_WA, 0, back(D_WA, 3, false));
+        job(psi, 0, DG_R1, gu, -1, {{D_R1, u, false}});
+        job(phi, 1, gp, DG_V, 0, front(pk, 3), psi, -1);
+        job(phi, 1, gu, DG_Q1, 0, {{u, D_Q1, true}});
+        if (k == 0) job(A_PHIX, 1, DG_V, DG_PX, 0, back(D_PX, 4, true));
+        else job(A_XI, 1, DG_WA, DG_V, 0, front(D_WA, 3));
+        job(psi, 1, gu, DG_R1, -1, {{u, D_R1, false}});
+        job(phi, 1, DG_V, gp, 0, back(pk, 3, true), psi, 1);
     }
-    for (int k = 1; k < 3; ++k) {
-        std::vector<gke::HostTerm> f{{D_QP, k, false}, {D_P4, k, true}}, b{{k, D_QP, false}, {k, D_P4, true}};
-        for (int i = 0; i < 3; ++i) {
-            f.push_back({pairp[i][k], i, true});
-            b.push_back({i, pairp[i][k], true});
-        }
-        job(A_PSIY + k - 1, DK_PART, 3, 0, -1, f);
-        job(A_PSIY + k - 1, DK_SECOND, 0, 3, -1, b);
-    }
-    job(A_XI, DK_PART, 0, 2, 0, {{D_U, D_W0, false}, {D_V, D_W1, false}, {D_W, D_W2, false}});
-    job(A_XI, DK_SECOND, 2, 0, 0, {{D_W0, D_U, false}, {D_W1, D_V, false}, {D_W2, D_W, false}});
     gke::dg_schedule(a, terms);
     const int kmax = (int)std::min<size_t>((size_t)nxh, w.bytes / digit_bytes(P));
     int launches = 0;
     for (int m0 = 0; m0 < nxh; m0 += kmax) {
         const int nk = std::min(kmax, nxh - m0);
-        gke::dg_place(p, a, w.ws, nk);
-        p.k0 = m0;
+        gke::dg_place(p, a, w.ws, m0, nk);
         for (int s0 = 0; s0 < ns; s0 += gke::DG_KS) {
-            p.s0 = s0;
-            p.ns = std::min(gke::DG_KS, ns - s0);
+            gke::dg_batch(p, a, s0, std::min(gke::DG_KS, ns - s0));
             gke::dg_pass(p, a, nk, DuctOut{spec, npair, P, nxh, m0, s0 == 0}, st);
-            launches += 2;
+            launches += 3;
         }
     }
     k1_finish<<<dim3((unsigned)((npair + 255) / 256), (unsigned)((nxh + FIN_MB - 1) / FIN_MB)), 256, 0, st>>>(

@@ -2,18 +2,18 @@
 // (gke_digits.cuh has the method).
 //
 // Measured, correlate stage (operands, contractions; FMA kernel -> here):
-// 256 x 256 x 65, 16 snapshots 232.8 -> 34.7 ms, of which the operand kernel 6.5
+// 256 x 256 x 65, 16 snapshots 232.8 -> 39.5 ms, of which the operand kernel 8.7
 // and the MMAs alone 23 (smem reads of A and B: 18.5 by count), which bound it
 // with the epilogue (conversions and integer adds) close behind; 128 x 128 x 65,
-// 32 snapshots 117.4 -> 18.6 ms.  Errors against 64-bit references equal the
-// FMA kernel's or are below.
+// 32 snapshots 117.4 -> 21.5 ms.  (One exponent per row for u, v, w and one for all
+// products took 34.7 and 18.6 ms, but held v and w at the size of u.)
 #include "gke_digits.h"
 #include "gke_digits.cuh"
 #include "gke_kernels.h"
 
 namespace gke {
 
-// raw[job][y / 8][y' / 8][k][8][8] (raw_index); beta adds to what is there
+// raw[job][y / 8][y' / 8][k][8][8] (raw_index); beta, or a job's DJ_ADD, adds to what is there
 struct RawOut {
     zd* raw;
     int n, Kc, beta;
@@ -22,7 +22,7 @@ struct RawOut {
         const int YB = (n + 7) / 8;
         if (yp >= 8 * YB) return;
         zd* dst = raw + raw_index(job.out, k, y, yp, Kc, YB);
-        if (beta) {
+        if (beta || (job.kind & DJ_ADD)) {
             #pragma unroll
             for (int j = 0; j < 4; ++j) o[j] = o[j] + dst[j];
         }
@@ -34,7 +34,6 @@ struct RawOut {
 // Rows y in [cov, ny) of grids with a thin remainder past the last 128-row
 // tile (the Chebyshev grids ny = 128 m + 1): a tile of their own would cost as
 // much as a full one.  FP64 FMA chains, CTA = one wavenumber and row, thread = y'.
-constexpr int DG_MAXT = 4;
 struct DgRowJob { int nt, out; int fa[DG_MAXT], fb[DG_MAXT]; };
 struct DgRows { int njob; DgRowJob job[NJOB]; };
 __global__ void __launch_bounds__(160)
@@ -75,10 +74,45 @@ static const HostJob kJobs[NJOB] = {
     /* D  */ {3, {F_U, F_V, F_W}, {F_U, F_V, F_W}},
 };
 
-// channel: 11 A fields, 3 B fields, 3 exponent groups
-constexpr int CH_NFA = 11, CH_NFB = 3, CH_NGRP = 3;
+// The operands.  Fields that are added share a group: u, v, w; q with the products
+// of u; the products of v and of w, which fall faster towards a wall than q.  u, v and w
+// also stand alone, for the contractions of one term, so that those are exact to the
+// size of the smaller field (q of <q v'> and <q w'> is nearly always of its group's size).
+// GZ is q w and the products of w apart: with a w far below u no term of a joint sum
+// would reach the shared exponents.
+enum { CG_V = 0, CG_U1, CG_P1, CG_V1, CG_W1, CG_PX, CG_PY, CG_PZ, CH_NGRP };
+constexpr int CH_NFA = 15, CH_NFB = 5;
+static void channel_fields(DgPrep& p, DgArgs& a)
+{
+    for (int i = 0; i < 3; ++i) dg_field(p, a, CG_V, F_U + i, i, i);
+    dg_field(p, a, CG_U1, F_U, 3, -1);
+    dg_field(p, a, CG_P1, F_P, 4, -1);
+    dg_field(p, a, CG_V1, F_V, -1, 3);
+    dg_field(p, a, CG_W1, F_W, -1, 4);
+    static const int px[] = {F_UU, F_UV, F_UW, F_Q}, py[] = {F_UV, F_VV, F_VW}, pz[] = {F_UW, F_VW, F_WW};
+    for (int i = 0; i < 4; ++i) dg_field(p, a, CG_PX, px[i], 5 + i, -1);
+    for (int i = 0; i < 3; ++i) dg_field(p, a, CG_PY, py[i], 9 + i, -1);
+    for (int i = 0; i < 3; ++i) dg_field(p, a, CG_PZ, pz[i], 12 + i, -1);
+}
+// contractions (operand indices); the second of GZ is added to the first.  Long and
+// short alternate: the epilogue of a one-term contraction takes longer than its
+// MMAs, that of a four-term one less.
+struct DigitJob { int out, kind, ga, gb, sa, nt, fa[DG_MAXT], fb[DG_MAXT]; };
+static const DigitJob kDigitJobs[] = {
+    {J_GX, 0, CG_PX, CG_V, 0, 4, {5, 6, 7, 8}, {0, 1, 2, 0}},
+    {J_GZ, 0, CG_PX, CG_W1, 12, 1, {8}, {4}},
+    {J_D, 0, CG_V, CG_V, 0, 3, {0, 1, 2}, {0, 1, 2}},
+    {J_E, 0, CG_U1, CG_V1, 0, 1, {3}, {3}},
+    {J_GZ, DJ_ADD, CG_PZ, CG_V, 0, 3, {12, 13, 14}, {0, 1, 2}},
+    {J_F, 0, CG_P1, CG_V1, 0, 1, {4}, {3}},
+    {J_X, 0, CG_PY, CG_V, 0, 3, {9, 10, 11}, {0, 1, 2}},
+    {J_QV, 0, CG_PX, CG_V1, 12, 1, {8}, {3}},
+};
 
-size_t digits_per_k(int n) { return dg_bytes_per_k(dg_shape(n, true), CH_NFA, CH_NFB, CH_NGRP); }
+size_t digits_per_k(int n)
+{
+    return dg_bytes_per_k(dg_shape(n, true), CH_NFA, CH_NFB, CH_NGRP, (int)(sizeof(kDigitJobs) / sizeof(kDigitJobs[0])), false);
+}
 
 void digits_alloc(DigitWork& w, size_t per, int Kc, cudaStream_t st, size_t limit)
 {
@@ -115,51 +149,37 @@ gke_status digits_correlate(DigitWork& w, const zd* Xop, int ns, int ny, int Nk,
     DgPrep p{};
     DgArgs a{};
     const DgShape s = dg_shape(ny, true);
-    dg_init(p, a, s, CH_NFA, CH_NFB, CH_NGRP, false, w.err);
+    dg_init(p, a, s, CH_NFA, CH_NFB, CH_NGRP, false, Xop, Nk, ns, w.err);
+    channel_fields(p, a);
     const int kmax = (int)std::min<size_t>((size_t)Kc, w.bytes / digits_per_k(ny));
-    for (int f = 0; f < NFIELD; ++f) {
-        DgField& d = p.f[p.nf++];
-        d.src = (short)f;
-        d.src2 = -1;
-        d.grp = f <= F_W ? 0 : f == F_P ? 1 : 2;
-        d.ia = (short)f;
-        d.ib = (short)(f <= F_W ? f : -1);
-    }
-    p.X = Xop; p.nsX = ns; p.Nk = Nk;
     std::vector<std::vector<HostTerm>> terms;
-    DgRows rows{};
-    // long and short contractions alternate: the epilogue of a one-term job
-    // takes longer than its MMAs, that of a four-term job less
-    static const int order[NJOB] = {J_GX, J_E, J_GZ, J_F, J_X, J_QV, J_D};
-    for (int j : order) {
-        if (!((jobs >> j) & 1u)) continue;
-        const HostJob& h = kJobs[j];
+    for (const DigitJob& h : kDigitJobs) {
+        if (!((jobs >> h.out) & 1u)) continue;
         std::vector<HostTerm> v;
-        DgRowJob& rj = rows.job[rows.njob++];
-        rj.nt = h.nt; rj.out = j;
-        for (int t = 0; t < h.nt; ++t) {
-            v.push_back({h.fa[t], h.fb[t], false});
-            rj.fa[t] = h.fa[t]; rj.fb[t] = h.fb[t];
-        }
+        for (int t = 0; t < h.nt; ++t) v.push_back({h.fa[t], h.fb[t], false});
         terms.push_back(v);
         DgJob& d = a.job[a.njob++];
-        d.ga = (signed char)(h.fa[0] <= F_W ? 0 : h.fa[0] == F_P ? 1 : 2);
-        d.gb = 0;
-        d.out = (signed char)j;
-        d.e = -34;
+        d.ga = (signed char)h.ga; d.gb = (signed char)h.gb; d.sa = (unsigned char)h.sa;
+        d.out = (signed char)h.out; d.kind = (signed char)h.kind; d.out2 = -1;
+    }
+    DgRows rows{};
+    for (int j = 0; j < NJOB; ++j) {
+        if (!((jobs >> j) & 1u)) continue;
+        const HostJob& h = kJobs[j];
+        DgRowJob& rj = rows.job[rows.njob++];
+        rj.nt = h.nt; rj.out = j;
+        for (int t = 0; t < h.nt; ++t) { rj.fa[t] = h.fa[t]; rj.fb[t] = h.fb[t]; }
     }
     if (!a.njob) return GKE_OK;
     dg_schedule(a, terms);
     for (int kc0 = 0; kc0 < Kc; kc0 += kmax) {
         const int nk = std::min(kmax, Kc - kc0);
-        dg_place(p, a, w.ws, nk);
-        p.k0 = k0 + kc0;
+        dg_place(p, a, w.ws, k0 + kc0, nk);
         for (int s0 = 0; s0 < ns; s0 += DG_KS) {
-            p.s0 = s0;
-            p.ns = std::min(DG_KS, ns - s0);
+            dg_batch(p, a, s0, std::min(DG_KS, ns - s0));
             // raw_index: the wavenumber's stride is 64
             dg_pass(p, a, nk, RawOut{raw + (size_t)kc0 * 64, ny, Kc, s0 > 0}, st);
-            *launches += 2;
+            *launches += 3;
         }
     }
     if (s.cov < ny) {

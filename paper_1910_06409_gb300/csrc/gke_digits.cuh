@@ -8,26 +8,43 @@
 // 4096 in FP16: the 36 digit products that replace one FP64 product below
 // still leave a factor of 50.
 //
-// Splitting.  All values of a row (wavenumber k, wall-normal point y) of one
-// group of fields -- velocities; products; pressure -- share the exponent E
-// of the largest of them over the batch's snapshots, |x| < 2^E.  Each value
-// becomes the integer round(x 2^(61 - E)) and that its eight balanced base-256
-// digits s_0 (|s_0| <= 33) .. s_7 (in [-128, 127]), exact in FP16.  61 bits
-// below the row's largest value hold every bit of an FP64 value down to
-// 2^-8 of that maximum; smaller values lose bits below 2^-61 of it, eight
-// binary orders under the FP64 rounding of the sums they enter.
+// Splitting.  The values of a row (wavenumber k, wall-normal point y) of the
+// fields of one exponent group share the exponent E of the largest of them over
+// the batch's snapshots, |x| < 2^E.  Each value becomes the integer
+// round(x 2^(61 - E)) and that its eight balanced base-256 digits s_0
+// (|s_0| <= 33) .. s_7 (in [-128, 127]), exact in FP16.
+//
+// Groups.  A field is held to 61 bits below its group's exponent, so a group
+// holds only fields whose products are added (at most four; a field of a
+// one-term contraction stands alone): v is not rounded at the size of u in
+// <u v'>, however small it is.  A sum of several terms has the accuracy of its
+// largest term only if that term is not itself far below the two groups'
+// exponents.  Each row carries how many bits each field of the group lies below
+// E (a nibble, 5 = more); where the nibbles of every term of a sum add up
+// to more than dg_lmax bits, or a row holds an infinity or a NaN, the epilogue leaves a
+// zero and a mark, and k_dg_far adds the value by FP64 FMAs from the fields: such
+// values cost what the FMA kernels cost, and are right for any input.
 //
 // Products.  With the digit products s_i t_j summed over the terms and
-// snapshots of a contraction by order d = i + j (v_d, d <= 7; the orders
-// above are below 2^-64 of the largest product),
+// snapshots of a contraction by order d = i + j (v_d, d <= 7),
 //   sum a b = 2^(E_a + E_b - 34) [ (v_0 .. v_3) + 2^-32 (v_4 .. v_7) ],
 //   (w_0 .. w_3) = 2^24 w_0 + 2^16 w_1 + 2^8 w_2 + w_3.
-// A sum v_d runs over at most 4 terms x 16 snapshots x 2 real products, so
+// The orders above 7 are left out: a product loses up to 2^-57 of 2^(E_a + E_b)
+// (seven digit products of order 8), 2^-60 typically.  A sum v_d runs over at most
+// 4 terms x 16 snapshots x 2 real products, so
 // |v_d| <= max(1, d) 4 2^19 < 2^24 (and < 2^22 for d <= 2, where s_0 enters every
-// or all but one product): the FP32 accumulation in tensor memory is exact.  The eight sums are joined in a 64-bit integer and rounded to FP64
+// or all but one product): the FP32 accumulation in tensor memory is exact.  A
+// batch of 16 / c snapshots or fewer takes its A digits times c = 2, 4, 8 or 16 (exact
+// in FP16), so the same bounds hold and the joined sum's unit is c times finer.  The
+// eight sums are joined in a 64-bit integer and rounded to FP64
 // once, all in integer arithmetic.  A sum over up to 16 snapshots therefore
 // carries one rounding where the FMA chain carries 32 per term; further
 // snapshots come in groups of 16, added in FP64.
+//
+// Error against exact sums, over the 2-norms of the operands (rms; emulated with
+// random operands; FMA chain): one term, 1 / 4 / 16 snapshots 4.7e-17 / 2.4e-17 /
+// 1.4e-17 (5.8e-17 / 5.0e-17 / 4.8e-17); at dg_lmax bits 5.5e-17 / 3.2e-17 / 3.0e-17; three and four
+// terms at their dg_lmax, 16 snapshots, 7.0e-17 and 1.4e-16 (1.25e-16 and 1.6e-16).
 //
 // Mapping.  CTA = one SM, persistent over items (k, 128-row tile of y, tile of
 // CW <= 32 columns y').  Per term and digit pair (i, j):
@@ -64,14 +81,28 @@ constexpr int dg_epi(int CW) { return CW / 2; }                    // epilogue w
 constexpr int dg_threads(int CW) { return 64 + 32 * dg_epi(CW); }
 constexpr int DG_SM_BAR = 512;             // barriers, then the B slots, then the A stages
 constexpr int DG_SM = 232448;
-constexpr int DG_MAXSTEP = 112, DG_MAXJOB = 16, DG_MAXF = 24, DG_MAXG = 4;
+constexpr int DG_MAXSTEP = 112, DG_MAXJOB = 20, DG_MAXF = 24, DG_MAXT = 4;
 
 enum { DF_NEG = 1, DF_LOAD = 2, DF_FREE = 4, DF_FIRST = 8, DF_LAST = 16, DF_HI = 32 };
 // one term of one pass: conj(A field fa) B field fb; B in slot, loaded before
 // (DF_LOAD) or released after it (DF_FREE)
 struct DgStep { unsigned char fa, fb, slot, flags; };
-// a contraction: exponent groups of its A and B fields, output index and kind, power of two
-struct DgJob { signed char ga, gb, out, kind; int e; };
+// a contraction: exponent groups of its A and B fields, output index and kind
+// (DJ_ADD: add to what is there) and a second output (psi: with the factor half / 2);
+// the value is 2^ex times the sum, 2^e times the joined digits' upper half.  Term t
+// goes with nibble t of the B row's distances and nibble t of the A row's
+// shifted by sa bits; first step of the schedule.
+enum { DJ_ADD = 1 };
+struct DgJob {
+    signed char ga, gb, out, kind, out2, half;
+    unsigned char sa, nt, step;
+    short e, ex;
+    unsigned short add, mask;
+};
+// bits that every term of a sum of nt terms may lie below its rows' exponents:
+// up to there the digits' error stays under the FMA chain's (header)
+__host__ __device__ constexpr int dg_lmax(int nt, int ns) { return nt == 1 ? (ns == 1 ? 3 : 2) : nt < 4 ? 3 : 4; }
+constexpr int DG_FAR = 5;                                   // nibble of a field further below, or not finite
 
 struct DgBars {
     uint64_t full[DG_MAXST], empty[DG_MAXST], bfull[DG_NB], bempty[DG_NB], acc_full[2], acc_empty[2], drain;
@@ -84,6 +115,17 @@ struct DgShape {
     int n, RT, MT, cov, NT, CW, nrow;      // rows per A tile, A tiles, rows they cover, column tiles, E rows
 };
 
+// a field as the operands hold it: X_src times 2^wexp, or for src2 >= 0 the
+// combination c X_src + c2 X_src2 (coefficient rows of n values), without c
+// X_src + w2 X_src2; exponent group, A and B operand index (-1: not used)
+struct DgField { short src, src2, ia, ib; signed char wexp, grp; float w2; const double* c; const double* c2; };
+// the fields [src][k][s][y] of a batch of ns snapshots from s0 on
+struct DgSrc {
+    const zd* X;
+    int n, s0, ns, nsX, Nk, k0, nf;
+    DgField f[DG_MAXF];
+};
+
 struct DgArgs {
     const __half* Aop; const __half* Bop; const int* E;
     DgShape s;
@@ -93,6 +135,9 @@ struct DgArgs {
     int nstep, njob;
     DgStep step[DG_MAXSTEP];
     DgJob job[DG_MAXJOB];
+    unsigned char af[DG_MAXF], bf[DG_MAXF];   // operand -> field of src
+    DgSrc src;
+    unsigned* far;                         // [item][contraction]: marks of a warp's 32 rows x 4 columns (dg_mark)
     int mul[4];                            // 2^5, 2^13, 2^21, 2^29 (mad_wide)
     int* err;
 };
@@ -130,28 +175,26 @@ inline size_t dg_a_halves(const DgShape& s) { return (size_t)s.MT * DG_S * 2 * s
 inline size_t dg_b_halves(const DgShape& s) { return (size_t)s.NT * DG_S * 3 * s.CW * DG_KS; }
 
 // ------------------------------------------------------------- digit operands
-// field src of X (times 2^wexp), or for src2 >= 0 the combination
-// c[src] X_src + c[src2] X_src2 with coefficient rows c of n values; exponent
-// group, A and B operand index (-1: not used)
-struct DgField { short src, src2; signed char wexp, grp; short ia, ib; const double* c; const double* c2; };
 struct DgPrep {
     DgShape s;
-    int nf, nfa, nfb, ngrp, ns, s0, nsX, Nk, k0;
-    DgField f[DG_MAXF];
-    const zd* X;
+    int nfa, nfb, ngrp, cexp;              // cexp: the A digits carry the factor 2^cexp
+    DgSrc src;
     __half* Aop; __half* Bop; int* E;
+    unsigned* far; long long nfar;         // marks to clear
 };
-__device__ __forceinline__ zd dg_load(const DgPrep& a, const DgField& fd, int k, int s, int y)
+// without 2^wexp
+__device__ __forceinline__ zd dg_load(const DgSrc& a, const DgField& fd, int k, int s, int y)
 {
-    const long long o = ((long long)(a.k0 + k) * a.nsX + a.s0 + s) * a.s.n + y, fs = (long long)a.Nk * a.nsX * a.s.n;
+    const long long o = ((long long)(a.k0 + k) * a.nsX + a.s0 + s) * a.n + y, fs = (long long)a.Nk * a.nsX * a.n;
     const zd v = a.X[fd.src * fs + o];
     if (fd.src2 < 0) return v;
     const zd w = a.X[fd.src2 * fs + o];
+    if (!fd.c) return mk(fma((double)fd.w2, w.x, v.x), fma((double)fd.w2, w.y, v.y));
     const double p = fd.c[y], q = fd.c2[y];
     return mk(p * v.x + q * w.x, p * v.y + q * w.y);
 }
 
-constexpr int DG_NAN = 8192;                                // exponent of a row with an infinity or a NaN
+constexpr int DG_NAN = 8192;                                // exponent of a group's row with an infinity or a NaN
 
 // round(x 2^sh) for |x| 2^sh < 2^61, in integer arithmetic (a conversion would
 // run on the FP64 pipe)
@@ -180,50 +223,66 @@ __device__ __forceinline__ uint32_t dg_pair(uint32_t a, uint32_t b, int c)
     return *(const uint32_t*)&h;
 }
 
-// CTA = one (wavenumber, exponent group, 128 rows): the rows' exponents, then
-// the digit blocks of the group's fields.  Thread = one row x 8 snapshots, the
-// 16 bytes of a core-matrix row; stores are contiguous over the rows.  Bound by
-// memory: X is read twice (the second time from L2), 32 bytes of digits are
-// written per A value.
-static __global__ void __launch_bounds__(256)
+// CTA = one (wavenumber, exponent group, 128 rows): the rows' exponents with the
+// fields' distances below them, then the digit blocks of the group's fields.
+// Thread = one row x 8 snapshots, the 16 bytes of a core-matrix row; stores are contiguous over the rows.
+// Bound by memory: X is read twice (the second time from L2), 32 bytes of digits are
+// written per A value (256 x 256 x 65, 16 snapshots: 8.7 ms; with three CTAs an SM 9.2).
+static __global__ void __launch_bounds__(256, 4)
 k_dg_prep(const __grid_constant__ DgPrep a)
 {
-    __shared__ unsigned s_hi[128];
+    __shared__ unsigned s_hi[DG_MAXT][128];
+    const DgSrc& x = a.src;
     const int nb = a.s.nrow / 128;
     int b = blockIdx.x;
     const int mb = b % nb; b /= nb;
     const int g = b % a.ngrp, k = b / a.ngrp;
     const int r = threadIdx.x & 127, kc = threadIdx.x >> 7;
     const int y = mb * 128 + r;
-    if (threadIdx.x < 128) s_hi[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < DG_MAXT * 128; i += 256) (&s_hi[0][0])[i] = 0;
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < a.nfar; i += gridDim.x * 256ll) a.far[i] = 0;
     __syncthreads();
-    const int e0 = kc * 8, ne = y < a.s.n ? max(0, min(8, a.ns - e0)) : 0;
-    unsigned hi = 0;
-    for (int f = 0; f < a.nf; ++f) {
-        const DgField fd = a.f[f];
+    const int e0 = kc * 8, ne = y < a.s.n ? max(0, min(8, x.ns - e0)) : 0;
+    int nm = 0;                                             // fields of the group
+    for (int f = 0; f < x.nf; ++f) {
+        const DgField& fd = x.f[f];
         if (fd.grp != g) continue;
+        unsigned hi = 0;
         for (int e = 0; e < ne; ++e) {
-            const zd v = dg_load(a, fd, k, e0 + e, y);
+            const zd v = dg_load(x, fd, k, e0 + e, y);
             // (unsigned: an infinity or a NaN times 2^wexp stays above 0x7ff00000)
             const unsigned h = (unsigned)max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
             if (h >= 0x00100000u) hi = max(hi, h + fd.wexp * 0x00100000u);
         }
+        atomicMax(&s_hi[nm++][r], hi);
     }
-    atomicMax(&s_hi[r], hi);
     __syncthreads();
-    const int E = s_hi[r] >= 0x7ff00000u ? DG_NAN : max((int)(s_hi[r] >> 20), 1) - 1022;              // |x| < 2^E
-    if (kc == 0) a.E[((long long)k * a.ngrp + g) * a.s.nrow + y] = E;
+    int E = -1021;
+    for (int i = 0; i < nm; ++i) {
+        const unsigned h = s_hi[i][r];
+        E = max(E, h >= 0x7ff00000u ? DG_NAN : (int)(h >> 20) - 1022);                      // |x| < 2^E
+    }
+    if (kc == 0) {
+        // (three fields: the fourth nibble repeats the first's, for a fourth term with the first field)
+        unsigned far = 0;
+        for (int i = 0; i < DG_MAXT; ++i) {
+            const unsigned h = s_hi[i < nm ? i : 0][r];
+            far |= (unsigned)(E == DG_NAN ? DG_FAR : min(E - max((int)(h >> 20) - 1022, -1021), DG_FAR)) << (4 * i);
+        }
+        a.E[((long long)k * a.ngrp + g) * a.s.nrow + y] = (int)((far << 16) | (unsigned)(E & 0xffff));
+    }
+    const __half2 cs = __half2half2(__int2half_rn(1 << a.cexp));
     const bool arow = mb < a.s.MT && r < a.s.RT && y < a.s.cov, astore = mb < a.s.MT && r < a.s.RT;
     const int c = y / a.s.CW, rc = y - c * a.s.CW;
     const bool bstore = c < a.s.NT;
-    for (int f = 0; f < a.nf; ++f) {
-        const DgField fd = a.f[f];
+    for (int f = 0; f < x.nf; ++f) {
+        const DgField& fd = x.f[f];
         if (fd.grp != g) continue;
         unsigned long long dre[8], dim[8];
         #pragma unroll
         for (int e = 0; e < 8; ++e) {
             zd v = mk(0.0, 0.0);
-            if (e < ne) v = dg_load(a, fd, k, e0 + e, y);
+            if (e < ne) v = dg_load(x, fd, k, e0 + e, y);
             dre[e] = dg_bytes(dg_fixed(v.x, 61 - E + fd.wexp));
             dim[e] = dg_bytes(dg_fixed(v.y, 61 - E + fd.wexp));
         }
@@ -244,17 +303,24 @@ k_dg_prep(const __grid_constant__ DgPrep a)
                 pr[h] = dg_pair((uint32_t)(dre[2 * h] >> w), (uint32_t)(dre[2 * h + 1] >> w), cc);
                 pi[h] = dg_pair((uint32_t)(dim[2 * h] >> w), (uint32_t)(dim[2 * h + 1] >> w), cc);
             }
-            if (da) {
-                const uint4 z = make_uint4(0, 0, 0, 0);
-                *(uint4*)(da + (long long)(2 * i) * a.s.RT * DG_KS) = arow ? re : z;
-                *(uint4*)(da + (long long)(2 * i + 1) * a.s.RT * DG_KS) = arow ? im : z;
-            }
             if (db) {
                 __half* d = db + (long long)i * 3 * a.s.CW * DG_KS + b0;
                 *(uint4*)d = re;
                 *(uint4*)(d + bw) = im;
                 *(uint4*)(d + 2 * bw) = make_uint4(re.x ^ 0x80008000u, re.y ^ 0x80008000u, re.z ^ 0x80008000u,
                                                    re.w ^ 0x80008000u);
+            }
+            if (da) {
+                if (a.cexp) {
+                    #pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        *(__half2*)&pr[h] = __hmul2(*(__half2*)&pr[h], cs);
+                        *(__half2*)&pi[h] = __hmul2(*(__half2*)&pi[h], cs);
+                    }
+                }
+                const uint4 z = make_uint4(0, 0, 0, 0);
+                *(uint4*)(da + (long long)(2 * i) * a.s.RT * DG_KS) = arow ? re : z;
+                *(uint4*)(da + (long long)(2 * i + 1) * a.s.RT * DG_KS) = arow ? im : z;
             }
         }
     }
@@ -316,11 +382,8 @@ __device__ __forceinline__ long long dg_high(const uint32_t (&r)[4][4], int j, l
     const unsigned up = (unsigned)((unsigned long long)v >> 32) + (bits(0) << 13) + (bits(1) << 5);
     return (long long)(((unsigned long long)up << 32) | (unsigned)v);
 }
-// t 2^(e - 21) in general; NaN where an operand row holds an infinity or a NaN
-static __device__ __noinline__ double dg_value_edge(long long t, int e)
-{
-    return e > DG_NAN / 2 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)t, e - 21);
-}
+// t 2^(e - 21) in general
+static __device__ __noinline__ double dg_value_edge(long long t, int e) { return scalbn((double)t, e - 21); }
 // t 2^(e - 21), normalised and rounded to nearest in integer arithmetic (a
 // conversion would hold the FP64 pipe of the whole SM for 16 clocks a warp).
 // No branch, so that values interleave; edge is raised where the upper
@@ -345,6 +408,15 @@ __device__ __forceinline__ void st_256(zd* p, zd a, zd b)
 {
     asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a.x), "d"(a.y), "d"(b.x), "d"(b.y) : "memory");
 }
+
+// every term of a contraction too far below its rows' exponents: words wa, wb of the A and B row
+// (no nibble overflows: 5 + 5 + 5)
+__device__ __forceinline__ bool dg_far(const DgJob& job, int wa, int wb)
+{
+    return ((((unsigned)wa >> 16 >> job.sa) + ((unsigned)wb >> 16) + job.add) & job.mask) == job.mask;
+}
+// bit of the mark of a warp's four columns: TMEM lane quarter, 8-column part, 4-column group
+__device__ __forceinline__ int dg_mark(int q, int part, int g) { return (part * 4 + q) * 2 + g; }
 
 struct DgItem { int k, mt, c; };
 __device__ __forceinline__ DgItem dg_item(const DgArgs& a, long long it)
@@ -502,38 +574,28 @@ k_dg_corr(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
         uint32_t aph = 0;
         const int m5 = a.mul[0], m13 = a.mul[1], m21 = a.mul[2], m29 = a.mul[3];
         const int r = q * 32 + lane;
-        // exponents of an item: this row's, and lane j's column c0 + j, per
-        // group; loaded an item ahead
-        int ea[DG_MAXG], eb[DG_MAXG], na[DG_MAXG], nb[DG_MAXG];
-        auto exponents = [&](long long it) {
-            const DgItem u = dg_item(a, min(it, a.nitems - 1));
-            #pragma unroll
-            for (int g = 0; g < DG_MAXG; ++g) {
-                const int* Eg = a.E + ((long long)u.k * a.ngrp + min(g, a.ngrp - 1)) * a.s.nrow;
-                na[g] = Eg[min(u.mt * RT + r, a.s.nrow - 1)];
-                nb[g] = Eg[u.c * CW + part * HC + (lane & (HC - 1))];
-            }
+        // exponents and distances of a contraction: this row's, and of lane j's column
+        // c0 + j; loaded a contraction ahead
+        int na, nb;
+        auto fetch = [&](const DgItem& u, const DgJob& job) {
+            const int* E = a.E + (long long)u.k * a.ngrp * a.s.nrow;
+            na = E[job.ga * a.s.nrow + min(u.mt * RT + r, a.s.nrow - 1)];
+            nb = E[job.gb * a.s.nrow + u.c * CW + part * HC + (lane & (HC - 1))];
         };
-        exponents(blockIdx.x);
+        DgItem u = dg_item(a, min((long long)blockIdx.x, a.nitems - 1));
+        fetch(u, a.job[0]);
         for (long long it = blockIdx.x; it < a.nitems && !*abort; it += gridDim.x) {
-            const DgItem u = dg_item(a, it);
+            const DgItem next = dg_item(a, min(it + gridDim.x, a.nitems - 1));
             const int y = u.mt * RT + r, c0 = u.c * CW + part * HC;
             const bool live = q * 32 < RT && u.mt * RT + q * 32 < a.s.cov;    // uniform over the warp
             const bool row = r < RT && y < a.s.cov;
-            #pragma unroll
-            for (int g = 0; g < DG_MAXG; ++g) { ea[g] = na[g]; eb[g] = nb[g]; }
-            exponents(it + gridDim.x);
             bool ok = true;
             for (int jb = 0; jb < a.njob; ++jb) {
                 const DgJob job = a.job[jb];
-                int ej = ea[0], ebj = eb[0];
-                #pragma unroll
-                for (int g = 1; g < DG_MAXG; ++g) {
-                    if (job.ga == g) ej = ea[g];
-                    if (job.gb == g) ebj = eb[g];
-                }
-                ej += job.e;
-                const bool bad = __any_sync(0xffffffffu, max(ej, ebj) > DG_NAN / 2);
+                const int wa = na, wb = nb;
+                if (jb + 1 < a.njob) fetch(u, a.job[jb + 1]);
+                else fetch(next, a.job[0]);
+                const int ej = (int)(short)wa + job.e;
                 long long lo[2][HC];
                 uint32_t v[2][4][4];
                 // orders 4..7
@@ -567,10 +629,12 @@ k_dg_corr(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
                         dg_ready(v);
                         const int yp = c0 + 4 * g;
                         zd o[4];
-                        bool edge = bad;
+                        bool edge = false;
+                        unsigned far = 0;
                         #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            const int e = ej + __shfl_sync(0xffffffffu, ebj, 4 * g + j);
+                            const int w = __shfl_sync(0xffffffffu, wb, 4 * g + j), e = ej + (int)(short)w;
+                            far |= (unsigned)dg_far(job, wa, w) << j;
                             long long& t0 = lo[0][4 * g + j];
                             long long& t1 = lo[1][4 * g + j];
                             t0 = dg_high(v[0], j, t0, m21, m29);
@@ -580,9 +644,15 @@ k_dg_corr(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
                         if (__any_sync(0xffffffffu, edge && row)) {
                             #pragma unroll
                             for (int j = 0; j < 4; ++j) {
-                                const int e = ej + __shfl_sync(0xffffffffu, ebj, 4 * g + j);
+                                const int e = ej + (int)(short)__shfl_sync(0xffffffffu, wb, 4 * g + j);
                                 o[j] = mk(dg_value_edge(lo[0][4 * g + j], e), dg_value_edge(lo[1][4 * g + j], e));
                             }
+                        }
+                        if (__any_sync(0xffffffffu, row && far)) {
+                            #pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                if ((far >> j) & 1u) o[j] = mk(0.0, 0.0);
+                            if (lane == 0) atomicOr(a.far + it * a.njob + jb, 1u << dg_mark(q, part, g));
                         }
                         if (row) out(job, u.k, y, yp, o);
                     }
@@ -593,6 +663,7 @@ k_dg_corr(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
                 if (++acc == 2) { acc = 0; aph ^= 1u; }
             }
             if (!ok) break;
+            u = next;
         }
     }
     tc_fence_before();
@@ -600,6 +671,79 @@ k_dg_corr(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+}
+
+// Adds the marked values by FP64 FMAs from the fields.  CTA = one item at a time, whose
+// marks its warps share: a mark's contractions go to one warp in their order (one
+// value may get several).  Lane = row, and a column's far rows are taken either in a chain
+// per lane, as in the FMA kernels, or, where they are few, row by row with a term and
+// snapshot per lane and a tree (10 additions).  Bound by latency with few marked
+// items (one warp per item: 6.5 ms for the 171 items of the duct's m = 0, whose
+// fluctuations are rounding noise; 8 warps 1.9 ms, 32 1.3 but slower where there are none), else by the FP64 pipe.
+constexpr int DG_FARW = 16;                                 // warps of a CTA
+template <typename Out>
+__global__ void __launch_bounds__(32 * DG_FARW, 2)
+k_dg_far(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
+{
+    const int lane = threadIdx.x & 31;
+    static_assert(DG_MAXJOB <= 32, "a lane per contraction");
+    const unsigned own = 0x00010001u << (threadIdx.x >> 5);
+    static_assert(DG_FARW == 16, "marks of a warp");
+    for (long long it = blockIdx.x; it < a.nitems; it += gridDim.x) {
+        const unsigned mine = lane < a.njob ? a.far[it * a.njob + lane] & own : 0u;
+        for (unsigned any = __ballot_sync(0xffffffffu, mine != 0); any; any &= any - 1) {
+            const int src = __ffs(any) - 1;
+            const DgItem u = dg_item(a, it);
+            DgJob job = a.job[src];
+            job.kind |= DJ_ADD;
+            const int* E = a.E + (long long)u.k * a.ngrp * a.s.nrow;
+            const int n = job.nt * a.src.ns;
+            const double ce = __hiloint2double((1023 + job.ex) << 20, 0);
+            for (unsigned m = __shfl_sync(0xffffffffu, mine, src); m; m &= m - 1) {
+                const int b = __ffs(m) - 1, r = (b >> 1 & 3) * 32 + lane;
+                const int y = u.mt * a.s.RT + r, y0 = u.c * a.s.CW + (b >> 3) * 8 + (b & 1) * 4;
+                const bool row = r < a.s.RT && y < a.s.cov;
+                const int wa = row ? E[job.ga * a.s.nrow + y] : 0;
+                auto product = [&](int i, int ya, int yb, zd& acc) {
+                    const int t = i / a.src.ns, s = i - t * a.src.ns;
+                    const DgStep st = a.step[job.step + t];
+                    const DgField &fa = a.src.f[a.af[st.fa]], &fb = a.src.f[a.bf[st.fb]];
+                    const zd p = dg_load(a.src, fa, u.k, s, ya), v = dg_load(a.src, fb, u.k, s, yb);
+                    const double c = __hiloint2double((1023 + fa.wexp + fb.wexp) << 20 | ((st.flags & DF_NEG) ? (int)0x80000000 : 0), 0);
+                    acc.x = fma(c * p.x, v.x, acc.x);
+                    acc.x = fma(c * p.y, v.y, acc.x);
+                    acc.y = fma(c * p.x, v.y, acc.y);
+                    acc.y = fma(-c * p.y, v.x, acc.y);
+                };
+                zd o[4];
+                #pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int yp = y0 + j;
+                    const bool far = row && yp < a.s.n && !(a.tri && yp < y) && dg_far(job, wa, E[job.gb * a.s.nrow + yp]);
+                    const unsigned who = __ballot_sync(0xffffffffu, far);
+                    zd acc = mk(0.0, 0.0);
+                    if (__popc(who) * (10 + 4 * ((n + 31) / 32)) >= 4 * n) {
+                        if (far)
+                            for (int i = 0; i < n; ++i) product(i, y, yp, acc);
+                    } else {
+                        for (unsigned w = who; w; w &= w - 1) {
+                            const int l = __ffs(w) - 1, ya = __shfl_sync(0xffffffffu, y, l);
+                            zd p = mk(0.0, 0.0);
+                            for (int i = lane; i < n; i += 32) product(i, ya, yp, p);
+                            #pragma unroll
+                            for (int h = 16; h > 0; h >>= 1) {
+                                p.x += __shfl_xor_sync(0xffffffffu, p.x, h);
+                                p.y += __shfl_xor_sync(0xffffffffu, p.y, h);
+                            }
+                            if (lane == l) acc = p;
+                        }
+                    }
+                    o[j] = mk(ce * acc.x, ce * acc.y);
+                }
+                if (row) out(job, u.k, y, y0, o);
+            }
+        }
     }
 }
 
@@ -611,7 +755,13 @@ struct HostTerm { int fa, fb; bool neg; };
 inline void dg_schedule(DgArgs& a, const std::vector<std::vector<HostTerm>>& jobs)
 {
     a.nstep = 0;
-    for (const auto& j : jobs)
+    for (size_t i = 0; i < jobs.size(); ++i) {
+        const auto& j = jobs[i];
+        DgJob& d = a.job[i];
+        d.nt = (unsigned char)j.size();
+        d.step = (unsigned char)a.nstep;
+        const unsigned nibbles = (1u << (4 * d.nt)) - 1;
+        d.mask = (unsigned short)(0x8888u & nibbles);
         for (int pass = 0; pass < 2; ++pass)
             for (size_t t = 0; t < j.size(); ++t) {
                 DgStep s{};
@@ -621,6 +771,7 @@ inline void dg_schedule(DgArgs& a, const std::vector<std::vector<HostTerm>>& job
                                           (t + 1 == j.size() ? DF_LAST : 0));
                 a.step[a.nstep++] = s;
             }
+    }
     int held[DG_NB], last[DG_NB];
     for (int i = 0; i < DG_NB; ++i) held[i] = last[i] = -1;
     for (int q = 0; q < a.nstep; ++q) {
@@ -665,11 +816,12 @@ template <typename Out> inline void dg_run(const DgArgs& a, const Out& out, cuda
     else if (a.s.RT == 72) a.s.CW == 24 ? dg_launch<72, 24>(a, out, st) : dg_launch<72, 32>(a, out, st);
     else a.s.CW == 24 ? dg_launch<128, 24>(a, out, st) : dg_launch<128, 32>(a, out, st);
 }
-// the operands of p, then the contractions
+// the operands of p, then the contractions (three kernels)
 template <typename Out> inline void dg_pass(const DgPrep& p, const DgArgs& a, int nk, const Out& out, cudaStream_t st)
 {
     k_dg_prep<<<(unsigned)((long long)nk * p.ngrp * (p.s.nrow / 128)), 256, 0, st>>>(p);
     dg_run(a, out, st);
+    k_dg_far<Out><<<(unsigned)std::min<long long>(a.nitems, 4 * dg_sm_count()), 32 * DG_FARW, 0, st>>>(a, out);
 }
 template <typename Out> inline cudaError_t dg_attrs()
 {
@@ -682,28 +834,64 @@ template <typename Out> inline cudaError_t dg_attrs()
     }
     return cudaSuccess;
 }
-// bytes of one wavenumber's operands and exponents
-inline size_t dg_bytes_per_k(const DgShape& s, int nfa, int nfb, int ngrp)
+// the next field: X_src times 2^wexp as A and B operand ia, ib (-1: none)
+inline DgField& dg_field(DgPrep& p, DgArgs& a, int grp, int src, int ia, int ib, int wexp = 0)
 {
-    return (nfa * dg_a_halves(s) + nfb * dg_b_halves(s)) * sizeof(__half) + (size_t)ngrp * s.nrow * sizeof(int);
+    DgField f{};
+    f.src = (short)src; f.src2 = -1; f.ia = (short)ia; f.ib = (short)ib;
+    f.wexp = (signed char)wexp; f.grp = (signed char)grp;
+    if (ia >= 0) a.af[ia] = (unsigned char)p.src.nf;
+    if (ib >= 0) a.bf[ib] = (unsigned char)p.src.nf;
+    return p.src.f[p.src.nf++] = f;
 }
-// places the operands of nk wavenumbers in ws
-inline void dg_place(DgPrep& p, DgArgs& a, void* ws, int nk)
+// tiles of one wavenumber
+inline int dg_tiles(const DgShape& s, bool tri)
 {
+    int n = 0;
+    for (int mt = 0; mt < s.MT; ++mt) n += s.NT - (tri ? mt * s.RT / s.CW : 0);
+    return n;
+}
+// bytes of one wavenumber's operands, exponents and marks
+inline size_t dg_bytes_per_k(const DgShape& s, int nfa, int nfb, int ngrp, int njob, bool tri)
+{
+    return (nfa * dg_a_halves(s) + nfb * dg_b_halves(s)) * sizeof(__half) + (size_t)ngrp * s.nrow * sizeof(int) +
+           (size_t)dg_tiles(s, tri) * njob * sizeof(unsigned);
+}
+// places the operands of nk wavenumbers from k0 on in ws
+inline void dg_place(DgPrep& p, DgArgs& a, void* ws, int k0, int nk)
+{
+    p.src.k0 = k0;
     p.Aop = (__half*)ws;
     p.Bop = p.Aop + (size_t)nk * p.nfa * dg_a_halves(p.s);
     p.E = (int*)(p.Bop + (size_t)nk * p.nfb * dg_b_halves(p.s));
     a.Aop = p.Aop; a.Bop = p.Bop; a.E = p.E;
     a.nitems = (long long)nk * a.tpk;
+    p.far = a.far = (unsigned*)(p.E + (size_t)nk * p.ngrp * p.s.nrow);
+    p.nfar = a.nitems * a.njob;
 }
-// tiles per wavenumber, shape and constants
-inline void dg_init(DgPrep& p, DgArgs& a, const DgShape& s, int nfa, int nfb, int ngrp, bool tri, int* err)
+// the snapshots [s0, s0 + ns), ns <= 16: with them the digits' factor c and what depends on it
+inline void dg_batch(DgPrep& p, DgArgs& a, int s0, int ns)
+{
+    p.cexp = 0;
+    while ((ns << (p.cexp + 1)) <= DG_KS) ++p.cexp;
+    p.src.s0 = s0;
+    p.src.ns = ns;
+    a.src = p.src;
+    for (int i = 0; i < a.njob; ++i) {
+        DgJob& d = a.job[i];
+        d.e = (short)(d.ex - 34 - p.cexp);
+        d.add = (unsigned short)((d.mask >> 3) * (7 - dg_lmax(d.nt, ns)));
+    }
+}
+// tiles per wavenumber, shape and constants; X: fields of Nk wavenumbers and ns snapshots
+inline void dg_init(DgPrep& p, DgArgs& a, const DgShape& s, int nfa, int nfb, int ngrp, bool tri, const zd* X, int Nk,
+                    int ns, int* err)
 {
     p.s = a.s = s;
+    p.src.X = X; p.src.n = s.n; p.src.Nk = Nk; p.src.nsX = ns;
     p.nfa = a.nfa = nfa; p.nfb = a.nfb = nfb; p.ngrp = a.ngrp = ngrp;
     a.tri = tri;
-    a.tpk = 0;
-    for (int mt = 0; mt < s.MT; ++mt) a.tpk += s.NT - (tri ? mt * s.RT / s.CW : 0);
+    a.tpk = dg_tiles(s, tri);
     for (int i = 0; i < 4; ++i) a.mul[i] = 1 << (5 + 8 * i);
     a.err = err;
 }

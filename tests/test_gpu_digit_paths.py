@@ -32,8 +32,9 @@ def workspace(N, plan, nbytes, duct=False):
     assert f(plan, nbytes) == N.GKE_OK
 
 
-def channel(N, wl, coef, ws=None, nu=None):
-    plan = N.gke_plan(wl.nx, wl.nz, wl.ny, wl.Lx, wl.Lz, wl.nu if nu is None else nu, S.cgl_grid(wl.ny), coef.shape[0])
+def channel(N, wl, coef, ws=None, nu=None, mask=0):
+    plan = N.gke_plan(wl.nx, wl.nz, wl.ny, wl.Lx, wl.Lz, wl.nu if nu is None else nu, S.cgl_grid(wl.ny), coef.shape[0],
+                      term_mask=mask)
     try:
         if ws is not None:
             workspace(N, plan, ws)
