@@ -249,9 +249,12 @@ k1_products(const zd* __restrict__ f, int ns, int P, int nx, const zd* __restric
 
 // The same for nx = N1 N2 = 128, 256 by register transforms in fixed point, the
 // fields packed in pairs: two inverse and four forward transforms a snapshot
-// instead of 4 + 7 in FP64 through shared memory.  CTA = one point; N2 lanes of a warp take one
+// instead of 4 + 7 in FP64 through shared memory, each field at its own exponent
+// (gke::FxPair: a small field beside a large one is not rounded at the large one's
+// size).  CTA = one point; N2 lanes of a warp take one
 // snapshot, u, v, w of it in shared memory between the transforms
-// (256 x 33 x 33, 16 snapshots: products stage 3.46 -> 1.35 ms, FP32 plans 3.87 -> 1.70).  512 points would
+// (256 x 33 x 33, 16 snapshots: products stage 3.46 -> 1.62 ms, FP32 plans 3.87 -> 1.91;
+// with one exponent a pair 1.37 and 1.71).  512 points would
 // need more registers than a thread has.
 template <typename TF, int N1, int N2>
 __global__ void __launch_bounds__(128)
@@ -277,26 +280,35 @@ k1_products_r(const zd* __restrict__ f, int ns, int P, const zd* __restrict__ tw
         zd vb[N1];
         #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const zd* fa = f + ((long long)(s * 4 + 2 * q) * P + p) * nxh;
-            const zd* fb = fa + (long long)P * nxh;
-            const double ma = prof[(long long)(R_U + 2 * q) * P + p], mb = prof[(long long)(R_U + 2 * q + 1) * P + p];
+            // coefficient lane + N2 m of field 2 q + h: fluctuation, Hermitian extension
+            const zd* f0 = f + ((long long)(s * 4 + 2 * q) * P + p) * nxh;
+            const double* mean = prof + (long long)(R_U + 2 * q) * P + p;
+            auto coef = [&](int h, int m) {
+                const int k = lane + N2 * m, kk = k < nxh ? k : N - k;
+                zd a = f0[(long long)h * P * nxh + kk];
+                nonfinite |= !isfinite(a.x) || !isfinite(a.y);
+                if (kk == 0) a.x -= mean[(long long)h * P];
+                if (kk == 0 || 2 * kk == N) a.y = 0.0;
+                else if (k >= nxh) a.y = -a.y;
+                return a;
+            };
+            const gke::FxPair pr(gke::fx_part_exponent<N1, N2>([&](int m) { return coef(0, m); }),
+                                 gke::fx_part_exponent<N1, N2>([&](int m) { return coef(1, m); }));
             #pragma unroll
             for (int m = 0; m < N1; ++m) {
-                const int k = lane + N2 * m, kk = k < nxh ? k : N - k;
-                zd a = fa[kk], b = fb[kk];
-                if (k < nxh) nonfinite |= !isfinite(a.x) || !isfinite(a.y) || !isfinite(b.x) || !isfinite(b.y);
-                if (kk == 0) { a.x -= ma; b.x -= mb; }
-                if (kk == 0 || 2 * kk == N) a.y = b.y = 0.0;
-                if (k < nxh) {
-                    if (live) {
-                        X[(((long long)(2 * q) * nxh + k) * ns + s) * P + p] = cvt<TF>(a);
-                        X[(((long long)(2 * q + 1) * nxh + k) * ns + s) * P + p] = cvt<TF>(b);
-                    }
-                } else { a.y = -a.y; b.y = -b.y; }
-                vb[m] = mk(a.x - b.y, a.y + b.x);        // a + i b
+                const int k = lane + N2 * m;
+                const zd a = coef(0, m), b = coef(1, m);
+                if (k < nxh && live) {
+                    X[(((long long)(2 * q) * nxh + k) * ns + s) * P + p] = cvt<TF>(a);
+                    X[(((long long)(2 * q + 1) * nxh + k) * ns + s) * P + p] = cvt<TF>(b);
+                }
+                const zd c = mk(pr.in(0, a.x), pr.in(0, a.y)), d = mk(pr.in(1, b.x), pr.in(1, b.y));
+                vb[m] = mk(c.x - d.y, c.y + d.x);        // a + i b
             }
             __syncwarp();
-            gke::fft2l_rows<double, N1, N2, true>(vb, lane, xr, N2 + 1, 1, stw);
+            const int e = pr.E - gke::FX_IB + gke::FX_S;
+            gke::fft2l_raw<N1, N2, true, true>(vb, pr.E, lane, (gke::zx*)xr, N2 + 1, 1, (const gke::zx*)stw,
+                [&](int m, gke::zx w, bool) { vb[m] = mk(pr.out(0, w.x, e), pr.out(1, w.y, e)); });
             if (q == 0) {
                 #pragma unroll
                 for (int m = 0; m < N1; ++m) { ph[N2 * m] = vb[m].x; ph[N + N2 * m] = vb[m].y; }
@@ -324,7 +336,7 @@ k1_products_r(const zd* __restrict__ f, int ns, int P, const zd* __restrict__ tw
             }
             const int fa = j == 0 ? G_UU : j == 1 ? G_WW : j == 2 ? G_UW : G_Q, fb = j == 0 ? G_VV : j == 1 ? G_UV : G_VW;
             __syncwarp();
-            gke::fft2l_split<double, N1, N2>(h, lane, xr, stw, [&](int k, zd a, zd b) {
+            gke::fft2l_split<double, N1, N2, true>(h, lane, xr, stw, [&](int k, zd a, zd b) {
                 if (!live) return;
                 X[(((long long)fa * nxh + k) * ns + s) * P + p] = cvt<TF>(a);
                 if (j < 3) X[(((long long)fb * nxh + k) * ns + s) * P + p] = cvt<TF>(b);

@@ -237,18 +237,18 @@ inline void fx_table(int n, zd* tab)
     }
 }
 
-// 1-norm of this thread's values in FP32, from their upper words, times
-// 2^(896 - bias); the usual bias is 896, the difference of the FP64 and FP32
-// exponent offsets
+// |x| in FP32, from its upper word, times 2^(896 - bias); the usual bias is 896, the
+// difference of the FP64 and FP32 exponent offsets
+__device__ __forceinline__ float fx_mag(double x, int bias)
+{
+    return __int_as_float(min(max((__double2hiint(x) & 0x7fffffff) - (bias << 20), 0), 0x0fe00000) << 3);
+}
+// 1-norm of this thread's values, scaled so
 template <int N1> __device__ __forceinline__ float fx_norm(const zd* v, int bias)
 {
-    const int b = bias << 20;
-    auto mag = [b](double x) {
-        return __int_as_float(min(max((__double2hiint(x) & 0x7fffffff) - b, 0), 0x0fe00000) << 3);
-    };
     float s = 0.f;
     #pragma unroll
-    for (int j = 0; j < N1; ++j) s += mag(v[j].x) + mag(v[j].y);
+    for (int j = 0; j < N1; ++j) s += fx_mag(v[j].x, bias) + fx_mag(v[j].y, bias);
     return s;
 }
 // largest upper word of |re|, |im|
@@ -290,6 +290,73 @@ template <int N1, int N2> __device__ __forceinline__ int fx_rows_exponent(const 
     }
     return fx_exponent(s, bias);
 }
+
+// Two sequences a, b in one transform (a + i b of real, or A + i B of Hermitian
+// sequences): the sum of both would round each at the size of the larger.  Each has its
+// own exponent (from its 1-norm), the smaller is scaled up to the larger's by a power of
+// two and the result's half scaled back: both come out as if transformed alone.
+constexpr int FX_ZERO = -9000;                            // exponent of a sequence of zeros
+// the exponent of get(0) .. get(N1 - 1) of N2 consecutive threads of a warp
+template <int N1, int N2, typename G> __device__ __forceinline__ int fx_part_exponent(G get)
+{
+    auto add = [](float a, float b) { return a + b; };
+    float s = 0.f;
+    int m = 0;
+    #pragma unroll
+    for (int j = 0; j < N1; ++j) {
+        const zd v = get(j);
+        s += fx_mag(v.x, 896) + fx_mag(v.y, 896);
+        m = max(m, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
+    }
+    const bool far = !(s > 1e-30f && s < 1e30f) && m != 0;
+    s = fx_reduce<N2>(s, add);
+    int bias = 896;
+    if (__any_sync(0xffffffffu, far)) {
+        m = fx_reduce<N2>(m, [](int a, int b) { return max(a, b); });
+        bias = (m >> 20) - 127;
+        s = 0.f;
+        #pragma unroll
+        for (int j = 0; j < N1; ++j) {
+            const zd v = get(j);
+            s += fx_mag(v.x, bias) + fx_mag(v.y, bias);
+        }
+        s = m == 0 ? 0.f : fx_reduce<N2>(s, add);
+        if (bias == 0x7ff - 127) return FX_NAN;
+    }
+    return s > 0.f ? fx_exponent(s, bias) : FX_ZERO;
+}
+// exponent of the sum, powers of two that a and b are scaled up by; a part with an
+// infinity or a NaN is left out of the transform (its results are NaN)
+struct FxPair {
+    int E, up[2];
+    bool nan[2], safe;
+    __device__ __forceinline__ FxPair(int ea, int eb)
+    {
+        nan[0] = ea == FX_NAN; nan[1] = eb == FX_NAN;
+        if (nan[0]) ea = FX_ZERO;
+        if (nan[1]) eb = FX_ZERO;
+        const int top = max(ea, eb);
+        up[0] = ea == FX_ZERO ? 0 : top - ea;
+        up[1] = eb == FX_ZERO ? 0 : top - eb;
+        E = top == FX_ZERO ? 0 : top + (ea != FX_ZERO && eb != FX_ZERO);
+        safe = fx_safe(E) && fx_safe(E - up[0]) && fx_safe(E - up[1]);
+    }
+    // a value of part h, scaled up
+    __device__ __forceinline__ double in(int h, double x) const
+    {
+        const int hi = __double2hiint(x);
+        if (nan[h]) return 0.0;
+        if (up[h] == 0) return x;
+        if ((hi & 0x7ff00000) == 0) return x == 0.0 ? x : fx_scale_edge(x, up[h]);
+        return __hiloint2double(hi + (up[h] << 20), __double2loint(x));
+    }
+    // an output w 2^e of part h, scaled back
+    __device__ __forceinline__ double out(int h, long long w, int e) const
+    {
+        if (nan[h]) return __longlong_as_double(0x7ff8000000000000ll);
+        return safe ? fx_to(w, e - up[h]) : fx_to_edge(w, e - up[h], 0);
+    }
+};
 
 // fft2l with the lanes of a sequence side by side (N2 consecutive threads of a
 // warp, xs their own: synchronises the warp only) or spread over the block
@@ -347,8 +414,9 @@ __device__ __forceinline__ void fft2l_cols(cplx<T>* v, int seq, int nseq, int la
 // N = N1 N2, handed to put(m, a^, b^), m = 0 .. N / 2, by the N2 lanes of the
 // sequence; xr: their shared buffer.  FP64: the sums are integers' and 1 / (2 N)
 // is in the exponent (in FP64 they took half of the row kernels' FP64 operations:
-// products stage of 256 x 256 x 65, 16 snapshots, 23.0 -> 21.0 ms).
-template <typename T, int N1, int N2, typename F>
+// products stage of 256 x 256 x 65, 16 snapshots, 23.0 -> 21.0 ms).  PARTS: a and b rounded
+// at their own sizes (FxPair).
+template <typename T, int N1, int N2, bool PARTS = false, typename F>
 __device__ __forceinline__ void fft2l_split(cplx<T>* f, int lane, cplx<T>* xr, const cplx<T>* stw, F put)
 {
     constexpr int N = N1 * N2;
@@ -365,7 +433,15 @@ __device__ __forceinline__ void fft2l_split(cplx<T>* f, int lane, cplx<T>* xr, c
             put(k, h * (Z + Zc), mk(h * D.y, -h * D.x));
         }
     } else {
-        const int E = fx_rows_exponent<N1, N2>(f);
+        auto part = [&](int h) {
+            return fx_part_exponent<N1, N2>([&](int j) { return mk(h ? f[j].y : f[j].x, 0.0); });
+        };
+        const FxPair pr = PARTS ? FxPair(part(0), part(1)) : FxPair(FX_ZERO, FX_ZERO);
+        if (PARTS) {
+            #pragma unroll
+            for (int m = 0; m < N1; ++m) f[m] = mk(pr.in(0, f[m].x), pr.in(1, f[m].y));
+        }
+        const int E = PARTS ? pr.E : fx_rows_exponent<N1, N2>(f);
         zx* x = (zx*)xr;
         zx w[N1];
         fft2l_raw<N1, N2, false, true>(f, E, lane, x, N2 + 1, 1, (const zx*)stw, [&](int m, zx a, bool) { w[m] = a; });
@@ -379,7 +455,8 @@ __device__ __forceinline__ void fft2l_split(cplx<T>* f, int lane, cplx<T>* xr, c
         for (int k = lane; k <= N / 2; k += N2) {
             const zx Z = x[k], Y = x[(N - k) & (N - 1)];
             const long long ax = Z.x + Y.x, ay = Z.y - Y.y, bx = Z.y + Y.y, by = Y.x - Z.x;
-            if (fx_safe(E)) put(k, mk(fx_to(ax, e), fx_to(ay, e)), mk(fx_to(bx, e), fx_to(by, e)));
+            if (PARTS) put(k, mk(pr.out(0, ax, e), pr.out(0, ay, e)), mk(pr.out(1, bx, e), pr.out(1, by, e)));
+            else if (fx_safe(E)) put(k, mk(fx_to(ax, e), fx_to(ay, e)), mk(fx_to(bx, e), fx_to(by, e)));
             else put(k, mk(fx_to_edge(ax, e, E), fx_to_edge(ay, e, E)), mk(fx_to_edge(bx, e, E), fx_to_edge(by, e, E)));
         }
     }
