@@ -8,6 +8,7 @@
 // complex sequence).  The transform arithmetic runs in TF = double (plain
 // path) or float (split path); one-point sums are always FP64.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "gke_common.cuh"
@@ -282,7 +283,8 @@ __global__ void k_row_products(const cplx<TF>* __restrict__ G, int ny, int nz, i
 // Per row: two inverse transforms (u + i v, w + i p), the row sums (p is not
 // needed after them), then per packed pair of products a forward transform and
 // its Hermitian split through the row's shared buffer.
-// Row sums: TF over a thread's N1 points, FP64 across threads.
+// Row sums: FP64; of FP32 passes at 256 points FP32 over a thread's 16 points (FP64 costs
+// 16 clocks an operation of a warp, and that pass is bound by its arithmetic).
 template <typename TF, int N1, int N2, int RZ>
 __global__ void __launch_bounds__(RZ * N2)
 k_row_products_r(const cplx<TF>* __restrict__ G, int ny, int nz, const cplx<TF>* __restrict__ tw_x,
@@ -304,7 +306,8 @@ k_row_products_r(const cplx<TF>* __restrict__ G, int ny, int nz, const cplx<TF>*
     load_twiddles2l<TF>(stw, tw_x, N);
     __syncthreads();
     TF* ph = (TF*)(xs + RZ * N1 * (N2 + 1)) + r * 3 * N + lane;
-    TF s6[6] = {0, 0, 0, 0, 0, 0};
+    typedef typename std::conditional<N == 256, TF, double>::type TS;
+    TS s6[6] = {0, 0, 0, 0, 0, 0};
     {
         C vb[N1];
         #pragma unroll
@@ -332,8 +335,8 @@ k_row_products_r(const cplx<TF>* __restrict__ G, int ny, int nz, const cplx<TF>*
         #pragma unroll
         for (int m = 0; m < N1; ++m) {
             const TF u = ph[N2 * m], vv = ph[N + N2 * m], w = vb[m].x, pp = vb[m].y;
-            const TF q = u * u + vv * vv + w * w;
-            s6[0] += q; s6[1] += u * vv; s6[2] += pp * vv; s6[3] += q * u; s6[4] += q * vv; s6[5] += q * w;
+            const TS us = u, vs = vv, ws = w, q = us * us + vs * vs + ws * ws;
+            s6[0] += q; s6[1] += us * vs; s6[2] += (TS)pp * vs; s6[3] += q * us; s6[4] += q * vs; s6[5] += q * ws;
             ph[2 * N + N2 * m] = w;
         }
     }
