@@ -37,3 +37,27 @@ def test_products_wider_than_fp32(nx, tmp_path):
     for precision in (N.GKE_PREC_F32, N.GKE_PREC_BF16X3):
         got = statistics(N, nx, precision, str(tmp_path / "f32"))
         assert (np.abs(got / want - 1) <= 1e-14).all(), np.abs(got / want - 1).max()
+
+
+def test_transforms_keep_the_energy(tmp_path):
+    """The mean energy of random fields from FP32 transforms of 128 x 128 points
+    (twiddles within half a unit of 2^-24) is the FP64 plan's within one FP32
+    rounding, 2^-24: sampling noise is 1e-10, what remains is the transforms' gain."""
+    import torch
+    N = native()
+    wl = S.small(128, 128, 9, 4, wid=77)
+    f = torch.from_numpy(S.coefficients(wl)).cuda()
+    q = []
+    for precision in (N.GKE_PREC_F64, N.GKE_PREC_F32):
+        path = str(tmp_path / "stats")
+        plan = N.gke_plan(wl.nx, wl.nz, wl.ny, wl.Lx, wl.Lz, wl.nu, S.cgl_grid(wl.ny), wl.nsnap, precision)
+        try:
+            N.gke_accumulate_mean(plan, f, wl.nsnap)
+            N.gke_accumulate_snapshot(plan, f, wl.nsnap)
+            N.gke_checkpoint(plan, path)
+        finally:
+            N.gke_destroy(plan)
+        q.append(np.fromfile(path, dtype=np.float64, offset=96, count=5 * wl.ny).reshape(5, wl.ny)[4])
+    inner = q[0] > 0
+    gain = (q[1][inner] / q[0][inner]).mean() - 1
+    assert abs(gain) <= 2.0 ** -24, gain
