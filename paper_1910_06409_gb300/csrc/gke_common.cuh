@@ -163,23 +163,6 @@ __device__ __forceinline__ void load_twiddles(cplx<T>* sh_tw, const cplx<T>* __r
 // ---------------------------------------------------------------- register FFT
 // W_32^j = e^{-2 pi i j / 32}, j < 16: values of the host libm cos / sin,
 // written out (each translation unit has its own copy)
-static __constant__ zd c_tw32d[16] = {
-    {1.0, -0.0},
-    {0.98078528040323043, -0.19509032201612825},
-    {0.92387953251128674, -0.38268343236508978},
-    {0.83146961230254524, -0.55557023301960218},
-    {0.70710678118654757, -0.70710678118654746},
-    {0.55557023301960229, -0.83146961230254524},
-    {0.38268343236508984, -0.92387953251128674},
-    {0.19509032201612833, -0.98078528040323043},
-    {6.123233995736766e-17, -1},
-    {-0.19509032201612819, -0.98078528040323043},
-    {-0.38268343236508973, -0.92387953251128674},
-    {-0.55557023301960196, -0.83146961230254546},
-    {-0.70710678118654746, -0.70710678118654757},
-    {-0.83146961230254535, -0.55557023301960218},
-    {-0.92387953251128674, -0.38268343236508989},
-    {-0.98078528040323043, -0.19509032201612861}};
 static __constant__ zf c_tw32f[16] = {
     {1.0f, -0.0f},
     {0.98078528f, -0.195090322f},
@@ -197,25 +180,22 @@ static __constant__ zf c_tw32f[16] = {
     {-0.831469612f, -0.555570233f},
     {-0.923879533f, -0.382683432f},
     {-0.98078528f, -0.195090322f}};
-template <typename T> __device__ __forceinline__ cplx<T> tw32(int j);
-template <> __device__ __forceinline__ zf tw32<float>(int j) { return c_tw32f[j]; }
-template <> __device__ __forceinline__ zd tw32<double>(int j) { return c_tw32d[j]; }
-
 // s sqrt(1/2) with one rounding.  FP32's sqrt(1/2) is 1.7e-8 too small, so every
 // transform lost energy (of a 128-point one 3.6e-8, 1.8e-8 so; the shared-memory
 // stages' 2.8e-8), which the one-point sums of its results keep.
-template <typename T> __device__ __forceinline__ T half_sqrt(T s)
+__device__ __forceinline__ float half_sqrt(float s)
 {
-    const T c = (T)0.70710678118654752440;
-    if constexpr (sizeof(T) == 4) return fmaf(c, s, (float)(0.70710678118654752440 - (double)0.70710678118654752440f) * s);
-    else return c * s;
+    const float c = 0.70710678118654752440f;
+    return fmaf(c, s, (float)(0.70710678118654752440 - (double)c) * s);
 }
 // w * W_32^m (conjugate twiddle if INV) for m known at compile time after
 // unrolling: m = 0 and m = 8 (-i) cost no arithmetic, m = 4 and m = 12
 // ((+-1 - i)/sqrt 2) two additions and two products by sqrt(1/2)
+// (FP32; FP64 sequences are transformed in fixed point, gke_fixed.cuh)
 template <typename T, bool INV>
 __device__ __forceinline__ cplx<T> twiddle_mul(cplx<T> w, int m)
 {
+    static_assert(sizeof(T) == 4, "FP32");
     if (m == 0) return w;
     if (m == 8) return INV ? mk(-w.y, w.x) : mk(w.y, -w.x);
     if (m == 4 || m == 12) {
@@ -223,7 +203,7 @@ __device__ __forceinline__ cplx<T> twiddle_mul(cplx<T> w, int m)
         if (m == 4) return INV ? mk(d, s) : mk(s, -d);
         return INV ? mk(-s, d) : mk(-d, -s);
     }
-    cplx<T> t = tw32<T>(m);
+    zf t = c_tw32f[m];
     if (INV) t.y = -t.y;
     return w * t;
 }

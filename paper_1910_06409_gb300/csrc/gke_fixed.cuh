@@ -59,7 +59,7 @@ __device__ __forceinline__ zx operator*(zx a, zx w)
 }
 __device__ __forceinline__ long long fx_mid(long long a) { return (a + (1 << (FX_S - 1))) >> FX_S; }
 
-// W_32^m for the register DFTs (c_tw32d's constants times 2^63 as signed word pairs)
+// W_32^m for the register DFTs (constants times 2^63 as signed word pairs)
 struct FxC { int h, l; };
 __host__ __device__ constexpr FxC fxc(double c)
 {

@@ -58,13 +58,8 @@ __device__ __forceinline__ uint64_t sdesc(const void* p, uint32_t lbo, uint32_t 
     d |= (uint64_t)1 << 46;
     return d;
 }
-__device__ __forceinline__ void mma_f16(uint32_t dtm, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(dtm), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
-}
-// the same issued by one lane of a converged warp, descriptors as (lower,
-// upper) words
+// D += A B (bf16 or f16, by idesc), issued by one lane of a converged warp; descriptors
+// as (lower, upper) words
 __device__ __forceinline__ void mma_f16_u(uint32_t dtm, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
                                           uint32_t idesc, uint32_t acc) {
     asm volatile("{\n .reg .pred p, q;\n .reg .b64 da, db;\n mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n"
@@ -75,10 +70,6 @@ __device__ __forceinline__ void mma_f16_u(uint32_t dtm, uint32_t alo, uint32_t a
 __device__ __forceinline__ void mma_commit_el(uint64_t* b) {
     asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
                  " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(su32(b))
-                 : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint64_t* b) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(b))
                  : "memory");
 }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
