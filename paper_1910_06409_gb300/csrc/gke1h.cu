@@ -890,7 +890,8 @@ constexpr int ND_JOB = 17;
 static gke::DgShape digit_shape(int P) { return gke::dg_shape(P, false); }
 static size_t digit_bytes(int P) { return gke::dg_bytes_per_k(digit_shape(P), ND, ND, ND_GRP, ND_JOB, true); }
 
-// the contractions of all wavenumbers into the spectra; kernels launched
+// the contractions of all wavenumbers into the spectra; kernels launched, or -1 for
+// contractions beyond the kernel's tables
 static int digit_correlate(gke::DigitWork& w, const zd* X, int ns, int P, int nx, double kx0, double nu,
                            const double* prof, const double* op, const int* pq, zd* spec, long long npair,
                            cudaStream_t st)
@@ -959,7 +960,7 @@ static int digit_correlate(gke::DigitWork& w, const zd* X, int ns, int P, int nx
         job(psi, 1, gu, DG_R1, -1, {{u, D_R1, false}});
         job(phi, 1, DG_V, gp, 0, back(pk, 3, true), psi, 1);
     }
-    gke::dg_schedule(a, terms);
+    if (!gke::dg_schedule(a, terms)) return -1;
     const int kmax = (int)std::min<size_t>((size_t)nxh, w.bytes / digit_bytes(P));
     int launches = 0;
     for (int m0 = 0; m0 < nxh; m0 += kmax) {
@@ -1551,10 +1552,13 @@ static void launch_pass(gke1h_plan_t p, const zd* f, int ns, TF* T)
     }
     {
         Scope1 sc(p, GKE_STAGE_CORRELATE);
-        const bool digits = sizeof(TF) == 8 && gke::digits_ready(p->digits);
-        if (digits)
-            p->launches += digit_correlate(p->digits, (const zd*)X, ns, P, nx, kx0, p->nu, p->prof, p->op, p->pq,
-                                           (zd*)spec, p->npair, p->st);
+        bool digits = sizeof(TF) == 8 && gke::digits_ready(p->digits);
+        if (digits) {
+            const int n = digit_correlate(p->digits, (const zd*)X, ns, P, nx, kx0, p->nu, p->prof, p->op, p->pq,
+                                          (zd*)spec, p->npair, p->st);
+            digits = n >= 0;
+            p->launches += std::max(n, 0);
+        }
         const int nfull = P / CT, rem = P - nfull * CT;
         const bool strips = nfull > 0 && rem > 0 && rem <= STRIP_MAX;
         const int nt = strips ? nfull : p->nt;

@@ -171,7 +171,7 @@ gke_status digits_correlate(DigitWork& w, const zd* Xop, int ns, int ny, int Nk,
         for (int t = 0; t < h.nt; ++t) { rj.fa[t] = h.fa[t]; rj.fb[t] = h.fb[t]; }
     }
     if (!a.njob) return GKE_OK;
-    dg_schedule(a, terms);
+    if (!dg_schedule(a, terms)) { err = "digit correlator: contractions beyond the kernel's tables"; return GKE_ERR_UNSUPPORTED; }
     for (int kc0 = 0; kc0 < Kc; kc0 += kmax) {
         const int nk = std::min(kmax, Kc - kc0);
         dg_place(p, a, w.ws, k0 + kc0, nk);

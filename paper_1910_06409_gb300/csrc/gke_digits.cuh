@@ -751,10 +751,19 @@ k_dg_far(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
 // The steps of an item: every contraction's terms with orders 4..7, then again
 // with orders 0..3; B fields stay in their slot until the slot whose field
 // is needed last has to give way.
+// False, and nothing scheduled, where a contraction has no term or more than DG_MAXT (more
+// would break the exactness of the FP32 sums), or where there are more
+// contractions or steps than the kernels' tables hold.
 struct HostTerm { int fa, fb; bool neg; };
-inline void dg_schedule(DgArgs& a, const std::vector<std::vector<HostTerm>>& jobs)
+inline bool dg_schedule(DgArgs& a, const std::vector<std::vector<HostTerm>>& jobs)
 {
     a.nstep = 0;
+    size_t steps = 0;
+    for (const auto& j : jobs) {
+        if (j.empty() || j.size() > DG_MAXT) return false;
+        steps += 2 * j.size();
+    }
+    if (jobs.size() > DG_MAXJOB || steps > DG_MAXSTEP) return false;
     for (size_t i = 0; i < jobs.size(); ++i) {
         const auto& j = jobs[i];
         DgJob& d = a.job[i];
@@ -795,6 +804,7 @@ inline void dg_schedule(DgArgs& a, const std::vector<std::vector<HostTerm>>& job
     }
     for (int i = 0; i < DG_NB; ++i)
         if (held[i] >= 0) a.step[last[i]].flags |= DF_FREE;
+    return true;
 }
 
 inline int dg_sm_count()
