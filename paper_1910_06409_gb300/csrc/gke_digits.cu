@@ -134,13 +134,14 @@ cudaError_t digits_setup(DigitWork& w, int n, int Kc, cudaStream_t st)
 }
 
 // Against the FMA kernel (correlate stage, us, FMA -> digits): 544 wavenumbers
-// x 4 snapshots: 507 -> 240 at ny = 17, 532 -> 407 at 33, 1954 -> 543 at 65,
-// 7535 -> 1130 at 129; 4160 wavenumbers x 16 snapshots: 7423 -> 1659, 8085 -> 2799,
-// 29421 -> 4326, 112586 -> 9462.  Only where the FMA kernel's CTAs, one
-// 32 x 32 tile of at most one snapshot chunk each, all run at once are the two
-// level (40 wavenumbers: 71 us, digits 66 at ny <= 17, 72 at 25): those keep it
-// and need no workspace.
-bool digits_pays(int n, int ns, long long Kc) { return !(Kc <= 64 && n <= 32 && ns <= 8); }
+// x 4 snapshots: 506 -> 307 at ny = 17, 532 -> 502 at 33, 1946 -> 648 at 65,
+// 7529 -> 1429 at 129; 4224 wavenumbers x 16 snapshots: 7548 -> 2185, 8218 -> 3644,
+// 29927 -> 5266, 114521 -> 12038; 144 x 4: 158 -> 108, 152 -> 163, 635 -> 217, 2224 -> 432.  Only
+// where the FMA kernel's CTAs, one 32 x 32 tile (and its strips) of at most one
+// snapshot chunk each, all run at once is it ahead (40 wavenumbers, up to 8 snapshots:
+// 70 to 80 us, digits 72 to 108 at ny <= 33; 267 against 109 at 65): those keep it and
+// need no workspace.
+bool digits_pays(int n, int ns, long long Kc) { return !(Kc <= 64 && n <= 33 && ns <= 8); }
 
 gke_status digits_correlate(DigitWork& w, const zd* Xop, int ns, int ny, int Nk, int k0, int Kc, zd* raw,
                             unsigned jobs, cudaStream_t st, std::string& err, int* launches)

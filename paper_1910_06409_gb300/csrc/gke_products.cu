@@ -506,7 +506,8 @@ int products_launch(const ProdArgs& a)
     const int nch = (ny + ll_rows<TF>() - 1) / ll_rows<TF>(), rows = (ny + nch - 1) / nch;
     // register transforms, but FP64 ones of 32 points only where enough rows
     // hide their longer chain of integer instructions (32 x 32 x 9, 2 snapshots: row
-    // pass 21 -> 46 us; 32 x 32 x 33, 4 snapshots: products stage 333 -> 322)
+    // pass 21 -> 46 us; products stage of 2 snapshots, us, shared memory against registers:
+    // 32 x 32 x 17 88 / 94, x 25 101 / 97, x 33 121 / 108, x 129 289 / 186; 32 x 8 x 65 102 / 124, x 129 172 / 166)
     auto reg = [&](int n, int other) { return reg_len(n) && (n > 32 || sizeof(TF) == 4 || (long long)other * ny >= 1024); };
     const bool reg_z = reg(nz, nxh * 2), reg_x = reg(nx, nz);
     // the register column pass writes the linear operands itself
@@ -616,7 +617,8 @@ int products_launch(const ProdArgs& a)
     const int neb = (Nk + EPS_KCHUNK - 1) / EPS_KCHUNK;
     // whole rows y per k, as many k side by side as fit; FP32 passes with a
     // thousand chunks fill the chip with one k at a time, whose rows stream
-    // better (256 x 256 x 129, 16 snapshots: products stage 10.55 -> 9.67 ms; FP64, bound by
+    // better (this kernel, us, one k / as many as fit: 128 x 128 x 65, 520 chunks, 487 / 321, 128 x 128 x 129, 4
+    // snapshots, 77 / 100; 256 x 128 x 65, 1032 chunks, 141 / 184, 256 x 256 x 65 574 / 572, 256 x 256 x 129 739 / 1078; FP64, bound by
     // its arithmetic, gains from more at any size: 256 x 256 x 65 24.4 -> 23.0 ms)
     const int yt = std::min(ny, EPS_Y);
     const int kt = sizeof(TF) == 4 && neb >= 1024 ? 1 : std::min(EPS_KCHUNK, EPS_THREADS / yt);

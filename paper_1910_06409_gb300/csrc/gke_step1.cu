@@ -457,7 +457,9 @@ static size_t col_smem(int nz) { return (size_t)(1 + 2 * col_nc(nz)) * nz * size
 static size_t row_smem(int nx) { return (size_t)7 * nx * sizeof(zd); }
 
 // register transforms, but those of 32 points only where enough rows hide their
-// longer chain of integer instructions (the rule of the products stage)
+// longer chain of integer instructions (a call of 2 snapshots, us, shared memory against
+// registers: 32 x 32 x 9 187 / 199, x 17 270 / 274, x 25 315 / 302, x 33 354 / 336, x 129 846 / 679; 32 x 8 x 65
+// 435 / 443, x 129 696 / 687)
 static bool s1_reg(int n, int other, int ny) { return reg_len(n) && (n > 32 || (long long)other * ny >= 1024); }
 static size_t col_r_smem(int n1, int n2) { return (size_t)(n1 * n2 + n1 * (256 + 1)) * sizeof(zd); }
 static size_t row_r_smem(int n1, int n2)

@@ -58,7 +58,7 @@ def duct(N, wl, coef, ws=None, nu=None):
         N.gke1h_destroy(plan)
 
 
-@pytest.mark.parametrize("dims", [(8, 8, 33, 9), (16, 8, 65, 17), (8, 8, 130, 2)])
+@pytest.mark.parametrize("dims", [(8, 8, 33, 9), (16, 8, 33, 1), (16, 8, 65, 17), (8, 8, 130, 2)])
 def test_channel_chunks_and_fallback(dims):
     N = native()
     nx, nz, ny, ns = dims

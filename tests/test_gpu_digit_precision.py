@@ -100,7 +100,7 @@ def check(got, want, bar, name, s):
 @pytest.mark.parametrize("field,bits,ns", CASES)
 def test_channel(field, bits, ns):
     N = native()
-    wl = S.small(8, 8, 33, ns, wid=76)
+    wl = S.small(16, 8, 33, ns, wid=76)                # 72 wavenumbers: digits at any snapshot count
     phys = scaled(S.physical(wl), field, bits)
     coef = S.to_coefficients(phys)
     y = S.cgl_grid(wl.ny)
