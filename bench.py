@@ -50,6 +50,8 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FP64_FLOP_PER_CLK_SM = 4.0
 FP32_FLOP_PER_CLK_SM = 256.0
 N_SM = 152
+# digit pairs (i, j), i + j <= 7, of one FP64 product on the tensor cores
+DIGIT_PAIRS = 36
 
 
 def peaks():
@@ -77,8 +79,7 @@ def correlator_cmac(wl, ns):
 # (profiles/dram_small_cases_split_and_f64.md); a stage missing here reports
 # null (not captured since its kernels changed).
 NCU_TRAFFIC_GB = {
-    "f64": {"stencil": 38.0},
-    "bf16x3": {"correlate": 36.6, "terms": 55.9, "stencil": 20.5, "products": 16.4},
+    "bf16x3": {"terms": 55.9, "stencil": 20.5},
 }
 
 
@@ -90,14 +91,22 @@ def ncu_traffic(wl, precision, stage):
     return None if gb is None else int(gb * 1e9)
 
 
+def fp64_fma_ratio(cmac, ms, pk):
+    """cmac complex FP64 multiply-adds in ms over the FP64 FMA pipe's peak (152 SM x 2
+    DFMA/clk x 2 flop x max SM clock, nominal 1.25 TFLOP/s)."""
+    peak = N_SM * FP64_FLOP_PER_CLK_SM * pk.get("sm_max_mhz", 2070.0) * 1e6
+    return 8.0 * cmac / (ms / 1e3) / peak
+
+
 def stage_rooflines(wl, ns, precision, stage_ms, pk, pk_kind):
     """Algorithmic work of each stage of one pass, and its roofline.
 
     Bytes count each stage's essential inputs read once and outputs written
     once (workspaces between kernels of a stage are not counted); the
-    contraction stage counts flops (tensor BF16 on the split path; FP64 on the
-    plain path, against the FP64 FMA pipe: the exact digit products on the tensor
-    cores pass it)."""
+    contraction stage counts flops (tensor cores: six BF16 slice products on the
+    split path, 36 FP16 digit products on the plain path, per product; padded
+    tiles not counted).  fp64_fma_ratio is the plain path's FP64 rate over the
+    FP64 FMA pipe's peak: a speed-up, not a share of what it runs on."""
     f32 = precision != "f64"
     cz = 8 if f32 else 16                          # bytes of one complex operand / spectrum value
     tz = 4 if f32 else 8                           # bytes of one term value
@@ -151,13 +160,14 @@ def stage_rooflines(wl, ns, precision, stage_ms, pk, pk_kind):
                                 "peak_source": f"bf16_tflops ({pk_kind})",
                                 "note": "stage = operand split + tcgen05 contractions + edge row"}
         else:
-            flops = 8.0 * cm
-            peak = N_SM * FP64_FLOP_PER_CLK_SM * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
-            out["correlate"] = {"bound": "alu", "achieved": flops / (ms / 1e3) / 1e12, "peak": peak,
+            flops = DIGIT_PAIRS * 8.0 * cm
+            peak = pk["bf16_tflops"]
+            out["correlate"] = {"bound": "tensor", "achieved": flops / (ms / 1e3) / 1e12, "peak": peak,
                                 "unit": "TFLOP/s", "flops": flops, "launch_ms": ms,
                                 "traffic": ncu_traffic(wl, precision, "correlate"),
-                                "peak_source": "derived: FP64 FMA pipe, 152 SM x 2 DFMA/clk x 2 flop x max SM clock "
-                                               "(nominal 1.25 TFLOP/s); exact digit products on the tensor cores pass it"}
+                                "peak_source": f"bf16_tflops ({pk_kind}); FP16 runs at the same rate",
+                                "fp64_fma_ratio": fp64_fma_ratio(cm, ms, pk),
+                                "note": "stage = digit operands + tcgen05 digit products + far values"}
         out["correlate"]["frac"] = out["correlate"]["achieved"] / out["correlate"]["peak"]
     return out
 
@@ -528,25 +538,26 @@ def run_step1(args, world, rank, local):
                "h2d_bytes_per_step": int(v_h.numel() * 16 + m_h.numel() * 8),
                "d2h_bytes_per_step": int(o_h.numel() * 16)}
     N.gke_destroy(plan)
-    # FP64 work of the transforms (5 N log2 N per complex length-N DFT): per
+    # arithmetic of the transforms (5 N log2 N per complex length-N DFT), which run in
+    # 64-bit integers for the register lengths: per
     # snapshot 3 + 6 column DFTs of length nz per (y, kx), 5 row DFTs of
     # length nx per (y, z)
     lg = lambda n: float(np.log2(n))
     flops = ns * wl.ny * ((3 + 6) * wl.nxh * 5 * wl.nz * lg(wl.nz) + wl.nz * 5 * 5 * wl.nx * lg(wl.nx))
     pk, pk_kind = peaks()
-    peak = N_SM * FP64_FLOP_PER_CLK_SM * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
-    ach = flops / (ms / 1e3) / 1e12
+    fp64_peak = N_SM * FP64_FLOP_PER_CLK_SM * pk.get("sm_max_mhz", 2070.0) * 1e6
     io_bytes = ns * 6 * wl.ny * wl.nz * wl.nxh * 16
     line = {"metric": "Step-1 velocity-vorticity -> u, v, w, p snapshots/s", "value": ns / (ms / 1e3),
             "unit": "snapshots/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": wl.name, "nx": wl.nx, "nz": wl.nz, "ny": wl.ny, "snapshots": ns,
                        "l2": "inputs and outputs larger than L2 (no flush)"},
-            "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                         "flops": flops, "note": "FP64 DFT work, 5 N log2 N per transform",
-                         "peak_source": "derived: 152 SM x 2 DFMA/clk x 2 flop x max SM clock"},
-            "hbm": {"bytes": io_bytes, "achieved_gbs": io_bytes / (ms / 1e3) / 1e9, "peak_gbs": pk["hbm_gbs"],
-                    "note": "inputs read once and outputs written once"},
+            "roofline": {"bound": "hbm", "achieved": io_bytes / (ms / 1e3) / 1e9, "peak": pk["hbm_gbs"], "unit": "GB/s",
+                         "frac": io_bytes / (ms / 1e3) / 1e9 / pk["hbm_gbs"], "bytes": io_bytes,
+                         "note": "inputs read once and outputs written once",
+                         "peak_source": f"hbm_gbs ({pk_kind})"},
+            "dft": {"flops": flops, "fp64_fma_ratio": flops / (ms / 1e3) / fp64_peak,
+                    "note": "5 N log2 N per transform over the FP64 FMA pipe's peak; they run on the integer units"},
             "e2e": e2e, "gpu_launches": launches, "clocks": clk.summary()}
     if rank == 0:
         print(json.dumps(line), flush=True)
@@ -556,10 +567,10 @@ def run_step1(args, world, rank, local):
 METRIC_1H = "GKE one-homogeneous-direction (p1,p2)-pair correlations/s, FP64"
 
 
-# DRAM bytes of one pass's k_dg_prep, k_dg_corr and k1_finish launches on the small
+# DRAM bytes of one pass's k_dg_prep, k_dg_corr, k_dg_far and k1_finish launches on the small
 # case duct_256x17x17_s16 (41,905 pairs), scaled in proportion to the pairs of the
 # workload run (profiles/counters_fp64_digits_128x128x65_s16_and_duct_256x17x17_s16.md)
-NCU_CORR_1H = (3.994e9, 41905)
+NCU_CORR_1H = (4.355e9, 41905)
 
 
 def correlator_cmac_1h(wl, ns):
@@ -646,16 +657,17 @@ def run_one_homog(args, world, rank, local):
     del terms
     N.gke1h_destroy(plan)
     pk, pk_kind = peaks()
-    peak = N_SM * FP64_FLOP_PER_CLK_SM * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
+    peak = pk["bf16_tflops"]
     cms = stage_ms.get("correlate", 0.0)
-    flops = 8.0 * correlator_cmac_1h(wl, ns)
+    cm = correlator_cmac_1h(wl, ns)
+    flops = DIGIT_PAIRS * 8.0 * cm
     ach = flops / (cms / 1e3) / 1e12 if cms > 0 else 0.0
-    roof = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+    roof = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
             "flops": flops, "launch_ms": cms, "stage": "correlate",
             "traffic": int(NCU_CORR_1H[0] * wl.npair / NCU_CORR_1H[1]) if ns == 16 else None,
             "traffic_note": "small-case ncu capture scaled by pairs",
-            "peak_source": "derived: FP64 FMA pipe, 152 SM x 2 DFMA/clk x 2 flop x max SM clock (nominal 1.25 TFLOP/s); "
-                           "exact digit products on the tensor cores pass it"}
+            "fp64_fma_ratio": fp64_fma_ratio(cm, cms, pk) if cms > 0 else None,
+            "peak_source": f"bf16_tflops ({pk_kind}); FP16 runs at the same rate"}
     cpu = None
     if not args.no_cpu:
         phys = S.duct_physical(wl)
@@ -703,11 +715,13 @@ def one_homog_compact(steps=3, warmup=2):
     del terms, f_dev
     torch.cuda.empty_cache()
     pk, _ = peaks()
-    peak = N_SM * FP64_FLOP_PER_CLK_SM * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
     cms = stage_ms.get("correlate", 0.0)
-    frac = 8.0 * correlator_cmac_1h(wl, ns) / (cms / 1e3) / 1e12 / peak if cms > 0 else None
+    cm = correlator_cmac_1h(wl, ns)
+    frac = DIGIT_PAIRS * 8.0 * cm / (cms / 1e3) / 1e12 / pk["bf16_tflops"] if cms > 0 else None
+    ratio = fp64_fma_ratio(cm, cms, pk) if cms > 0 else None
     return {"metric": METRIC_1H, "workload": wl.name, "value": wl.npair * ns / (ms / 1e3), "unit": UNIT,
-            "ms_per_step": round(ms, 3), "correlator_fp64_frac": None if frac is None else round(frac, 4),
+            "ms_per_step": round(ms, 3), "correlator_tensor_frac": None if frac is None else round(frac, 4),
+            "correlator_fp64_fma_ratio": None if ratio is None else round(ratio, 2),
             "stage_ms": {k: round(v, 3) for k, v in stage_ms.items()},
             "f32": {"value": f32["value"], "ms_per_step": f32["ms_per_step"],
                     "speedup_vs_f64": f32["speedup_vs_f64"], "max_rel_err_vs_f64": f32["max_rel_err_vs_f64"]}}
@@ -1023,7 +1037,7 @@ def short_roof(r):
     """A stage roofline with rounded figures."""
     if r is None:
         return None
-    keep = ("bound", "achieved", "peak", "unit", "frac", "launch_ms", "traffic")
+    keep = ("bound", "achieved", "peak", "unit", "frac", "launch_ms", "traffic", "fp64_fma_ratio")
     return {k: (round(r[k], 4) if isinstance(r.get(k), float) else r.get(k)) for k in keep if k in r}
 
 

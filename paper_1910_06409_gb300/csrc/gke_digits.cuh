@@ -676,11 +676,15 @@ k_dg_corr(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
 
 // Adds the marked values by FP64 FMAs from the fields.  CTA = one item at a time, whose
 // marks its warps share: a mark's contractions go to one warp in their order (one
-// value may get several).  Lane = row, and a column's far rows are taken either in a chain
-// per lane, as in the FMA kernels, or, where they are few, row by row with a term and
-// snapshot per lane and a tree (10 additions).  Bound by latency with few marked
-// items (one warp per item: 6.5 ms for the 171 items of the duct's m = 0, whose
-// fluctuations are rounding noise; 8 warps 1.9 ms, 32 1.3 but slower where there are none), else by the FP64 pipe.
+// value may get several).  Lane = row; a mark's far values are taken in a chain per lane
+// and column, as in the FMA kernels, where most rows have some, else row by row, the
+// lanes shared out over its far columns and their products, and a tree.  Bound by latency with few
+// marked items (one warp per item took 6.5 ms for the 171 items of the duct's m = 0,
+// whose fluctuations are rounding noise; 16 warps, a column at a time, 1.9, so 1.4), else
+// by the FP64 pipe.  Milliseconds at 128 x 128 x 65 / duct 256 x 33 x 33, 16 snapshots, where components
+// differ in size: all equal 0.3 / 1.4; v (and w) falling one power faster to their walls 0.3 / 2.4;
+// v and w 2^-10 of u 0.6 / 4.6; u 2^-4 of v and w 2.7 / 13.6; u 2^-10 of them 33 / 128 (the
+// contractions by the FMA kernels: 59 / 334).
 constexpr int DG_FARW = 16;                                 // warps of a CTA
 template <typename Out>
 __global__ void __launch_bounds__(32 * DG_FARW, 2)
@@ -716,31 +720,49 @@ k_dg_far(const __grid_constant__ DgArgs a, const __grid_constant__ Out out)
                     acc.y = fma(c * p.x, v.y, acc.y);
                     acc.y = fma(-c * p.y, v.x, acc.y);
                 };
-                zd o[4];
+                unsigned who[4], rows = 0;
                 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int yp = y0 + j;
                     const bool far = row && yp < a.s.n && !(a.tri && yp < y) && dg_far(job, wa, E[job.gb * a.s.nrow + yp]);
-                    const unsigned who = __ballot_sync(0xffffffffu, far);
-                    zd acc = mk(0.0, 0.0);
-                    if (__popc(who) * (10 + 4 * ((n + 31) / 32)) >= 4 * n) {
-                        if (far)
-                            for (int i = 0; i < n; ++i) product(i, y, yp, acc);
-                    } else {
-                        for (unsigned w = who; w; w &= w - 1) {
-                            const int l = __ffs(w) - 1, ya = __shfl_sync(0xffffffffu, y, l);
-                            zd p = mk(0.0, 0.0);
-                            for (int i = lane; i < n; i += 32) product(i, ya, yp, p);
-                            #pragma unroll
-                            for (int h = 16; h > 0; h >>= 1) {
-                                p.x += __shfl_xor_sync(0xffffffffu, p.x, h);
-                                p.y += __shfl_xor_sync(0xffffffffu, p.y, h);
-                            }
-                            if (lane == l) acc = p;
+                    who[j] = __ballot_sync(0xffffffffu, far);
+                    rows |= who[j];
+                }
+                zd o[4] = {mk(0.0, 0.0), mk(0.0, 0.0), mk(0.0, 0.0), mk(0.0, 0.0)};
+                if (__popc(rows) >= 24) {
+                    #pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if ((who[j] >> lane) & 1u)
+                            for (int i = 0; i < n; ++i) product(i, y, y0 + j, o[j]);
+                } else {
+                    for (unsigned w = rows; w; w &= w - 1) {
+                        const int l = __ffs(w) - 1, ya = __shfl_sync(0xffffffffu, y, l);
+                        unsigned m = 0;                      // the row's far columns; g lanes side by side share them
+                        #pragma unroll
+                        for (int j = 0; j < 4; ++j) m |= ((who[j] >> l) & 1u) << j;
+                        const int c = __popc(m), g = c > 2 ? 4 : c;
+                        unsigned mine = m;
+                        for (int i = lane & (g - 1); i > 0; --i) mine &= mine - 1;
+                        zd p = mk(0.0, 0.0);
+                        if (mine) {
+                            const int yb = y0 + __ffs(mine) - 1;
+                            for (int i = lane / g; i < n; i += 32 / g) product(i, ya, yb, p);
+                        }
+                        for (int h = 16; h >= g; h >>= 1) {
+                            p.x += __shfl_xor_sync(0xffffffffu, p.x, h);
+                            p.y += __shfl_xor_sync(0xffffffffu, p.y, h);
+                        }
+                        #pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if (!((m >> j) & 1u)) continue;
+                            const int k = __popc(m & ((1u << j) - 1));
+                            const zd v = mk(__shfl_sync(0xffffffffu, p.x, k), __shfl_sync(0xffffffffu, p.y, k));
+                            if (lane == l) o[j] = v;
                         }
                     }
-                    o[j] = mk(ce * acc.x, ce * acc.y);
                 }
+                #pragma unroll
+                for (int j = 0; j < 4; ++j) o[j] = mk(ce * o[j].x, ce * o[j].y);
                 if (row) out(job, u.k, y, y0, o);
             }
         }

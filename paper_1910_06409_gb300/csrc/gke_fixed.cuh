@@ -10,8 +10,9 @@
 // transform exceeds it, so the integers take 61 bits below 2^E and nothing
 // overflows (x +- y of a complex value: 2^61.5).  Rounding: half a unit 2^(E - 61) per
 // input, half a unit per constant product, and S = 2 bits in the twiddle product;
-// at N = 256 about 7 units in an output, 2^-58 of the 1-norm, which is at most
-// 16 times the 2-norm.  An FP64 transform's error is about 2^-52.3 of the 2-norm.
+// at N = 256 about 7 units in an output, 2^-58 of 2^E.  2^E is at most twice the 1-norm and
+// that sqrt(2 N) = 22.6 times the 2-norm, so at worst 2^-52.7 of the 2-norm; an
+// FP64 transform's error is about 2^-52.3 of it.
 //
 // Measured (FP64 transforms -> here): 256 x 256 x 65, 16 snapshots: inverse transforms
 // of the terms 56.9 -> 19.3 ms, products stage 46.7 -> 20.6 ms; duct 256 x 33 x 33:
