@@ -60,17 +60,17 @@ __device__ __forceinline__ zx operator*(zx a, zx w)
 }
 __device__ __forceinline__ long long fx_mid(long long a) { return (a + (1 << (FX_S - 1))) >> FX_S; }
 
-// W_32^m for the register DFTs (constants times 2^63 as signed word pairs)
+// W_32^m for the register DFTs: constants times 2^63, rounded to integers, as signed word
+// pairs (an FP64 constant is up to 8.5e-17 of itself off, sqrt(1/2) 6.8e-17 too large, and every
+// value of a stage would carry that)
 struct FxC { int h, l; };
-__host__ __device__ constexpr FxC fxc(double c)
+__host__ __device__ constexpr FxC fxc(long long v)
 {
-    // |c| < 1: c 2^63 is an exact integer (53 significant bits)
-    const long long v = (long long)(c * 4611686018427387904.0) * 2;
     return FxC{(int)((v - (long long)(int)(v & 0xffffffffll)) >> 32), (int)(v & 0xffffffffll)};
 }
 template <bool INV> __device__ __forceinline__ zx fx_twiddle(zx w, int m)
 {
-    constexpr FxC q = fxc(0.70710678118654752440);
+    constexpr FxC q = fxc(6521908912666391106ll);
     if (m == 0) return w;
     if (m == 8) return INV ? mk(-w.y, w.x) : mk(w.y, -w.x);
     if (m == 4 || m == 12) {
@@ -79,8 +79,8 @@ template <bool INV> __device__ __forceinline__ zx fx_twiddle(zx w, int m)
         return INV ? mk(-s, d) : mk(-d, -s);
     }
     // cos, sin of 2 pi m / 32 in the first octant, then by symmetry
-    constexpr FxC c1 = fxc(0.98078528040323043), s1 = fxc(0.19509032201612825), c2 = fxc(0.92387953251128674),
-                  s2 = fxc(0.38268343236508978), c3 = fxc(0.83146961230254524), s3 = fxc(0.55557023301960218);
+    constexpr FxC c1 = fxc(9046147529429926059ll), s1 = fxc(1799390620744551094ll), c2 = fxc(8521284645587064995ll),
+                  s2 = fxc(3529631669043774883ll), c3 = fxc(7668953571605777421ll), s3 = fxc(5124230951741890994ll);
     const int k = m < 8 ? m : 16 - m;                       // cos of m in 9..15 is minus that of 16 - m
     const FxC c = k == 1 ? c1 : k == 2 ? c2 : k == 3 ? c3 : k == 5 ? s3 : k == 6 ? s2 : s1;
     const FxC s = k == 1 ? s1 : k == 2 ? s2 : k == 3 ? s3 : k == 5 ? c3 : k == 6 ? c2 : c1;
