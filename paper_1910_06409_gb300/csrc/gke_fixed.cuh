@@ -106,7 +106,9 @@ __device__ __forceinline__ long long fx_from(double x, int s)
     const long long sg = (long long)(hi >> 31);
     return (v ^ sg) - sg;
 }
-// v 2^e, exponents known to stay in the normal range
+// v 2^e, exponents known to stay in the normal range.  Ties go to even: a transform's results have
+// only a few bits to drop, so ties are frequent, and away from zero they would raise the
+// energy (by 2.5e-17 to 4e-17 in the two transforms of 32 or 128 points a side).
 __device__ __forceinline__ double fx_to(long long v, int e)
 {
     const unsigned sg = (unsigned)((int)(v >> 32) >> 31);
@@ -117,7 +119,7 @@ __device__ __forceinline__ double fx_to(long long v, int e)
     const int lz = __clz((int)h);
     const unsigned mh = __funnelshift_l(l, h, lz), ml = l << (lz & 31);
     unsigned rl = __funnelshift_r(ml, mh, 11), rh = (mh >> 11) + ((unsigned)(1022 + 63 + e - (z ? 32 : 0) - lz) << 20);
-    const unsigned up = (ml >> 10) & 1u;
+    const unsigned up = ((ml & 0x7ffu) + 0x3ffu + (rl & 1u)) >> 11;
     rl += up;
     rh += rl < up;
     return h == 0 ? 0.0 : __hiloint2double((int)(rh | (sg & 0x80000000u)), (int)rl);

@@ -63,7 +63,7 @@ def test_transforms_keep_the_energy(tmp_path):
     assert abs(gain) <= 2.0 ** -24, gain
 
 
-@pytest.mark.parametrize("n", [64, 128, 256])
+@pytest.mark.parametrize("n", [32, 64, 128, 256])
 def test_fp64_transforms_keep_the_energy(n, tmp_path):
     """The mean energy of random fields from fixed-point transforms of n x n points
     against Parseval's sum in extended precision, averaged over 31 planes: their sums
