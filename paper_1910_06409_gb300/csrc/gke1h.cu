@@ -781,7 +781,7 @@ k1_correlate_strip(const cplx<TF>* __restrict__ X, int ns, int P, int nx, int co
 // the SM's FP64 pipe.  k1_finish then brings the mean-flow couplings.  With
 // the couplings in the epilogue the stage took 44.1 ms at 256 x 33 x 33.
 //   Correlate stage (us, k1_correlate -> here), 16 snapshots: 256 x 33 x 33
-// 333880 -> 34204 (k1_finish 4760 of it, the marked values of m = 0 1850); no size tried keeps the
+// 333880 -> 33302 (k1_finish 4760 of it, the marked values of m = 0 1400); no size tried keeps the
 // FMA kernel (nx = 8, 25 points, 1 snapshot 356 -> 188).  Bound by the epilogue and the L2
 // reductions; the MMAs (37 terms x 36 digit pairs a tile) take 10 ms by count.
 // (Q, X and 4 p in joint sums of five terms took 28984, but lost what lies far below q u.)
@@ -1027,7 +1027,7 @@ k1_transform(const cplx<TF>* __restrict__ spec, int nx, long long npair, int NB,
 // Register-FFT variant for nx = N1 N2 (gke::fft2l, twiddles resolved at
 // compile time): CTA = RZ sequences x N2 lanes, each sequence two pairs
 // packed as above; lane l holds the wavenumbers l + N2 j of its sequence.
-// Two CTAs per SM (256 x 33 x 33, FP64: 12.5 -> 9.6 ms, one CTA at 190 registers before).
+// Two CTAs per SM (256 x 33 x 33, FP64: 12.5 -> 9.6 ms, one CTA at 190 registers before; 9.9 with ties to even).
 template <typename TF, int N1, int N2>
 __global__ void __launch_bounds__(256, N1 == 32 ? 1 : 2)
 k1_transform_r(const cplx<TF>* __restrict__ spec, long long npair, const cplx<TF>* __restrict__ tw,

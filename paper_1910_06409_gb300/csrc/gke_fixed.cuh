@@ -15,10 +15,10 @@
 // FP64 transform's error is about 2^-52.3 of it.
 //
 // Measured (FP64 transforms -> here): 256 x 256 x 65, 16 snapshots: inverse transforms
-// of the terms 56.9 -> 19.3 ms, products stage 46.7 -> 20.6 ms; duct 256 x 33 x 33:
-// 30.0 -> 9.6 ms; 128 x 128 x 65, 32 snapshots (from shared-memory stages of FP64):
-// products 28.7 -> 10.9 ms, terms 15.3 -> 4.8 ms.  Errors of the terms against 64-bit references do not grow (duct
-// A 1.6e-16 -> 1.2e-16).  (Exponents from the largest component and 56 bits were as
+// of the terms 56.9 -> 19.7 ms, products stage 46.7 -> 21.1 ms; duct 256 x 33 x 33:
+// 30.0 -> 9.9 ms; 128 x 128 x 65, 32 snapshots (from shared-memory stages of FP64):
+// products 28.7 -> 11.1 ms, terms 15.3 -> 4.9 ms.  Errors of the terms against 64-bit references do not grow (duct
+// A 1.7e-16 -> 1.1e-16).  (Exponents from the largest component and 56 bits were as
 // fast, but raised them by up to a half.)
 #pragma once
 #include "gke_common.cuh"
@@ -468,7 +468,7 @@ __device__ __forceinline__ void fft2l_split(cplx<T>* f, int lane, cplx<T>* xr, c
 template <typename T> __host__ __device__ constexpr int fx_smx(int threads) { return sizeof(T) == 4 ? 1 : threads; }
 
 // stages fft2l's twiddles: FP32 the table itself, FP64 its fixed-point copy,
-// which follows the N FP64 entries (tw_table)
+// which follows the N FP64 entries (fx_table)
 template <typename T>
 __device__ __forceinline__ void load_twiddles2l(cplx<T>* sh_tw, const cplx<T>* __restrict__ tw, int N)
 {

@@ -193,7 +193,8 @@ __global__ void k_terms_rowpass(const cplx<TF>* __restrict__ W, const int* __res
 // register-FFT row pass for nx = N1 N2: CTA = RZ rows of one pair x N2 lanes;
 // the seven terms are transformed as four packed sequences (t0 + i t1, ...).
 // FP64: eight CTAs of 64 threads per SM and one operation for scale and one-point
-// part (transforms of 256 x 256 x 65: 20.7 -> 19.3 ms, five CTAs and two operations before)
+// part (transforms of 256 x 256 x 65: 20.7 -> 19.3 ms, five CTAs and two operations before;
+// 19.7 with ties to even)
 template <typename TF, typename TO, int N1, int N2, bool US>
 __global__ void __launch_bounds__(sizeof(TF) == 8 ? 64 : 256, sizeof(TF) == 8 ? 8 : 0)
 k_terms_rowpass_r(const cplx<TF>* __restrict__ W, const int* __restrict__ pair_i, long long pair0, long long npair,
